@@ -121,6 +121,16 @@ def _batch_shapes(case):
     return out
 
 
+def _placed(make, seed, **kw):
+    """make(seed=seed, ...); the bowl generator cannot place its twelve fruits for a few seeds
+    in a hundred: the next seed of a fixed sequence stands in."""
+    while True:
+        try:
+            return make(seed=seed, **kw)
+        except RuntimeError:
+            seed = (seed + 104729) & 0x7FFFFFFF
+
+
 def _scenes(case, seed):
     """The numpy scene dicts of a case (one, or one per scene of a batch), from the seed alone."""
     seed = int(seed) & 0x7FFFFFFF
@@ -128,15 +138,15 @@ def _scenes(case, seed):
         # the shapes of scenes.uneven_batch (its draw from seed 1000 on), the contents from this seed
         out = []
         for q, (n, L, nd, nb) in enumerate(_batch_shapes(case)):
-            out.append(scenes.fruit_bowl(n=n, seed=seed + 7919 * q, L=L, nd=nd, nb=nb, n_lights=case["lights"]))
+            out.append(_placed(scenes.fruit_bowl, seed + 7919 * q, n=n, L=L, nd=nd, nb=nb, n_lights=case["lights"]))
     else:
-        kw = dict(n=case["n"], seed=seed, L=case["L"], nd=max(case["nd"], 32), nb=case["nb"])
+        kw = dict(n=case["n"], L=case["L"], nd=max(case["nd"], 32), nb=case["nb"])
         if case["scene"] == "box":
-            sc = scenes.box_scene(**kw)
+            sc = scenes.box_scene(seed=seed, **kw)
         elif case["scene"] == "room":
-            sc = scenes.large_scene(n_lights=case["lights"], **kw)
+            sc = _placed(scenes.large_scene, seed, n_lights=case["lights"], **kw)
         else:
-            sc = scenes.fruit_bowl(n_lights=1 if case.get("env") else case["lights"], **kw)
+            sc = _placed(scenes.fruit_bowl, seed, n_lights=1 if case.get("env") else case["lights"], **kw)
         if case.get("env"):
             sc = scenes.with_env_map(sc, 16, case["lights"] // 16, seed=seed)
         out = [sc]
