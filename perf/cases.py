@@ -123,7 +123,7 @@ def _batch_shapes(case):
 
 def _placed(make, seed, **kw):
     """make(seed=seed, ...); the bowl generator cannot place its twelve fruits for a few seeds
-    in a hundred: the next seed of a fixed sequence stands in."""
+    in a thousand: the next seed of a fixed sequence stands in."""
     while True:
         try:
             return make(seed=seed, **kw)
