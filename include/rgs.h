@@ -414,9 +414,9 @@ rgs_status rgs_set_wait_limit(rgs_transport *t, int64_t ns);
  * up = right x forward; fov is the vertical field of view in radians (0, pi); pixel (x, y),
  * y pointing down, is sampled at its centre.  B: device float [N][nc][C] in caller order (the
  * layout rgs_solve writes); img: device float [H][W][C], fully written.  Device buffers are
- * the caller's; pooled scratch (40 bytes per pixel and 8 per composited hit) is returned
- * before the call ends.  Every pixel ray is traced twice (count, then fill).  Synchronises
- * `stream` once (the record count and the traversal's overflow check).  Errors: RGS_ERR_ARG (NULL
+ * the caller's; pooled scratch (a copy of B and at most 319 MB of hit lists) is returned
+ * before the call ends.  Every pixel ray is traced, composited and shaded in one pass.
+ * Synchronises `stream` once (the traversal's overflow check).  Errors: RGS_ERR_ARG (NULL
  * pointer, W or H <= 0, W*H > 2^26, fov outside (0, pi)), RGS_ERR_NONFINITE (camera),
  * RGS_ERR_STATE (t not traced), RGS_ERR_CAPACITY (traversal stack), RGS_ERR_OOM,
  * RGS_ERR_CUDA. */

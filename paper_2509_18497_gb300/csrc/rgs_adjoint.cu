@@ -14,10 +14,11 @@
 #include <algorithm>
 #include <vector>
 
-#include "rgs_internal.cuh"
+#include "rgs_warp_trace.cuh"
 
 namespace {
 
+constexpr int SHADOW_THREADS = 128;
 constexpr int ADJ_THREADS = 128;
 static_assert(ADJ_THREADS == 128, "RGS_ADJ_LB assumes 128 threads");
 
@@ -131,97 +132,124 @@ __global__ void RGS_ADJ_LB k_adj_src(RaysDev rays, int C, int col0, const long l
 // term H (n_i.w) fall T moves with w (through Y(R_i w) and n_i.w), with fall = 1/r^2 and with
 // each shadow occluder's crossing point; a directional light has a fixed w and fall = 1.
 // gF (with dp): the frame gradients, through n_i (cos and R_i) and the occluders' frames.
-template <int NC>
-__global__ void k_shadow_bwd(SceneDev sc, int nl, int ldir, const float *__restrict__ lpos, const float *__restrict__ lint,
+// A warp per 32 (surfel, light) pairs, their shadow rays traced together twice (rgs_warp_trace.cuh):
+// for the transmittances, then for the occluders' terms.
+struct ShadowWarp {
+    WarpOcclusion w;
+    float q[32], T[32]; // dL/dT and the product of the factors that are not 0
+    int nz[32];         // how many are 0
+    float gp[32][3], gw[32][3];
+};
+template <int NC, bool GEO>
+__global__ void __launch_bounds__(SHADOW_THREADS) k_shadow_bwd(SceneDev sc, int nl, int ldir, const float *__restrict__ lpos, const float *__restrict__ lint,
                              int C, const float *__restrict__ u, float *P, float *dop, float *dp, float *ds, float *gF) {
+    extern __shared__ __align__(16) unsigned char shadow_smem[];
+    ShadowWarp &sm = reinterpret_cast<ShadowWarp *>(shadow_smem)[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
     const int tid = blockIdx.x * blockDim.x + threadIdx.x;
-    if (tid >= sc.n * nl) return;
-    const int i = tid / nl, lt = tid - i * nl;
+    const bool live = tid < sc.n * nl;
+    const int i = live ? tid / nl : 0, lt = live ? tid - i * nl : 0;
     const float4 Pi = sc.P[i];
     const float3 o = f3(Pi), n = f3(sc.N4[i]);
     float r, fall;
     const float3 w = light_dir(lpos, lt, o, ldir, r, fall);
     const float cs = dot3(n, w);
-    if (!(cs > 0.f)) return;
+    const bool lit = live && cs > 0.f;
     const float eps = *sc.eps_plane;
-    float Tnz = 1.f;
-    int nzero = 0;
-    auto pass1 = [&](int j) {
-        float t, g;
-        if (!hit_surfel(sc, j, i, o, w, r, eps, t, g)) return;
-        const float om = 1.f - alpha_of(sc, __ldg(&sc.P[j].w), g);
-        if (om == 0.f) ++nzero;
-        else Tnz *= om;
-    };
-    bvh_traverse(sc, o, w, r, pass1);
+    float Tnz;
+    int nzero;
+    warp_transmittance(sc, sm.w, o, w, r, i, lit, eps, Tnz, nzero, [](int, int) { return true; });
+    float qv = 0.f, H = 0.f;
     const float T = nzero ? 0.f : Tnz;
-    float Y[NC], h[NC];
-    const float3 rw = reflect_n(n, w);
-    sh_eval<NC>(rw, Y);
-    const float pre = cs * fall;
-    const float *ui = u + ((size_t)i * C + lt * 3) * NC;
-    const float ai = alpha_center(sc, i);
-    float qv = 0.f;
-    float acc[4][3] = {};
-#pragma unroll
-    for (int k = 0; k < NC; ++k) h[k] = 0.f;
-    for (int ch = 0; ch < 3; ++ch) {
-        const float I = lint[3 * lt + ch];
-#pragma unroll
-        for (int k = 0; k < NC; ++k) {
-            const float cl = sc.cl[(size_t)i * 12 + band_of(k) * 3 + ch];
-            const float uy = ui[ch * NC + k] * Y[k] * I * pre;
-            qv += uy * cl;
-            acc[band_of(k)][ch] += uy * T;
-            h[k] += ui[ch * NC + k] * I * cl;
-        }
-    }
-    for (int b = 0; b < 4; ++b)
-        for (int ch = 0; ch < 3; ++ch)
-            if (acc[b][ch] != 0.f) atomicAdd(&P[(size_t)i * 12 + b * 3 + ch], acc[b][ch]);
-    qv *= ai;
     float3 gw = make_float3(0.f, 0.f, 0.f), gpi = make_float3(0.f, 0.f, 0.f);
-    float H = 0.f;
-    if (dp) {
+    if (lit) {
+        float Y[NC], h[NC];
+        const float3 rw = reflect_n(n, w);
+        sh_eval<NC>(rw, Y);
+        const float pre = cs * fall;
+        const float *ui = u + ((size_t)i * C + lt * 3) * NC;
+        const float ai = alpha_center(sc, i);
+        float acc[4][3] = {};
 #pragma unroll
-        for (int k = 0; k < NC; ++k) {
-            h[k] *= ai;
-            H += h[k] * Y[k];
-        }
-        const float3 t1 = sh_grad_dot<NC>(rw, h);
-        const float3 t3 = reflect_n(n, t1);
-        const float f = fall * T;
-        gw = make_float3(f * (cs * t3.x + H * n.x), f * (cs * t3.y + H * n.y), f * (cs * t3.z + H * n.z));
-        const float3 gn = reflect_grad_n(n, w, (f * cs) * t1) + (H * f) * w; // R_i w and cos = n_i.w
-        geo_add3(gF + GEO_GF * (size_t)i + GEO_N, gn);
-    }
-    if (qv != 0.f && nzero <= 1) {
-        auto pass2 = [&](int j) {
-            float t, g;
-            if (!hit_surfel(sc, j, i, o, w, r, eps, t, g)) return;
-            const float oj = __ldg(&sc.P[j].w);
-            const float om = 1.f - alpha_of(sc, oj, g);
-            float others;
-            if (nzero == 0) others = Tnz / om;
-            else others = (om == 0.f) ? Tnz : 0.f;
-            if (others == 0.f) return;
-            atomicAdd(&dop[j], -qv * others * dalpha_do(sc, oj, g));
-            if (dp) {
-                const float coef = -qv * others * dalpha_dq(sc, oj, g);
-                if (coef == 0.f) return;
-                float uu, vv;
-                const float3 pw = crossing_pw(sc, j, o, w, t, uu, vv);
-                gpi = gpi + coef * pw;
-                gw = gw + (coef * t) * pw;
-                geo_add3(dp + GEO_DP * (size_t)j, (-coef) * pw);
-                geo_add2(ds + 2 * (size_t)j, coef * (-2.f * uu * uu * __ldg(&sc.FU[j].w)),
-                         coef * (-2.f * vv * vv * __ldg(&sc.FV[j].w)));
-                occluder_frame_grad(sc, j, o, w, t, uu, vv, coef, gF);
+        for (int k = 0; k < NC; ++k) h[k] = 0.f;
+        for (int ch = 0; ch < 3; ++ch) {
+            const float I = lint[3 * lt + ch];
+#pragma unroll
+            for (int k = 0; k < NC; ++k) {
+                const float cl = sc.cl[(size_t)i * 12 + band_of(k) * 3 + ch];
+                const float uy = ui[ch * NC + k] * Y[k] * I * pre;
+                qv += uy * cl;
+                acc[band_of(k)][ch] += uy * T;
+                h[k] += ui[ch * NC + k] * I * cl;
             }
-        };
-        bvh_traverse(sc, o, w, r, pass2);
+        }
+        for (int b = 0; b < 4; ++b)
+            for (int ch = 0; ch < 3; ++ch)
+                if (acc[b][ch] != 0.f) atomicAdd(&P[(size_t)i * 12 + b * 3 + ch], acc[b][ch]);
+        qv *= ai;
+        if constexpr (GEO) {
+#pragma unroll
+            for (int k = 0; k < NC; ++k) {
+                h[k] *= ai;
+                H += h[k] * Y[k];
+            }
+            const float3 t1 = sh_grad_dot<NC>(rw, h);
+            const float3 t3 = reflect_n(n, t1);
+            const float f = fall * T;
+            gw = make_float3(f * (cs * t3.x + H * n.x), f * (cs * t3.y + H * n.y), f * (cs * t3.z + H * n.z));
+            const float3 gn = reflect_grad_n(n, w, (f * cs) * t1) + (H * f) * w; // R_i w and cos = n_i.w
+            geo_add3(gF + GEO_GF * (size_t)i + GEO_N, gn);
+        }
     }
-    if (dp) {
+    const bool second = lit && qv != 0.f && nzero <= 1;
+    if (__any_sync(WT_FULL, second)) {
+        sm.q[lane] = qv;
+        sm.T[lane] = Tnz;
+        sm.nz[lane] = nzero;
+        __syncwarp();
+        auto test = [&](int j, int ray, bool valid) {
+            bool terms = false;
+            if (valid) {
+                const float4 ro = sm.w.o[ray], rd = sm.w.d[ray];
+                const float3 oo = f3(ro), dd = f3(rd);
+                float t, g, oj;
+                if (hit_surfel(sc, j, __float_as_int(ro.w), oo, dd, rd.w, eps, t, g, oj)) {
+                    const float om = 1.f - alpha_of(sc, oj, g);
+                    const float others = sm.nz[ray] == 0 ? sm.T[ray] / om : (om == 0.f ? sm.T[ray] : 0.f);
+                    if (others != 0.f) {
+                        const float q = sm.q[ray];
+                        atomicAdd(&dop[j], -q * others * dalpha_do(sc, oj, g));
+                        if constexpr (GEO) {
+                            const float coef = -q * others * dalpha_dq(sc, oj, g);
+                            if (coef != 0.f) {
+                                terms = true;
+                                float uu, vv;
+                                const float3 pw = crossing_pw(sc, j, oo, dd, t, uu, vv);
+                                sm.gp[lane][0] = coef * pw.x;
+                                sm.gp[lane][1] = coef * pw.y;
+                                sm.gp[lane][2] = coef * pw.z;
+                                sm.gw[lane][0] = (coef * t) * pw.x;
+                                sm.gw[lane][1] = (coef * t) * pw.y;
+                                sm.gw[lane][2] = (coef * t) * pw.z;
+                                geo_add3(dp + GEO_DP * (size_t)j, (-coef) * pw);
+                                geo_add2(ds + 2 * (size_t)j, coef * (-2.f * uu * uu * __ldg(&sc.FU[j].w)),
+                                         coef * (-2.f * vv * vv * __ldg(&sc.FV[j].w)));
+                                occluder_frame_grad(sc, j, oo, dd, t, uu, vv, coef, gF);
+                            }
+                        }
+                    }
+                }
+            }
+            if constexpr (GEO)
+                warp_owner_loop(sm.w.own, terms, ray, [&](int b) {
+                    gpi = gpi + make_float3(sm.gp[b][0], sm.gp[b][1], sm.gp[b][2]);
+                    gw = gw + make_float3(sm.gw[b][0], sm.gw[b][1], sm.gw[b][2]);
+                });
+        };
+        warp_traverse<false>(sc, o, w, r, second, sm.w.q, test, [](float m) { return m; });
+    }
+    if constexpr (GEO) {
+        if (!lit) return;
         float3 gp = gpi;
         if (!ldir) { // w = (p_L - p_i)/r, fall = 1/r^2
             const float ww = dot3(w, gw), gr = H * cs * T * (-2.f * fall / r);
@@ -231,6 +259,16 @@ __global__ void k_shadow_bwd(SceneDev sc, int nl, int ldir, const float *__restr
         }
         geo_add3(dp + GEO_DP * (size_t)i, gp);
     }
+}
+
+template <int NC>
+void launch_shadow(rgs_transport *t, cudaStream_t st, float *dp, float *ds, float *gF) {
+    const int nth = t->n * t->nl;
+    const unsigned blocks = (unsigned)((nth + SHADOW_THREADS - 1) / SHADOW_THREADS);
+    const size_t smem = sizeof(ShadowWarp) * (SHADOW_THREADS / 32);
+    ProfScope ps_("k_shadow_bwd", st);
+    if (dp) k_shadow_bwd<NC, true><<<blocks, SHADOW_THREADS, smem, st>>>(t->sc->dev(), t->nl, t->ldir, t->lpos, t->lint, t->C, t->u, t->Pg, t->dop, dp, ds, gF);
+    else k_shadow_bwd<NC, false><<<blocks, SHADOW_THREADS, smem, st>>>(t->sc->dev(), t->nl, t->ldir, t->lpos, t->lint, t->C, t->u, t->Pg, t->dop, dp, ds, gF);
 }
 
 // Hemisphere rays, part 1: for every stored hit h of ray r (receiver i, source j_h),
@@ -333,8 +371,9 @@ __global__ void RGS_OPAREC_LB k_opacity_rec(SceneDev sc, RaysDev rays, const flo
         const long long slot = base + h;
         const int2 ja = __ldg(&rays.rec_ja[slot]);
         const int j = ja.x;
-        const float G = stored_hit_G(sc, j, o, d);
-        const float oj = __ldg(&sc.P[j].w);
+        float t, r2, oj;
+        accepted_hit(sc, j, o, d, t, r2, oj);
+        const float G = surfel_G(sc, r2);
         const float alpha = alpha_of(sc, oj, G);
         const float g = gh[slot];
         // the transmittance in front of the hit from its stored weight a_h = alpha_h T_h
@@ -373,8 +412,9 @@ __global__ void __launch_bounds__(128) k_hemi_geo(SceneDev sc, RaysDev rays, int
         for (int h = cnt - 1; h >= 0; --h) {
             const int2 ja = __ldg(&rays.rec_ja[base + h]);
             const int j = ja.x;
-            const float G = stored_hit_G(sc, j, o, d);
-            const float oj = __ldg(&sc.P[j].w);
+            float th, r2, oj;
+            accepted_hit(sc, j, o, d, th, r2, oj);
+            const float G = surfel_G(sc, r2);
             const float al = alpha_of(sc, oj, G);
             const float g = gh[base + h];
             // the transmittance in front of the hit from its stored weight a_h = alpha_h T_h
@@ -773,8 +813,7 @@ rgs_status run_adjoint(rgs_transport *t, const float *g, float *dE, float *dad, 
     }
     if (nb >= 1 && (r = KT(nb)) != RGS_OK) return r; // v^(n) only adds to u
     if (t->nl > 0) {
-        const int nth = n * t->nl;
-        { ProfScope ps_("k_shadow_bwd", st); k_shadow_bwd<NC><<<(nth + 127) / 128, 128, 0, st>>>(sd, t->nl, t->ldir, t->lpos, t->lint, C, t->u, t->Pg, t->dop, geo ? geo->dp : nullptr, geo ? geo->ds : nullptr, geo ? geo->gF : nullptr); }
+        launch_shadow<NC>(t, st, geo ? geo->dp : nullptr, geo ? geo->ds : nullptr, geo ? geo->gF : nullptr);
         RGS_LAUNCH("shadow backward");
     }
     if (nb >= 1 && dopo) {
@@ -820,8 +859,7 @@ template <int NC> rgs_status accum_nc(rgs_transport *t, const float *X, const fl
 }
 template <int NC> rgs_status shadow_nc(rgs_transport *t, cudaStream_t st, float *dp, float *ds, float *gF) {
     if (t->nl <= 0) return RGS_OK;
-    const int nth = t->n * t->nl;
-    { ProfScope ps_("k_shadow_bwd", st); k_shadow_bwd<NC><<<(nth + 127) / 128, 128, 0, st>>>(t->sc->dev(), t->nl, t->ldir, t->lpos, t->lint, t->C, t->u, t->Pg, t->dop, dp, ds, gF); }
+    launch_shadow<NC>(t, st, dp, ds, gF);
     RGS_LAUNCH("shadow backward");
     return RGS_OK;
 }

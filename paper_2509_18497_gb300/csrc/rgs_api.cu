@@ -600,12 +600,14 @@ void rgs_destroy_scene(rgs_scene *s) {
     dev_free(s->N4);
     dev_free(s->FU);
     dev_free(s->FV);
+    dev_free(s->rec);
     dev_free(s->GS);
     dev_free(s->cl);
     dev_free(s->kk);
     dev_free(s->uid);
     dev_free(s->inv);
     dev_free(s->nodes);
+    dev_free(s->kids);
     dev_free(s->boxes);
     dev_free(s->parent);
     dev_free(s->visit);

@@ -2,7 +2,8 @@
 //
 // Data layout in HBM (all arrays in the library's internal Morton order of the surfels):
 //   P[j]  = (p.xyz, o)          N4[j] = (n.xyz, 0)
-//   FU[j] = (t^u.xyz, 1/s^u)    FV[j] = (t^v.xyz, 1/s^v)        64 B read per intersection test
+//   FU[j] = (t^u.xyz, 1/s^u)    FV[j] = (t^v.xyz, 1/s^v)
+//   rec[j] = (P, N, FU, FV): the 64 B that an intersection test reads, in one place
 //   cl[j] = c_{j,l,ch} as [4][3] floats (bands beyond L are zero)
 //   uid[j] = caller index of internal surfel j (ray seeds and depth-tie order use it)
 //   radiosity-like arrays (S, B^(b), Q^(b), v^(a), u): [N][C][NC] float, SH index innermost
@@ -17,7 +18,8 @@
 
 #define RGS_HMAX 96           // per-ray hit buffer; when full the nearest RGS_HMAX hits are kept
 #define RGS_T_EPS 1e-6f       // compositing stops once the transmittance is below this
-#define RGS_STACK 64          // BVH traversal stack depth (tree depth is bounded by 32 + log2 N)
+#define RGS_STACK 96          // BVH traversal stack depth: three waiting nodes per level of the four-wide
+                              // tree, at most (30 Morton bits + log2 N) / 2 levels
 
 // Launch bounds of the gather kernels: with RGS_<KERNEL>_MINB defined, the register budget
 // is sized for that many resident blocks per SM (these latency-bound kernels gain from more
@@ -71,19 +73,32 @@ enum {
 };
 
 // ------------------------------------------------------------------ BVH node
-// Internal node of a binary LBVH; stores both children's boxes. A child index c >= 0
-// is an internal node, c < 0 is the leaf (surfel) ~c.
-struct __align__(16) BvhNode {
-    float4 a; // l.lo.x l.lo.y l.lo.z l.hi.x
-    float4 b; // l.hi.y l.hi.z r.lo.x r.lo.y
-    float4 c; // r.lo.z r.hi.x r.hi.y r.hi.z
-    int4 d;   // left, right, 0, 0
+// Node of the traversal's four-wide tree, 64 bytes (two 32-byte requests): the boxes of a
+// binary LBVH node's up to four grandchildren (a child that is a leaf stands for itself) in 8
+// bits per coordinate, org + scale q rounded outwards, on the grid of their union (whose
+// widest side is 253 steps, so a box grows by under 1 % of the node).  A traversal step costs
+// mostly what is not box arithmetic (votes, queue, stack, branches); four boxes per step
+// make half the steps of two.
+struct __align__(64) BvhNode {
+    float ox, oy, oz, scale;
+    unsigned lox, hix, loy, hiy; // byte c: child c
+    unsigned loz, hiz;
+    unsigned mask;               // bit c: child c is a node, bit 4 + c: child c is a surfel
+    unsigned pad;
+    int kid[4];
+};
+
+// What an intersection test reads of a surfel, one 64-byte record (the same values as the
+// separate P, N4, FU, FV arrays, which the kernels that need one of them read).
+struct __align__(64) SurfelRec {
+    float4 P, N, U, V;
 };
 
 struct SceneDev {
     int n, L, alpha_model;
     float cutoff2;
     const float4 *P, *N4, *FU, *FV;
+    const SurfelRec *rec;
     const float *cl; // [n][4][3]
     const int *uid; // caller index of internal surfel i
     const int *inv; // internal index of caller surfel k
@@ -316,17 +331,38 @@ __device__ __forceinline__ float3 ray_dir(unsigned long long seed, int uid, int 
 }
 
 // ------------------------------------------------------------------ intersection
+// 32 bytes in one request (the widest there is).  Lanes of a divergent warp read 32 different
+// records; 16-byte requests made the L1 tag and data stages see every line four times (the
+// trace held the L1 data pipe at 83 % of peak).
+__device__ __forceinline__ void ld_rec32(const void *p, float4 &a, float4 &b) {
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
+        : "l"(p));
+}
+__device__ __forceinline__ SurfelRec ld_surfel(const SceneDev &sc, int j) {
+    SurfelRec s;
+    ld_rec32(&sc.rec[j].P, s.P, s.N);
+    ld_rec32(&sc.rec[j].U, s.U, s.V);
+    return s;
+}
+__device__ __forceinline__ BvhNode ld_node(const SceneDev &sc, int k) {
+    float4 a, b, c, d;
+    const char *p = reinterpret_cast<const char *>(&sc.nodes[k]);
+    ld_rec32(p, a, b);
+    ld_rec32(p + 32, c, d);
+    return BvhNode{a.x, a.y, a.z, a.w, __float_as_uint(b.x), __float_as_uint(b.y), __float_as_uint(b.z),
+                   __float_as_uint(b.w), __float_as_uint(c.x), __float_as_uint(c.y), __float_as_uint(c.z), 0u,
+                   {__float_as_int(d.x), __float_as_int(d.y), __float_as_int(d.z), __float_as_int(d.w)}};
+}
+
 // Squared local radius u^2 + v^2 of the point o + t d on the plane of surfel j (Eq. G),
 // with explicitly rounded operations so that every call site computes identical bits
 // (the trace recomputes it after sorting instead of storing it).
-__device__ __forceinline__ float surfel_r2(const SceneDev &sc, int j, float3 o, float3 d, float t) {
-    const float4 Pj = __ldg(&sc.P[j]);
-    const float wx = __fsub_rn(Pj.x, o.x), wy = __fsub_rn(Pj.y, o.y), wz = __fsub_rn(Pj.z, o.z);
+__device__ __forceinline__ float surfel_r2(const SurfelRec &s, float3 o, float3 d, float t) {
+    const float wx = __fsub_rn(s.P.x, o.x), wy = __fsub_rn(s.P.y, o.y), wz = __fsub_rn(s.P.z, o.z);
     const float qx = __fmaf_rn(t, d.x, -wx), qy = __fmaf_rn(t, d.y, -wy), qz = __fmaf_rn(t, d.z, -wz); // x - p_j
-    const float4 U = __ldg(&sc.FU[j]);
-    const float4 V = __ldg(&sc.FV[j]);
-    const float u = __fmul_rn(__fmaf_rn(qz, U.z, __fmaf_rn(qy, U.y, __fmul_rn(qx, U.x))), U.w);
-    const float v = __fmul_rn(__fmaf_rn(qz, V.z, __fmaf_rn(qy, V.y, __fmul_rn(qx, V.x))), V.w);
+    const float u = __fmul_rn(__fmaf_rn(qz, s.U.z, __fmaf_rn(qy, s.U.y, __fmul_rn(qx, s.U.x))), s.U.w);
+    const float v = __fmul_rn(__fmaf_rn(qz, s.V.z, __fmaf_rn(qy, s.V.y, __fmul_rn(qx, s.V.x))), s.V.w);
     return __fmaf_rn(v, v, __fmul_rn(u, u));
 }
 
@@ -420,161 +456,104 @@ __device__ __forceinline__ float dalpha_center(const SceneDev &sc, int i) {
     return dalpha_do(sc, __ldg(&sc.P[i].w), 1.f);
 }
 
+// n . (p - o) and n . d of a surfel's plane and the ray o + t d
+__device__ __forceinline__ float plane_h(const SurfelRec &s, float3 o) {
+    return __fmaf_rn(s.N.z, __fsub_rn(s.P.z, o.z),
+                     __fmaf_rn(s.N.y, __fsub_rn(s.P.y, o.y), __fmul_rn(s.N.x, __fsub_rn(s.P.x, o.x))));
+}
+__device__ __forceinline__ float plane_den(const SurfelRec &s, float3 d) {
+    return __fmaf_rn(s.N.z, d.z, __fmaf_rn(s.N.y, d.y, __fmul_rn(s.N.x, d.x)));
+}
+
 // Ray o + t d against the plane of surfel j (Eq. G). Returns true with t and r2 when the
-// hit is accepted: j != self, |n_j.(p_j - o)| > eps, 0 < t < tmax, inside the cutoff.
+// hit is accepted: j != self, |n_j.(p_j - o)| > eps, 0 < t < tmax, inside the cutoff; op is
+// then its opacity parameter.
 __device__ __forceinline__ bool hit_surfel_t(const SceneDev &sc, int j, int self, float3 o, float3 d, float tmax,
-                                             float eps, float &t_out, float &r2_out) {
+                                             float eps, float &t_out, float &r2_out, float &op) {
     if (j == self) return false;
-    const float4 Nj = __ldg(&sc.N4[j]);
-    const float den = __fmaf_rn(Nj.z, d.z, __fmaf_rn(Nj.y, d.y, __fmul_rn(Nj.x, d.x)));
+    const SurfelRec s = ld_surfel(sc, j);
+    const float den = plane_den(s, d);
     if (fabsf(den) < 1e-12f) return false;
-    const float4 Pj = __ldg(&sc.P[j]);
-    const float h = __fmaf_rn(Nj.z, __fsub_rn(Pj.z, o.z),
-                              __fmaf_rn(Nj.y, __fsub_rn(Pj.y, o.y), __fmul_rn(Nj.x, __fsub_rn(Pj.x, o.x))));
+    const float h = plane_h(s, o);
     if (fabsf(h) <= eps) return false;
     const float t = __fdiv_rn(h, den);
     if (!(t > 0.f) || !(t < tmax)) return false;
-    const float r2 = surfel_r2(sc, j, o, d, t);
+    const float r2 = surfel_r2(s, o, d, t);
     if (r2 > sc.cutoff2) return false;
     t_out = t;
     r2_out = r2;
+    op = s.P.w;
     return true;
 }
 
-// G of a hit that the trace stored (ray o + t d on surfel j), recomputed with the same
-// rounding as hit_surfel_t, so it equals the value the compositing used bit for bit.
-__device__ __forceinline__ float stored_hit_G(const SceneDev &sc, int j, float3 o, float3 d) {
-    const float4 Nj = __ldg(&sc.N4[j]);
-    const float den = __fmaf_rn(Nj.z, d.z, __fmaf_rn(Nj.y, d.y, __fmul_rn(Nj.x, d.x)));
-    const float4 Pj = __ldg(&sc.P[j]);
-    const float h = __fmaf_rn(Nj.z, __fsub_rn(Pj.z, o.z),
-                              __fmaf_rn(Nj.y, __fsub_rn(Pj.y, o.y), __fmul_rn(Nj.x, __fsub_rn(Pj.x, o.x))));
-    return surfel_G(sc, surfel_r2(sc, j, o, d, __fdiv_rn(h, den)));
+// t, u^2 + v^2 and the opacity parameter of a hit that the trace has accepted (ray o + t d on
+// surfel j), recomputed with the same rounding as hit_surfel_t: the same bits.
+__device__ __forceinline__ void accepted_hit(const SceneDev &sc, int j, float3 o, float3 d, float &t, float &r2,
+                                             float &op) {
+    const SurfelRec s = ld_surfel(sc, j);
+    t = __fdiv_rn(plane_h(s, o), plane_den(s, d));
+    r2 = surfel_r2(s, o, d, t);
+    op = s.P.w;
 }
 
 __device__ __forceinline__ bool hit_surfel(const SceneDev &sc, int j, int self, float3 o, float3 d, float tmax,
-                                           float eps, float &t_out, float &g_out) {
+                                           float eps, float &t_out, float &g_out, float &op) {
     float r2;
-    if (!hit_surfel_t(sc, j, self, o, d, tmax, eps, t_out, r2)) return false;
+    if (!hit_surfel_t(sc, j, self, o, d, tmax, eps, t_out, r2, op)) return false;
     g_out = surfel_G(sc, r2);
     return true;
 }
 
-// slab test of the box [lo, hi] against the segment (0, tmax); NaNs from 0*inf are ignored
-__device__ __forceinline__ bool slab(float lox, float loy, float loz, float hix, float hiy, float hiz, float3 o,
-                                     float3 inv, float tmax) {
-    float tx0 = (lox - o.x) * inv.x, tx1 = (hix - o.x) * inv.x;
-    float ty0 = (loy - o.y) * inv.y, ty1 = (hiy - o.y) * inv.y;
-    float tz0 = (loz - o.z) * inv.z, tz1 = (hiz - o.z) * inv.z;
-    float tmin = fmaxf(fmaxf(fminf(tx0, tx1), fminf(ty0, ty1)), fmaxf(fminf(tz0, tz1), 0.f));
-    float tmx = fminf(fminf(fmaxf(tx0, tx1), fmaxf(ty0, ty1)), fminf(fmaxf(tz0, tz1), tmax));
-    return tmin <= tmx;
+// A ray as the slab tests use it: 1/d and -o/d.  A direction component of (nearly) zero takes
+// a huge finite reciprocal, so that no product below is 0 * inf.
+struct SlabRay {
+    float3 inv, noi;
+};
+__device__ __forceinline__ SlabRay slab_ray(float3 o, float3 d) {
+    auto rcp = [](float v) { return fabsf(v) > 1e-18f ? 1.f / v : copysignf(1e18f, v); };
+    SlabRay r;
+    r.inv = make_float3(rcp(d.x), rcp(d.y), rcp(d.z));
+    r.noi = make_float3(-o.x * r.inv.x, -o.y * r.inv.y, -o.z * r.inv.z);
+    return r;
 }
-
-// slab test returning the entry distance (clamped to 0) of a hit box
-__device__ __forceinline__ bool slab_t(float lox, float loy, float loz, float hix, float hiy, float hiz, float3 o,
-                                       float3 inv, float tmax, float &tnear) {
-    float tx0 = (lox - o.x) * inv.x, tx1 = (hix - o.x) * inv.x;
-    float ty0 = (loy - o.y) * inv.y, ty1 = (hiy - o.y) * inv.y;
-    float tz0 = (loz - o.z) * inv.z, tz1 = (hiz - o.z) * inv.z;
-    float tmin = fmaxf(fmaxf(fminf(tx0, tx1), fminf(ty0, ty1)), fmaxf(fminf(tz0, tz1), 0.f));
-    float tmx = fminf(fminf(fmaxf(tx0, tx1), fmaxf(ty0, ty1)), fminf(fmaxf(tz0, tz1), tmax));
-    tnear = tmin;
-    return tmin <= tmx;
+__device__ __forceinline__ float max3(float a, float b, float c) {
+    float r;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
 }
-
-// Nearer-first traversal for rays that need all hits in depth order: children are
-// visited in order of their entry distance, so hits arrive almost sorted and the
-// per-ray insertion sort does little work.  Leaves are tested as soon as they are
-// reached (postponing them to test all lanes' leaves together was measured slower here:
-// lanes holding a leaf idled while the others searched).  Calls f(j) for every surfel
-// whose box the ray crosses; returns false if the stack overflowed.
-template <class F>
-__device__ __forceinline__ bool bvh_traverse_ordered(const SceneDev &sc, float3 o, float3 d, F &&f) {
-    if (sc.n == 1) {
-        f(0);
-        return true;
-    }
-    const float3 inv = make_float3(1.f / d.x, 1.f / d.y, 1.f / d.z);
-    int stack[RGS_STACK];
-    int sp = 0;
-    int node = 0;
-    bool ok = true;
-    while (true) {
-        const BvhNode nd = sc.nodes[node];
-        int cn = nd.d.x, cf = nd.d.y; // near / far child
-        float tn, tf;
-        bool hn = slab_t(nd.a.x, nd.a.y, nd.a.z, nd.a.w, nd.b.x, nd.b.y, o, inv, INFINITY, tn);
-        bool hf = slab_t(nd.b.z, nd.b.w, nd.c.x, nd.c.y, nd.c.z, nd.c.w, o, inv, INFINITY, tf);
-        if (hn && hf && tf < tn) {
-            const int tc = cn;
-            cn = cf;
-            cf = tc;
-        }
-        if (hn && cn < 0) {
-            f(~cn);
-            hn = false;
-        }
-        if (hf && cf < 0) {
-            f(~cf);
-            hf = false;
-        }
-        if (hn && hf) {
-            if (sp < RGS_STACK) stack[sp++] = cf;
-            else ok = false;
-            node = cn;
-        } else if (hn) {
-            node = cn;
-        } else if (hf) {
-            node = cf;
-        } else {
-            if (sp == 0) break;
-            node = stack[--sp];
-        }
-    }
-    return ok;
+__device__ __forceinline__ float min3(float a, float b, float c) {
+    float r;
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
 }
-
-// Visits every surfel whose box the segment (0, tmax) crosses and calls f(j).
-// Returns false if the stack overflowed (then part of the tree was skipped).
-template <class F>
-__device__ __forceinline__ bool bvh_traverse(const SceneDev &sc, float3 o, float3 d, float tmax, F &&f) {
-    if (sc.n == 1) {
-        f(0);
-        return true;
+// plane distance of child c on one axis: byte c of w placed in a float's mantissa is
+// v = 1 + q 2^-15 (one byte permutation), so t = (org + scale q - o)/d = v S + C with
+// S = 2^15 scale/d and C = (org - o)/d - S (exact to 0.002 steps)
+__device__ __forceinline__ float slab_dist(unsigned w, int c, float S, float C) {
+    return fmaf(__uint_as_float(__byte_perm(w, 0x3f800000u, 0x7604u | (c << 4))), S, C);
+}
+// Slab tests of a node's four boxes against the segment (0, tmax): bit c of the result is set
+// where box c is crossed, t[c] is then its entry distance (clamped to 0).  The near and far
+// planes are picked by the sign of d before the bytes are taken apart, which leaves two
+// three-input minima and maxima per box.  The rounding of org/d - o/d, of the order of
+// 1e-7 |o|, is within the boxes' padding, as that of (org - o)/d is.
+__device__ __forceinline__ unsigned slab4(const BvhNode &nd, const SlabRay &r, float tmax, float (&t)[4]) {
+    const float s15 = 32768.f * nd.scale;
+    const float Sx = s15 * r.inv.x, Sy = s15 * r.inv.y, Sz = s15 * r.inv.z;
+    const float Cx = fmaf(nd.ox, r.inv.x, r.noi.x) - Sx, Cy = fmaf(nd.oy, r.inv.y, r.noi.y) - Sy,
+                Cz = fmaf(nd.oz, r.inv.z, r.noi.z) - Sz;
+    const bool nx = r.inv.x < 0.f, ny = r.inv.y < 0.f, nz = r.inv.z < 0.f;
+    const unsigned ax = nx ? nd.hix : nd.lox, bx = nx ? nd.lox : nd.hix;
+    const unsigned ay = ny ? nd.hiy : nd.loy, by = ny ? nd.loy : nd.hiy;
+    const unsigned az = nz ? nd.hiz : nd.loz, bz = nz ? nd.loz : nd.hiz;
+    unsigned hit = 0u;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        t[c] = fmaxf(max3(slab_dist(ax, c, Sx, Cx), slab_dist(ay, c, Sy, Cy), slab_dist(az, c, Sz, Cz)), 0.f);
+        const float f = fminf(min3(slab_dist(bx, c, Sx, Cx), slab_dist(by, c, Sy, Cy), slab_dist(bz, c, Sz, Cz)), tmax);
+        if (t[c] <= f) hit |= 0x11u << c;
     }
-    const float3 inv = make_float3(1.f / d.x, 1.f / d.y, 1.f / d.z);
-    int stack[RGS_STACK];
-    int sp = 0;
-    int node = 0;
-    bool ok = true;
-    while (true) {
-        const BvhNode nd = sc.nodes[node];
-        const int cl = nd.d.x, cr = nd.d.y;
-        bool hl = slab(nd.a.x, nd.a.y, nd.a.z, nd.a.w, nd.b.x, nd.b.y, o, inv, tmax);
-        bool hr = slab(nd.b.z, nd.b.w, nd.c.x, nd.c.y, nd.c.z, nd.c.w, o, inv, tmax);
-        if (hl && cl < 0) {
-            f(~cl);
-            hl = false;
-        }
-        if (hr && cr < 0) {
-            f(~cr);
-            hr = false;
-        }
-        if (hl && hr) {
-            if (sp < RGS_STACK) stack[sp++] = cr;
-            else ok = false;
-            node = cl;
-        } else if (hl) {
-            node = cl;
-        } else if (hr) {
-            node = cr;
-        } else {
-            if (sp == 0) break;
-            node = stack[--sp];
-        }
-    }
-    return ok;
+    return hit & nd.mask;
 }
 
 // ------------------------------------------------------------------ host-side handles
@@ -582,10 +561,12 @@ struct rgs_scene {
     int device = 0;
     int n = 0, cap = 0, L = 0, nc = 1, alpha_model = 0;
     float4 *P = nullptr, *N4 = nullptr, *FU = nullptr, *FV = nullptr;
+    SurfelRec *rec = nullptr;
     float4 *GS = nullptr; // Gram-Schmidt record of the frame inputs: |tu|, |tv - (t^u.tv) t^u|, t^u.tv
     float *cl = nullptr, *kk = nullptr;
     int *uid = nullptr, *inv = nullptr;
     BvhNode *nodes = nullptr;
+    int2 *kids = nullptr; // the hierarchy while it is built: children (c >= 0 internal, c < 0 leaf ~c)
     float *boxes = nullptr; // [2n-1][6]
     int *parent = nullptr, *visit = nullptr;
     unsigned *keys = nullptr, *keys_alt = nullptr;
@@ -605,6 +586,7 @@ struct rgs_scene {
         s.N4 = N4;
         s.FU = FU;
         s.FV = FV;
+        s.rec = rec;
         s.cl = cl;
         s.uid = uid;
         s.inv = inv;

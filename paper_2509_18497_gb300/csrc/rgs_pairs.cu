@@ -16,9 +16,11 @@
 // every (receiver, 256-source chunk) block exactly; the fill pass traces each front pair's
 // segment and writes its record at the chunk's offset plus its rank in the block.
 #include <algorithm>
+#include <type_traits>
 #include <vector>
 
 #include "rgs_bounce_body.cuh"
+#include "rgs_warp_trace.cuh"
 
 namespace {
 
@@ -86,16 +88,35 @@ __device__ __forceinline__ float3 unit_dir(float3 dv, float &r) {
     return make_float3(dv.x * inv, dv.y * inv, dv.z * inv);
 }
 
-// occluder k of the segment i -> j (t in (0, r)): a regular hit that is not the source and
-// whose plane is more than eps from the source's centre
-__device__ __forceinline__ bool pair_occluder(const SceneDev &sc, int k, int i, int j, float3 o, float3 d, float r,
-                                              float3 pj, float eps, float &g, float &t) {
+// a hit on surfel k of the segment i -> j occludes it if k is not the source and k's plane is
+// more than eps from the source's centre
+__device__ __forceinline__ bool pair_occludes(const SceneDev &sc, int k, int j, float3 pj, float eps) {
     if (k == j) return false;
-    if (!hit_surfel(sc, k, i, o, d, r, eps, t, g)) return false;
     const float4 Nk = __ldg(&sc.N4[k]);
     const float4 Pk = __ldg(&sc.P[k]);
     const float e = Nk.x * (pj.x - Pk.x) + Nk.y * (pj.y - Pk.y) + Nk.z * (pj.z - Pk.z);
     return fabsf(e) > eps;
+}
+
+// The front sources of a (receiver, 256-source chunk) block in increasing order, packed so that
+// the first warps hold them all and no lane idles beside a source behind the receiver.
+struct PairChunk {
+    int base[PCH / 32];
+    int j[PCH];
+};
+__device__ __forceinline__ int pack_front(PairChunk &s, bool front, int j) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned bal = __ballot_sync(WT_FULL, front);
+    if (lane == 0) s.base[warp] = __popc(bal);
+    __syncthreads();
+    int base = 0, total = 0;
+    for (int w = 0; w < PCH / 32; ++w) {
+        if (w < warp) base += s.base[w];
+        total += s.base[w];
+    }
+    if (front) s.j[base + __popc(bal & ((1u << lane) - 1u))] = j;
+    __syncthreads();
+    return total;
 }
 
 __global__ void __launch_bounds__(PCH) k_pair_count(SceneDev sc, int n, int chunks, int *chunk_cnt, int *src_cnt) {
@@ -111,35 +132,43 @@ __global__ void __launch_bounds__(PCH) k_pair_count(SceneDev sc, int n, int chun
     if (front) atomicAdd(&src_cnt[j], 1);
 }
 
-__global__ void __launch_bounds__(PCH) k_pair_fill(SceneDev sc, int n, int chunks, const long long *__restrict__ chunk_off,
+// A warp per 32 front sources: their segments leave one centre towards neighbouring sources and
+// are traced together (rgs_warp_trace.cuh).
+struct PairWarp {
+    WarpOcclusion w;
+    float4 pj[32]; // the segment's end and its source
+};
+constexpr size_t PAIR_FILL_SMEM = sizeof(PairChunk) + (PCH / 32) * sizeof(PairWarp);
+__global__ void __launch_bounds__(PCH, 3) k_pair_fill(SceneDev sc, int n, int chunks, const long long *__restrict__ chunk_off,
                                                    const float *__restrict__ lam, const float *__restrict__ aarea,
                                                    int2 *rec, int *flags) {
-    __shared__ int warp_base[PCH / 32];
+    extern __shared__ __align__(16) unsigned char pair_smem[];
+    PairChunk &ck = *reinterpret_cast<PairChunk *>(pair_smem);
+    PairWarp &sm = reinterpret_cast<PairWarp *>(pair_smem + sizeof(PairChunk))[threadIdx.x >> 5];
     const int blk = blockIdx.x;
     const int i = blk / chunks, c = blk - i * chunks;
-    const int j = c * PCH + threadIdx.x;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const float eps = *sc.eps_plane;
     const float3 pi = f3(sc.P[i]), ni = f3(sc.N4[i]);
     float3 dv;
-    const bool front = j < n && j != i && pair_front(sc, pi, ni, j, eps, dv);
-    // rank of this pair in the block (sources in increasing order)
-    const unsigned bal = __ballot_sync(0xffffffffu, front);
-    if (lane == 0) warp_base[warp] = __popc(bal);
-    __syncthreads();
-    int base = 0;
-    for (int w = 0; w < warp; ++w) base += warp_base[w];
-    if (!front) return;
-    const int rank = base + __popc(bal & ((1u << lane) - 1u));
-    float r;
+    const int own = c * PCH + threadIdx.x;
+    const int total = pack_front(ck, own < n && own != i && pair_front(sc, pi, ni, own, eps, dv), own);
+    const int rank = threadIdx.x, lane = threadIdx.x & 31;
+    if (rank - lane >= total) return; // whole warps
+    const bool live = rank < total;
+    const int j = ck.j[live ? rank : rank - lane];
+    const float4 Pj = __ldg(&sc.P[j]);
+    dv = make_float3(__fsub_rn(Pj.x, pi.x), __fsub_rn(Pj.y, pi.y), __fsub_rn(Pj.z, pi.z));
+    float r, T;
     const float3 d = unit_dir(dv, r);
-    const float3 pj = f3(sc.P[j]);
-    float T = 1.f;
-    auto visit = [&](int k) {
-        float g, t;
-        if (pair_occluder(sc, k, i, j, pi, d, r, pj, eps, g, t)) T *= 1.f - alpha_of(sc, __ldg(&sc.P[k].w), g);
-    };
-    if (!bvh_traverse(sc, pi, d, r, visit)) atomicAdd(&flags[FLAG_STACK], 1);
+    sm.pj[lane] = make_float4(Pj.x, Pj.y, Pj.z, __int_as_float(j));
+    int nzero;
+    const bool ok = warp_transmittance(sc, sm.w, pi, d, r, i, live, eps, T, nzero, [&](int k, int ray) {
+        const float4 e = sm.pj[ray];
+        return pair_occludes(sc, k, __float_as_int(e.w), f3(e), eps);
+    });
+    if (!ok) atomicAdd(&flags[FLAG_STACK], 1);
+    if (!live) return;
+    if (nzero) T = 0.f;
     const float3 nj = f3(sc.N4[j]);
     const float geo = fabsf(dot3(ni, d)) * fabsf(dot3(nj, d)) / (r * r);
     const float V = __ldg(&lam[j]) * __ldg(&aarea[j]) * T * geo;
@@ -364,65 +393,90 @@ __global__ void __launch_bounds__(PAIR_THREADS) k_pair_g(SceneDev sc, int C, int
 }
 
 // Source-side gradients of every pair, laid out as the fill pass (one block per receiver
-// and 256-source chunk, a thread per source, so a warp's segments leave one centre towards
-// neighbouring sources):
+// and 256-source chunk, the front sources packed, a lane per source):
 //   dL/dlambda_j += g A_j T geo,  dL/do_j += g lambda_j (A_j/o_j) T geo,
-//   dL/do_k += -g lambda_j A_j geo prod_{m != k}(1 - alpha_m) G_k for the segment's occluders
-// (the segment is traced again: once for T and the zero factors, once for the occluders).
+//   dL/do_k += -g lambda_j A_j geo prod_{m != k}(1 - alpha_m) G_k for the segment's occluders.
+// T is V / (lambda_j A_j geo) from the pair's record, so the segment is traced once, for its
+// occluders; only where the record is 0 (an opaque occluder, a T below FP32's range, lambda = 0)
+// does a first trace find T and the zero factors (the 20k-bowl's backward used to trace every
+// segment twice).
 // With dp (and ds) also the geometry gradients of Eqs. dl-dgeo-0/1: the decay term
 // V = lambda_j A_j T geo through geo = (n_i.d)|n_j.d|/r^2, through A_j (proportional to
 // s^u_j s^v_j) and through every occluder's crossing point and scales, plus the directional
 // part gq from k_pair_g; d = (p_j - p_i)/r moves with (I - d d^T)/r (dp_j - dp_i).
+struct PairGradWarp {
+    PairWarp p;
+    float q[32], T[32]; // -g lambda_j A_j geo and the product of the factors that are not 0
+    int nz[32];         // how many are 0
+};
+struct PairGeoWarp {
+    PairGradWarp g;
+    float gp[32][3], gd[32][3];
+};
 template <bool GEO>
-__global__ void __launch_bounds__(PCH) k_pair_grad(SceneDev sc, int n, int chunks, const long long *__restrict__ chunk_off,
-                                                   const float *__restrict__ lam, const float *__restrict__ aarea,
-                                                   const float *__restrict__ daarea, const float *__restrict__ gpair,
-                                                   const float4 *__restrict__ gq, float *dop, float *dlam, float *dp,
-                                                   float *ds, float *gF, int *flags) {
-    __shared__ int warp_base[PCH / 32];
+constexpr size_t PAIR_GRAD_SMEM = sizeof(PairChunk) + (PCH / 32) * (GEO ? sizeof(PairGeoWarp) : sizeof(PairGradWarp));
+template <bool GEO>
+__global__ void __launch_bounds__(PCH, 2) k_pair_grad(SceneDev sc, int n, int chunks, const long long *__restrict__ chunk_off,
+                                                   const int2 *__restrict__ rec, const float *__restrict__ lam,
+                                                   const float *__restrict__ aarea, const float *__restrict__ daarea,
+                                                   const float *__restrict__ gpair, const float4 *__restrict__ gq,
+                                                   float *dop, float *dlam, float *dp, float *ds, float *gF, int *flags) {
+    extern __shared__ __align__(16) unsigned char pair_smem[];
+    PairChunk &ck = *reinterpret_cast<PairChunk *>(pair_smem);
+    using Warp = typename std::conditional<GEO, PairGeoWarp, PairGradWarp>::type;
+    Warp &smw = reinterpret_cast<Warp *>(pair_smem + sizeof(PairChunk))[threadIdx.x >> 5];
+    PairGradWarp &sm = reinterpret_cast<PairGradWarp &>(smw);
     const int blk = blockIdx.x;
     const int i = blk / chunks, c = blk - i * chunks;
-    const int j = c * PCH + threadIdx.x;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const float eps = *sc.eps_plane;
     const float3 pi = f3(sc.P[i]), ni = f3(sc.N4[i]);
     float3 dv;
-    const bool front = j < n && j != i && pair_front(sc, pi, ni, j, eps, dv);
-    const unsigned bal = __ballot_sync(0xffffffffu, front);
-    if (lane == 0) warp_base[warp] = __popc(bal);
-    __syncthreads();
-    int base = 0;
-    for (int w = 0; w < warp; ++w) base += warp_base[w];
+    const int own = c * PCH + threadIdx.x;
+    const int total = pack_front(ck, own < n && own != i && pair_front(sc, pi, ni, own, eps, dv), own);
+    const int rank = threadIdx.x, lane = threadIdx.x & 31;
+    if (rank - lane >= total) return; // whole warps
+    const bool have = rank < total;
+    const int j = ck.j[have ? rank : rank - lane];
+    const long long e = chunk_off[blk] + (have ? rank : rank - lane);
+    const float g = have ? gpair[e] : 0.f;
+    const float4 gs = GEO && have ? gq[e] : make_float4(0.f, 0.f, 0.f, 0.f);
+    const bool live = g != 0.f || gs.x != 0.f || gs.y != 0.f || gs.z != 0.f;
+    const float4 Pj = __ldg(&sc.P[j]);
+    dv = make_float3(__fsub_rn(Pj.x, pi.x), __fsub_rn(Pj.y, pi.y), __fsub_rn(Pj.z, pi.z));
+    float r;
+    const float3 d = unit_dir(dv, r);
+    const float3 nj = f3(sc.N4[j]);
+    const float Aj = __ldg(&aarea[j]), dAj = __ldg(&daarea[j]), lj = __ldg(&lam[j]);
+    const float nid = dot3(ni, d), njd = dot3(nj, d);
+    const float geo = fabsf(nid) * fabsf(njd) / (r * r);
+    sm.p.pj[lane] = make_float4(Pj.x, Pj.y, Pj.z, __int_as_float(j));
+    auto occ = [&](int k, int ray) {
+        const float4 x = sm.p.pj[ray];
+        return pair_occludes(sc, k, __float_as_int(x.w), f3(x), eps);
+    };
+    // T from the record; a record of (nearly) 0 says too little about it
+    const float V = __int_as_float(__ldg(&rec[e].y)), den = lj * Aj * geo;
+    const bool known = fabsf(V) > 1e-30f && fabsf(den) > 1e-30f;
+    float Tnz = known ? V / den : 0.f;
+    int nzero = 0;
+    if (__any_sync(WT_FULL, live && !known)) {
+        float T1;
+        int nz1;
+        if (!warp_transmittance(sc, sm.p.w, pi, d, r, i, live && !known, eps, T1, nz1, occ)) atomicAdd(&flags[FLAG_STACK], 1);
+        if (!known) {
+            Tnz = T1;
+            nzero = nz1;
+        }
+    }
+    const float T = nzero ? 0.f : Tnz;
+    float3 gd = make_float3(gs.x, gs.y, gs.z), gpi = make_float3(0.f, 0.f, 0.f);
     // the receiver's own position and normal terms are summed over the warp (all 32 lanes
     // share receiver i) and added once per warp
     float3 dpi = make_float3(0.f, 0.f, 0.f), gni = make_float3(0.f, 0.f, 0.f);
-    auto body = [&]() {
-        if (!front) return;
-        const long long e = chunk_off[blk] + base + __popc(bal & ((1u << lane) - 1u));
-        const float g = gpair[e];
-        const float4 gs = GEO ? gq[e] : make_float4(0.f, 0.f, 0.f, 0.f);
-        if (g == 0.f && gs.x == 0.f && gs.y == 0.f && gs.z == 0.f) return;
-        float r;
-        const float3 d = unit_dir(dv, r);
-        const float3 pj = f3(sc.P[j]), nj = f3(sc.N4[j]);
-        const float Aj = __ldg(&aarea[j]), dAj = __ldg(&daarea[j]), lj = __ldg(&lam[j]);
-        const float nid = dot3(ni, d), njd = dot3(nj, d);
-        const float geo = fabsf(nid) * fabsf(njd) / (r * r);
-        float Tnz = 1.f;
-        int nzero = 0;
-        auto pass1 = [&](int k) {
-            float gk, tk;
-            if (!pair_occluder(sc, k, i, j, pi, d, r, pj, eps, gk, tk)) return;
-            const float om = 1.f - alpha_of(sc, __ldg(&sc.P[k].w), gk);
-            if (om == 0.f) ++nzero;
-            else Tnz *= om;
-        };
-        if (!bvh_traverse(sc, pi, d, r, pass1)) atomicAdd(&flags[FLAG_STACK], 1);
-        const float T = nzero ? 0.f : Tnz;
+    float gr = 0.f;
+    if (live) {
         if (dlam) atomicAdd(&dlam[j], g * Aj * T * geo);
         if (dop && T != 0.f) atomicAdd(&dop[j], g * lj * dAj * T * geo);
-        float3 gd = make_float3(gs.x, gs.y, gs.z), gpi = make_float3(0.f, 0.f, 0.f);
-        float gr = 0.f;
         if constexpr (GEO) {
             const float f = g * lj * Aj * T / (r * r), sj = njd >= 0.f ? 1.f : -1.f;
             gd = gd + f * (fabsf(njd) * ni + (fabsf(nid) * sj) * nj);
@@ -434,43 +488,64 @@ __global__ void __launch_bounds__(PCH) k_pair_grad(SceneDev sc, int n, int chunk
             gni = gni + fi * d;
             geo_add3(gF + GEO_GF * (size_t)j + GEO_N, fj * d);
         }
-        if ((dop || GEO) && nzero <= 1 && g != 0.f) {
-            const float q = -g * lj * Aj * geo;
-            auto pass2 = [&](int k) {
-                float gk, tk;
-                if (!pair_occluder(sc, k, i, j, pi, d, r, pj, eps, gk, tk)) return;
-                const float ok = __ldg(&sc.P[k].w);
-                const float om = 1.f - alpha_of(sc, ok, gk);
-                float others;
-                if (nzero == 0) others = Tnz / om;
-                else others = (om == 0.f) ? Tnz : 0.f;
-                if (others == 0.f) return;
-                if (dop) atomicAdd(&dop[k], q * others * dalpha_do(sc, ok, gk));
-                if constexpr (GEO) {
-                    const float coef = q * others * dalpha_dq(sc, ok, gk);
-                    if (coef == 0.f) return;
-                    float uu, vv;
-                    const float3 pw = crossing_pw(sc, k, pi, d, tk, uu, vv);
-                    gpi = gpi + coef * pw;
-                    gd = gd + (coef * tk) * pw;
-                    geo_add3(dp + GEO_DP * (size_t)k, (-coef) * pw);
-                    geo_add2(ds + 2 * (size_t)k, coef * (-2.f * uu * uu * __ldg(&sc.FU[k].w)),
-                             coef * (-2.f * vv * vv * __ldg(&sc.FV[k].w)));
-                    occluder_frame_grad(sc, k, pi, d, tk, uu, vv, coef, gF);
+    }
+    const bool second = live && (dop || GEO) && nzero <= 1 && g != 0.f;
+    if (__any_sync(WT_FULL, second)) {
+        sm.q[lane] = -g * lj * Aj * geo;
+        sm.T[lane] = Tnz;
+        sm.nz[lane] = nzero;
+        sm.p.w.d[lane] = make_float4(d.x, d.y, d.z, r);
+        sm.p.w.own.who[lane] = 0u;
+        __syncwarp();
+        auto test = [&](int k, int ray, bool valid) {
+            bool terms = false;
+            if (valid) {
+                const float4 rd = sm.p.w.d[ray];
+                const float3 dd = f3(rd);
+                float t, gk, ok;
+                if (hit_surfel(sc, k, i, pi, dd, rd.w, eps, t, gk, ok) && occ(k, ray)) {
+                    const float om = 1.f - alpha_of(sc, ok, gk);
+                    const float others = sm.nz[ray] == 0 ? sm.T[ray] / om : (om == 0.f ? sm.T[ray] : 0.f);
+                    if (others != 0.f) {
+                        const float q = sm.q[ray];
+                        if (dop) atomicAdd(&dop[k], q * others * dalpha_do(sc, ok, gk));
+                        if constexpr (GEO) {
+                            const float coef = q * others * dalpha_dq(sc, ok, gk);
+                            if (coef != 0.f) {
+                                terms = true;
+                                float uu, vv;
+                                const float3 pw = crossing_pw(sc, k, pi, dd, t, uu, vv);
+                                smw.gp[lane][0] = coef * pw.x;
+                                smw.gp[lane][1] = coef * pw.y;
+                                smw.gp[lane][2] = coef * pw.z;
+                                smw.gd[lane][0] = (coef * t) * pw.x;
+                                smw.gd[lane][1] = (coef * t) * pw.y;
+                                smw.gd[lane][2] = (coef * t) * pw.z;
+                                geo_add3(dp + GEO_DP * (size_t)k, (-coef) * pw);
+                                geo_add2(ds + 2 * (size_t)k, coef * (-2.f * uu * uu * __ldg(&sc.FU[k].w)),
+                                         coef * (-2.f * vv * vv * __ldg(&sc.FV[k].w)));
+                                occluder_frame_grad(sc, k, pi, dd, t, uu, vv, coef, gF);
+                            }
+                        }
+                    }
                 }
-            };
-            bvh_traverse(sc, pi, d, r, pass2);
-        }
-        if constexpr (GEO) {
-            const float dd = dot3(d, gd);
-            const float3 gp = make_float3((gd.x - d.x * dd) / r + d.x * gr, (gd.y - d.y * dd) / r + d.y * gr,
-                                          (gd.z - d.z * dd) / r + d.z * gr);
-            geo_add3(dp + GEO_DP * (size_t)j, gp);
-            dpi = gpi - gp;
-        }
-    };
-    body();
+            }
+            if constexpr (GEO)
+                warp_owner_loop(sm.p.w.own, terms, ray, [&](int b) {
+                    gpi = gpi + make_float3(smw.gp[b][0], smw.gp[b][1], smw.gp[b][2]);
+                    gd = gd + make_float3(smw.gd[b][0], smw.gd[b][1], smw.gd[b][2]);
+                });
+        };
+        if (!warp_traverse<false>(sc, pi, d, r, second, sm.p.w.q, test, [](float m) { return m; })) atomicAdd(&flags[FLAG_STACK], 1);
+    }
     if constexpr (!GEO) return;
+    if (live) {
+        const float dd = dot3(d, gd);
+        const float3 gp = make_float3((gd.x - d.x * dd) / r + d.x * gr, (gd.y - d.y * dd) / r + d.y * gr,
+                                      (gd.z - d.z * dd) / r + d.z * gr);
+        geo_add3(dp + GEO_DP * (size_t)j, gp);
+        dpi = gpi - gp;
+    }
     float red[6] = {dpi.x, dpi.y, dpi.z, gni.x, gni.y, gni.z};
 #pragma unroll
     for (int q = 0; q < 6; ++q)
@@ -583,7 +658,8 @@ rgs_status rgs_trace_pairs_impl(rgs_transport *t, const rgs_lights *L, const flo
     t->n_hits = total;
     t->n_slots = total;
     t->n_full = 0;
-    { ProfScope ps_("k_pair_fill", st); k_pair_fill<<<(unsigned)nchunk, PCH, 0, st>>>(sd, n, chunks, t->chunk_off, t->lam, t->aarea, t->pair_rec, t->flags); }
+    RGS_CUDA(cudaFuncSetAttribute(k_pair_fill, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PAIR_FILL_SMEM));
+    { ProfScope ps_("k_pair_fill", st); k_pair_fill<<<(unsigned)nchunk, PCH, PAIR_FILL_SMEM, st>>>(sd, n, chunks, t->chunk_off, t->lam, t->aarea, t->pair_rec, t->flags); }
     { ProfScope ps_("k_pair_off", st); k_pair_off<<<(n + 256) / 256, 256, 0, st>>>(t->chunk_off, chunks, n, t->pair_off); }
     RGS_LAUNCH("pair fill");
     if ((r = rgs_direct_term(t, st)) != RGS_OK) return r;
@@ -664,11 +740,13 @@ rgs_status run_adjoint_pairs(rgs_transport *t, const float *g, float *dE, float 
             k_pair_g<NC, false><<<n, PAIR_THREADS, 0, st>>>(sd, C, nb, t->pair_off, t->pair_rec, A, t->v, t->iters, t->gh, nullptr, nullptr);
         }
         if (geo.dp) {
+            RGS_CUDA(cudaFuncSetAttribute(k_pair_grad<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PAIR_GRAD_SMEM<true>));
             ProfScope ps_("k_pair_grad", st);
-            k_pair_grad<true><<<(unsigned)((long long)n * chunks), PCH, 0, st>>>(sd, n, chunks, t->chunk_off, t->lam, t->aarea, t->daarea, t->gh, geo.gq, dopo ? t->dop : nullptr, dlam_acc, geo.dp, geo.ds, geo.gF, t->flags);
+            k_pair_grad<true><<<(unsigned)((long long)n * chunks), PCH, PAIR_GRAD_SMEM<true>, st>>>(sd, n, chunks, t->chunk_off, t->pair_rec, t->lam, t->aarea, t->daarea, t->gh, geo.gq, dopo ? t->dop : nullptr, dlam_acc, geo.dp, geo.ds, geo.gF, t->flags);
         } else {
+            RGS_CUDA(cudaFuncSetAttribute(k_pair_grad<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PAIR_GRAD_SMEM<false>));
             ProfScope ps_("k_pair_grad", st);
-            k_pair_grad<false><<<(unsigned)((long long)n * chunks), PCH, 0, st>>>(sd, n, chunks, t->chunk_off, t->lam, t->aarea, t->daarea, t->gh, nullptr, dopo ? t->dop : nullptr, dlam_acc, nullptr, nullptr, nullptr, t->flags);
+            k_pair_grad<false><<<(unsigned)((long long)n * chunks), PCH, PAIR_GRAD_SMEM<false>, st>>>(sd, n, chunks, t->chunk_off, t->pair_rec, t->lam, t->aarea, t->daarea, t->gh, nullptr, dopo ? t->dop : nullptr, dlam_acc, nullptr, nullptr, nullptr, t->flags);
         }
         RGS_LAUNCH("pair backward");
     }

@@ -153,7 +153,7 @@ __global__ void k_radix_scatter(const unsigned *__restrict__ kin, const int *__r
 
 // ---------------------------------------------------------------- surfel gather
 __global__ void k_gather(rgs_surfels in, int n, int L, int alpha_model, const int *__restrict__ perm, float4 *P,
-                         float4 *N4, float4 *FU, float4 *FV, float4 *GS, float *cl, float *kk, int *uid, int *inv,
+                         float4 *N4, float4 *FU, float4 *FV, SurfelRec *rec, float4 *GS, float *cl, float *kk, int *uid, int *inv,
                          float *boxes, int *flags) {
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
@@ -178,6 +178,7 @@ __global__ void k_gather(rgs_surfels in, int n, int L, int alpha_model, const in
     N4[k] = make_float4(nn.x, nn.y, nn.z, 0.f);
     FU[k] = make_float4(a.x, a.y, a.z, 1.f / su);
     FV[k] = make_float4(b.x, b.y, b.z, 1.f / sv);
+    rec[k] = SurfelRec{P[k], N4[k], FU[k], FV[k]};
     // BRDF coefficients (App. A): c_0 = 4 k a^d + (1-k) a^s, c_l = (1-k) a^s rho_l(s)
     float kd = in.k[i], s = in.shin[i];
     float rho[4] = {1.f, (s + 1.f) / (s + 2.f), s / (s + 3.f), (s + 1.f) * (s - 1.f) / ((s + 2.f) * (s + 4.f))};
@@ -215,7 +216,7 @@ __device__ __forceinline__ int delta(const unsigned *keys, int n, int i, int j) 
     return 32 + __clz((unsigned)i ^ (unsigned)j);
 }
 
-__global__ void k_karras(const unsigned *__restrict__ keys, int n, BvhNode *nodes, int *parent, int *visit) {
+__global__ void k_karras(const unsigned *__restrict__ keys, int n, int2 *kids, int *parent, int *visit) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n - 1) return;
     visit[i] = 0;
@@ -236,14 +237,14 @@ __global__ void k_karras(const unsigned *__restrict__ keys, int n, BvhNode *node
     int gamma = i + s * d + min(d, 0);
     int left = (min(i, j) == gamma) ? ~gamma : gamma;
     int right = (max(i, j) == gamma + 1) ? ~(gamma + 1) : gamma + 1;
-    nodes[i].d = make_int4(left, right, 0, 0);
+    kids[i] = make_int2(left, right); // ~gamma or gamma, ~(gamma + 1) or gamma + 1
     // parent array over all 2n-1 nodes: internal x -> x, leaf k -> n-1+k
     parent[left < 0 ? (n - 1 + ~left) : left] = i;
     parent[right < 0 ? (n - 1 + ~right) : right] = i;
 }
 
 // bottom-up refit: each leaf walks up; the second visitor of a node computes its box
-__global__ void k_refit(int n, const BvhNode *__restrict__ nodes, const int *__restrict__ parent, int *visit,
+__global__ void k_refit(int n, const int2 *__restrict__ kids, const int *__restrict__ parent, int *visit,
                         float *boxes) {
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
@@ -252,7 +253,7 @@ __global__ void k_refit(int n, const BvhNode *__restrict__ nodes, const int *__r
         __threadfence();
         if (atomicAdd(&visit[x], 1) == 0) return; // first arrival: the sibling will finish
         __threadfence();
-        int4 c = nodes[x].d;
+        const int2 c = kids[x];
         const volatile float *bl = boxes + (size_t)(c.x < 0 ? (n - 1 + ~c.x) : c.x) * 6;
         const volatile float *br = boxes + (size_t)(c.y < 0 ? (n - 1 + ~c.y) : c.y) * 6;
         volatile float *bx = boxes + (size_t)x * 6;
@@ -265,15 +266,67 @@ __global__ void k_refit(int n, const BvhNode *__restrict__ nodes, const int *__r
     }
 }
 
-__global__ void k_pack(int n, BvhNode *nodes, const float *__restrict__ boxes) {
+// The traversal's four-wide node i from the binary node i: its grandchildren (a child that is a
+// leaf stands for itself), their boxes in 8 bits per coordinate, rounded outwards on the grid
+// of their union.  Infinite sides are cut at 1e18 (the node then covers everything).  A walk
+// from the root only meets nodes of even depth; the others are written all the same.
+__global__ void k_pack(int n, const int2 *__restrict__ kids, const float *__restrict__ boxes, BvhNode *nodes) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n - 1) return;
-    int4 c = nodes[i].d;
-    const float *bl = boxes + (size_t)(c.x < 0 ? (n - 1 + ~c.x) : c.x) * 6;
-    const float *br = boxes + (size_t)(c.y < 0 ? (n - 1 + ~c.y) : c.y) * 6;
-    nodes[i].a = make_float4(bl[0], bl[1], bl[2], bl[3]);
-    nodes[i].b = make_float4(bl[4], bl[5], br[0], br[1]);
-    nodes[i].c = make_float4(br[2], br[3], br[4], br[5]);
+    const int2 c = kids[i];
+    int kid[4], m = 0;
+    const int two[2] = {c.x, c.y};
+    for (int q = 0; q < 2; ++q) {
+        if (two[q] < 0) {
+            kid[m++] = two[q];
+        } else {
+            const int2 g = kids[two[q]];
+            kid[m++] = g.x;
+            kid[m++] = g.y;
+        }
+    }
+    float lo[4][3], hi[4][3], org[3], ext = 0.f;
+    for (int a = 0; a < 3; ++a) {
+        float l = INFINITY, h = -INFINITY;
+        for (int q = 0; q < m; ++q) {
+            const float *b = boxes + (size_t)(kid[q] < 0 ? (n - 1 + ~kid[q]) : kid[q]) * 6;
+            lo[q][a] = fmaxf(b[a], -1e18f);
+            hi[q][a] = fminf(b[3 + a], 1e18f);
+            l = fminf(l, lo[q][a]);
+            h = fmaxf(h, hi[q][a]);
+        }
+        org[a] = l;
+        ext = fmaxf(ext, h - l);
+    }
+    const float scale = fmaxf(ext / 253.f, 1e-30f), inv = 1.f / scale;
+    unsigned wl[3] = {0u, 0u, 0u}, wh[3] = {0u, 0u, 0u}, mask = 0u;
+    BvhNode out;
+    for (int q = 0; q < 4; ++q) out.kid[q] = 0;
+    for (int q = 0; q < m; ++q) {
+        for (int a = 0; a < 3; ++a) {
+            int ql = min(max((int)floorf((lo[q][a] - org[a]) * inv), 0), 255);
+            int qh = min(max((int)ceilf((hi[q][a] - org[a]) * inv), 0), 255);
+            while (ql > 0 && org[a] + scale * (float)ql > lo[q][a]) --ql;
+            while (qh < 255 && org[a] + scale * (float)qh < hi[q][a]) ++qh;
+            wl[a] |= (unsigned)ql << (8 * q);
+            wh[a] |= (unsigned)qh << (8 * q);
+        }
+        mask |= (kid[q] < 0 ? 0x10u : 1u) << q;
+        out.kid[q] = kid[q] < 0 ? ~kid[q] : kid[q];
+    }
+    out.ox = org[0];
+    out.oy = org[1];
+    out.oz = org[2];
+    out.scale = scale;
+    out.lox = wl[0];
+    out.hix = wh[0];
+    out.loy = wl[1];
+    out.hiy = wh[1];
+    out.loz = wl[2];
+    out.hiz = wh[2];
+    out.mask = mask;
+    out.pad = 0u;
+    nodes[i] = out;
 }
 
 // ---------------------------------------------------------------- int -> int64 scan
@@ -363,8 +416,8 @@ rgs_status rgs_scene_build_impl(rgs_scene *s, const rgs_surfels *in, const rgs_b
         s->cap = 0;                                                                                                    \
         return r;                                                                                                      \
     }
-        ALLOC(P, n) ALLOC(N4, n) ALLOC(FU, n) ALLOC(FV, n) ALLOC(GS, n) ALLOC(cl, (size_t)n * 12) ALLOC(kk, n) ALLOC(uid, n)
-        ALLOC(inv, n) ALLOC(nodes, n > 1 ? n - 1 : 1) ALLOC(boxes, (size_t)(2 * n - 1) * 6) ALLOC(parent, 2 * n)
+        ALLOC(P, n) ALLOC(N4, n) ALLOC(FU, n) ALLOC(FV, n) ALLOC(rec, n) ALLOC(GS, n) ALLOC(cl, (size_t)n * 12) ALLOC(kk, n) ALLOC(uid, n)
+        ALLOC(inv, n) ALLOC(nodes, n > 1 ? n - 1 : 1) ALLOC(kids, n > 1 ? n - 1 : 1) ALLOC(boxes, (size_t)(2 * n - 1) * 6) ALLOC(parent, 2 * n)
         ALLOC(visit, n) ALLOC(keys, n) ALLOC(keys_alt, n) ALLOC(vals, n) ALLOC(vals_alt, n)
 #undef ALLOC
         s->hist_cap = 256 * ((n + SORT_TILE - 1) / SORT_TILE);
@@ -403,13 +456,13 @@ rgs_status rgs_scene_build_impl(rgs_scene *s, const rgs_surfels *in, const rgs_b
     }
     RGS_LAUNCH("radix sort");
     // after an even number of passes ka == keys, va == vals
-    { ProfScope ps_("k_gather", st); k_gather<<<(n + 127) / 128, 128, 0, st>>>(*in, n, s->L, s->alpha_model, va, s->P, s->N4, s->FU, s->FV, s->GS, s->cl,
+    { ProfScope ps_("k_gather", st); k_gather<<<(n + 127) / 128, 128, 0, st>>>(*in, n, s->L, s->alpha_model, va, s->P, s->N4, s->FU, s->FV, s->rec, s->GS, s->cl,
                                               s->kk, s->uid, s->inv, s->boxes, s->flags); }
     RGS_LAUNCH("gather");
     if (n > 1) {
-        { ProfScope ps_("k_karras", st); k_karras<<<(n - 1 + 255) / 256, 256, 0, st>>>(ka, n, s->nodes, s->parent, s->visit); }
-        { ProfScope ps_("k_refit", st); k_refit<<<(n + 255) / 256, 256, 0, st>>>(n, s->nodes, s->parent, s->visit, s->boxes); }
-        { ProfScope ps_("k_pack", st); k_pack<<<(n - 1 + 255) / 256, 256, 0, st>>>(n, s->nodes, s->boxes); }
+        { ProfScope ps_("k_karras", st); k_karras<<<(n - 1 + 255) / 256, 256, 0, st>>>(ka, n, s->kids, s->parent, s->visit); }
+        { ProfScope ps_("k_refit", st); k_refit<<<(n + 255) / 256, 256, 0, st>>>(n, s->kids, s->parent, s->visit, s->boxes); }
+        { ProfScope ps_("k_pack", st); k_pack<<<(n - 1 + 255) / 256, 256, 0, st>>>(n, s->kids, s->boxes, s->nodes); }
         RGS_LAUNCH("bvh");
     }
     if (o && o->check_finite) {

@@ -1,172 +1,135 @@
 // Transport tracing (rgs_trace_transport).
 //
-//  k_trace_hemi : one thread per hemisphere ray (App. B); a warp is 32 consecutive rays
-//                 of one surfel.  Hits are collected during BVH traversal, put in depth
-//                 order (near-equal depths by caller index), alpha-composited (Eq. L_I)
-//                 and stored as warp-interleaved records (coalesced 256-B rows).
-//  k_direct     : one thread per (surfel, light) shadow ray; transmittance product and
+//  k_trace_hemi : a warp per 32 hemisphere rays (App. B) of one surfel.  Hits are collected
+//                 during BVH traversal, put in depth order (near-equal depths by caller
+//                 index), alpha-composited (Eq. L_I) and stored contiguously per ray.
+//  k_direct     : a lane per (surfel, light) shadow ray; transmittance product and
 //                 the direct term D (Sec. 5.2) for every column of that light.
 //  k_src_*      : the same records grouped by source surfel (transposed index) for the
 //                 adjoint's gather form of K^T.
 #include <algorithm>
 
-#include "rgs_internal.cuh"
+#include "rgs_warp_trace.cuh"
 
 #ifndef RGS_TRACE_PATCH_A
 #define RGS_TRACE_PATCH_A 8
 #endif
 #ifndef RGS_TRACE_MINB
-#define RGS_TRACE_MINB 12 // resident 128-thread blocks per SM the register budget is sized for (measured best)
+#define RGS_TRACE_MINB 8 // resident 128-thread blocks per SM the register budget is sized for (measured best)
 #endif
+constexpr int HEMI_THREADS = 128, DIRECT_THREADS = 128;
 
 namespace {
 
-// One thread per hemisphere ray; the 32 rays of a warp belong to one surfel.
-// Hits are kept as one 64-bit key each, (bits of t) << 32 | j: t > 0, so the unsigned key
-// order is the depth order and ties of exactly equal t fall back to the internal index
-// (such ties are always re-ordered inside their run).  After compositing, the warp
-// allocates exactly its rays' kept hits with one atomic (prefix sum over the lanes) and
-// every ray stores its records contiguously.
-__global__ void __launch_bounds__(128, RGS_TRACE_MINB) k_trace_hemi(SceneDev sc, RaysDev rays, int n_rays, long long cap_slots,
-                                                       unsigned long long *slot_ctr, int2 *rec_ja,
+// A warp per patch of 32 rays of one surfel, patches handed out by a counter.  The lanes walk
+// the tree for their own rays and pool the surfel tests (rgs_warp_trace.cuh); accepted hits
+// go to per-ray lists in this warp's scratch (rewritten for every patch, so it stays in
+// L2), each ray's traversal ends once the hits found make the rest invisible, and the warp
+// then orders and composites one ray after the other, a lane per hit.  It allocates exactly
+// its rays' kept hits with one atomic and stores every ray's records contiguously.
+__global__ void __launch_bounds__(HEMI_THREADS, RGS_TRACE_MINB) k_trace_hemi(SceneDev sc, RaysDev rays, int n_patches, long long cap_slots,
+                                                       unsigned long long *slot_ctr, unsigned *work, int2 *rec_ja,
                                                        long long *off_out, int *cnt_out, float4 *dir_out,
-                                                       int *src_cnt, int *flags, int pa) {
-    const unsigned FULL = 0xffffffffu;
-    const int tid = blockIdx.x * blockDim.x + threadIdx.x;
-    if (tid - (int)(threadIdx.x & 31) >= n_rays) return; // whole warps only (n_rays % 32 == 0)
+                                                       int *src_cnt, int *flags, int pa, int4 *lists) {
+    __shared__ WarpHits sm_all[HEMI_THREADS / 32];
     const int lane = threadIdx.x & 31;
-    // the warps of surfel i take patches of pa x (32 / pa) strata (elevation x azimuth) of its
-    // na x nbs grid, so that a warp's rays leave in similar directions; pa = 0: 32 consecutive rays
-    const int i = tid / rays.nd;
-    int q = tid - i * rays.nd;
-    if (pa > 0) {
-        const int pb = 32 / pa, w = q >> 5, per_row = rays.nbs / pb;
-        const int a = (w / per_row) * pa + lane / pb, b = (w % per_row) * pb + lane % pb;
-        q = a * rays.nbs + b;
-    }
-    const int r = i * rays.nd + q; // the ray this thread traces (outputs are indexed by ray)
-    const float3 o = f3(sc.P[i]);
-    const float3 d = ray_dir(rays.seed, sc.uid[i], q, rays.na, rays.nbs, f3(sc.FU[i]), f3(sc.FV[i]), f3(sc.N4[i]));
-    dir_out[r] = make_float4(d.x, d.y, d.z, 0.f);
+    WarpHits &sm = sm_all[threadIdx.x >> 5];
+    int4 *list = lists + (size_t)(blockIdx.x * (HEMI_THREADS / 32) + (threadIdx.x >> 5)) * (32 * WT_LIST);
     const float eps = *sc.eps_plane;
-
-    unsigned long long key[RGS_HMAX];
-    int H = 0;
-    bool full = false;
-    auto visit = [&](int j) {
-        float t, r2;
-        if (!hit_surfel_t(sc, j, i, o, d, INFINITY, eps, t, r2)) return;
-        const unsigned long long k = ((unsigned long long)__float_as_uint(t) << 32) | (unsigned)j;
-        if (H < RGS_HMAX) {
-            key[H++] = k;
-            return;
+    const int per = rays.nd >> 5; // patches of a surfel
+    while (true) {
+        unsigned w = 0;
+        if (lane == 0) w = atomicAdd(work, 1u);
+        w = __shfl_sync(WT_FULL, w, 0);
+        if (w >= (unsigned)n_patches) return;
+        // the warps of surfel i take patches of pa x (32 / pa) strata (elevation x azimuth) of its
+        // na x nbs grid, so that a warp's rays leave in similar directions; pa = 0: 32 consecutive rays
+        const int i = (int)(w / (unsigned)per), pt = (int)(w - (unsigned)i * (unsigned)per);
+        int q = pt * 32 + lane;
+        if (pa > 0) {
+            const int pb = 32 / pa, per_row = rays.nbs / pb;
+            const int a = (pt / per_row) * pa + lane / pb, b = (pt % per_row) * pb + lane % pb;
+            q = a * rays.nbs + b;
         }
-        full = true; // keep the RGS_HMAX nearest: replace the farthest if this one is nearer
-        int far = 0;
-        for (int m = 1; m < RGS_HMAX; ++m)
-            if (key[m] > key[far]) far = m;
-        if (k < key[far]) key[far] = k;
-    };
-    if (!bvh_traverse_ordered(sc, o, d, visit)) atomicAdd(&flags[FLAG_STACK], 1);
-
-    for (int a = 1; a < H; ++a) { // insertion sort by key (hits arrive almost sorted)
-        const unsigned long long k = key[a];
-        int b = a - 1;
-        while (b >= 0 && key[b] > k) {
-            key[b + 1] = key[b];
-            --b;
-        }
-        key[b + 1] = k;
-    }
-    for (int k0 = 0; k0 < H;) { // runs of near-equal depth are ordered by caller index
-        int e = k0;
-        float te = __uint_as_float((unsigned)(key[e] >> 32));
-        while (e + 1 < H) {
-            const float tn = __uint_as_float((unsigned)(key[e + 1] >> 32));
-            if (tn - te > 1e-6f * fmaxf(1.f, te)) break;
-            ++e;
-            te = tn;
-        }
-        for (int a = k0 + 1; a <= e; ++a) {
-            const unsigned long long k = key[a];
-            const int uk = sc.uid[(int)(unsigned)k];
-            int b = a - 1;
-            while (b >= k0 && sc.uid[(int)(unsigned)key[b]] > uk) {
-                key[b + 1] = key[b];
-                --b;
+        const int r = i * rays.nd + q; // this lane's ray (outputs are indexed by ray)
+        const float3 o = f3(sc.P[i]);
+        const float3 d = ray_dir(rays.seed, sc.uid[i], q, rays.na, rays.nbs, f3(sc.FU[i]), f3(sc.FV[i]), f3(sc.N4[i]));
+        dir_out[r] = make_float4(d.x, d.y, d.z, 0.f);
+        bool full;
+        if (!warp_collect<false>(sc, o, d, i, true, eps, 0, sm, list, full)) atomicAdd(&flags[FLAG_STACK], 1);
+        int kept = 0; // of this lane's ray
+        for (int x = 0; x < 32; ++x) {
+            int H = sm.cnt[x];
+            if (H == 0) continue;
+            float T = 1.f;
+            unsigned long long last;
+            const int k = warp_composite_any(sc, H, list + x * WT_LIST, sm, false, T, last);
+            __syncwarp();
+            if (lane == x) {
+                kept = k;
+                // a full list only loses something if the transmittance is still above the cut
+                if (full && k == H && T >= RGS_T_EPS) atomicAdd(&flags[FLAG_FULL_RAYS], 1);
             }
-            key[b + 1] = k;
         }
-        k0 = e + 1;
-    }
-    // composite: a_h = alpha_h prod_{k<h} (1 - alpha_k); stop below RGS_T_EPS
-    int kept = 0;
-    {
-        float T = 1.f;
-        for (; kept < H; ++kept) {
-            if (T < RGS_T_EPS) break;
-            const int j = (int)(unsigned)key[kept];
-            T *= 1.f - alpha_of(sc, __ldg(&sc.P[j].w),
-                                surfel_G(sc, surfel_r2(sc, j, o, d, __uint_as_float((unsigned)(key[kept] >> 32)))));
-        }
-        // a full buffer only loses something if the transmittance is still above the cut
-        if (full && kept == H && T >= RGS_T_EPS) atomicAdd(&flags[FLAG_FULL_RAYS], 1);
-    }
-    // warp-aggregated, exactly sized record allocation
-    int incl = kept;
+        // warp-aggregated, exactly sized record allocation
+        int incl = kept;
 #pragma unroll
-    for (int offs = 1; offs < 32; offs <<= 1) {
-        const int v = __shfl_up_sync(FULL, incl, offs);
-        if (lane >= offs) incl += v;
-    }
-    const int total = __shfl_sync(FULL, incl, 31);
-    unsigned long long sbase = 0;
-    if (lane == 31 && total > 0) sbase = atomicAdd(slot_ctr, (unsigned long long)total);
-    sbase = __shfl_sync(FULL, sbase, 31);
-    const unsigned long long mine = sbase + (unsigned long long)(incl - kept);
-    const bool fits = mine + (unsigned long long)kept <= (unsigned long long)cap_slots;
-    off_out[r] = (long long)mine;
-    cnt_out[r] = fits ? kept : 0;
-    if (!fits) {
-        atomicAdd(&flags[FLAG_CAPACITY], 1);
-        return;
-    }
-    float T = 1.f;
-    for (int h = 0; h < kept; ++h) {
-        const int j = (int)(unsigned)key[h];
-        const float G = surfel_G(sc, surfel_r2(sc, j, o, d, __uint_as_float((unsigned)(key[h] >> 32))));
-        const float alpha = alpha_of(sc, __ldg(&sc.P[j].w), G);
-        rec_ja[mine + h] = make_int2(j, __float_as_int(alpha * T));
-        T *= 1.f - alpha;
-        atomicAdd(&src_cnt[j], 1); // transposed-index histogram
+        for (int offs = 1; offs < 32; offs <<= 1) {
+            const int v = __shfl_up_sync(WT_FULL, incl, offs);
+            if (lane >= offs) incl += v;
+        }
+        const int total = __shfl_sync(WT_FULL, incl, 31);
+        unsigned long long sbase = 0;
+        if (lane == 31 && total > 0) sbase = atomicAdd(slot_ctr, (unsigned long long)total);
+        sbase = __shfl_sync(WT_FULL, sbase, 31);
+        const unsigned long long mine = sbase + (unsigned long long)(incl - kept);
+        const bool fits = mine + (unsigned long long)kept <= (unsigned long long)cap_slots;
+        off_out[r] = (long long)mine;
+        cnt_out[r] = fits ? kept : 0;
+        if (!fits) atomicAdd(&flags[FLAG_CAPACITY], 1);
+        const unsigned store = __ballot_sync(WT_FULL, fits && kept > 0);
+        for (unsigned m = store; m; m &= m - 1) {
+            const int x = __ffs(m) - 1;
+            const int k = __shfl_sync(WT_FULL, kept, x);
+            int2 *out = rec_ja + sbase + (unsigned)__shfl_sync(WT_FULL, incl - kept, x);
+            for (int e = lane; e < k; e += 32) {
+                const int2 ja = wt_hit(list + x * WT_LIST, e);
+                out[e] = ja;
+                atomicAdd(&src_cnt[ja.x], 1); // transposed-index histogram
+            }
+        }
+        __syncwarp(); // the lists are rewritten by the next patch
     }
 }
 
 // Direct term (Sec. 5.2): D_i[L*3+ch][k] = o_i c_{i,l(k),ch} Y_k(R_i w) I_{L,ch} (n_i.w)/r^2 T
 // (no 1/r^2 and a shadow ray to infinity for a directional light)
+// A warp per 32 (surfel, light) pairs, their shadow rays traced together (rgs_warp_trace.cuh).
 template <int NC>
-__global__ void k_direct(SceneDev sc, int nl, int ldir, const float *__restrict__ lpos, const float *__restrict__ lint,
-                         int C, float *D, int *flags) {
+__global__ void __launch_bounds__(DIRECT_THREADS) k_direct(SceneDev sc, int nl, int ldir, const float *__restrict__ lpos,
+                                                          const float *__restrict__ lint, int C, float *D, int *flags) {
+    __shared__ WarpOcclusion sm[DIRECT_THREADS / 32];
     const int tid = blockIdx.x * blockDim.x + threadIdx.x;
-    if (tid >= sc.n * nl) return;
-    const int i = tid / nl, lt = tid - i * nl;
+    const bool live = tid < sc.n * nl;
+    const int i = live ? tid / nl : 0, lt = live ? tid - i * nl : 0;
     const float4 Pi = sc.P[i];
     const float3 o = f3(Pi), n = f3(sc.N4[i]);
     float r, fall;
     const float3 w = light_dir(lpos, lt, o, ldir, r, fall);
     const float cs = dot3(n, w);
+    const bool lit = live && cs > 0.f;
+    float T;
+    int nzero;
+    if (!warp_transmittance(sc, sm[threadIdx.x >> 5], o, w, r, i, lit, *sc.eps_plane, T, nzero,
+                            [](int, int) { return true; }))
+        atomicAdd(&flags[FLAG_STACK], 1);
+    if (!live) return;
     float *Dout = D + ((size_t)i * C + lt * 3) * NC;
-    if (!(cs > 0.f)) {
+    if (!lit) {
         for (int q = 0; q < 3 * NC; ++q) Dout[q] = 0.f;
         return;
     }
-    const float eps = *sc.eps_plane;
-    float T = 1.f;
-    auto visit = [&](int j) {
-        float t, g;
-        if (hit_surfel(sc, j, i, o, w, r, eps, t, g)) T *= 1.f - alpha_of(sc, __ldg(&sc.P[j].w), g);
-    };
-    if (!bvh_traverse(sc, o, w, r, visit)) atomicAdd(&flags[FLAG_STACK], 1);
+    if (nzero) T = 0.f;
     float Y[NC];
     sh_eval<NC>(reflect_n(n, w), Y);
     const float pre = alpha_center(sc, i) * cs * fall * T;
@@ -233,10 +196,10 @@ rgs_status rgs_direct_term(rgs_transport *t, cudaStream_t st) {
     if (t->nl > 0) {
         const int nth = t->n * t->nl;
         switch (t->nc) {
-        case 1: { ProfScope ps_("k_direct", st); k_direct<1><<<(nth + 127) / 128, 128, 0, st>>>(sd, t->nl, t->ldir, t->lpos, t->lint, t->C, t->D, t->flags); } break;
-        case 4: { ProfScope ps_("k_direct", st); k_direct<4><<<(nth + 127) / 128, 128, 0, st>>>(sd, t->nl, t->ldir, t->lpos, t->lint, t->C, t->D, t->flags); } break;
-        case 9: { ProfScope ps_("k_direct", st); k_direct<9><<<(nth + 127) / 128, 128, 0, st>>>(sd, t->nl, t->ldir, t->lpos, t->lint, t->C, t->D, t->flags); } break;
-        default: { ProfScope ps_("k_direct", st); k_direct<16><<<(nth + 127) / 128, 128, 0, st>>>(sd, t->nl, t->ldir, t->lpos, t->lint, t->C, t->D, t->flags); }
+        case 1: { ProfScope ps_("k_direct", st); k_direct<1><<<(nth + DIRECT_THREADS - 1) / DIRECT_THREADS, DIRECT_THREADS, 0, st>>>(sd, t->nl, t->ldir, t->lpos, t->lint, t->C, t->D, t->flags); } break;
+        case 4: { ProfScope ps_("k_direct", st); k_direct<4><<<(nth + DIRECT_THREADS - 1) / DIRECT_THREADS, DIRECT_THREADS, 0, st>>>(sd, t->nl, t->ldir, t->lpos, t->lint, t->C, t->D, t->flags); } break;
+        case 9: { ProfScope ps_("k_direct", st); k_direct<9><<<(nth + DIRECT_THREADS - 1) / DIRECT_THREADS, DIRECT_THREADS, 0, st>>>(sd, t->nl, t->ldir, t->lpos, t->lint, t->C, t->D, t->flags); } break;
+        default: { ProfScope ps_("k_direct", st); k_direct<16><<<(nth + DIRECT_THREADS - 1) / DIRECT_THREADS, DIRECT_THREADS, 0, st>>>(sd, t->nl, t->ldir, t->lpos, t->lint, t->C, t->D, t->flags); }
         }
         RGS_LAUNCH("direct");
     } else {
@@ -282,6 +245,9 @@ rgs_status rgs_trace_impl(rgs_transport *t, const rgs_lights *L, const rgs_trace
     int pa = 0;
     for (int c = RGS_TRACE_PATCH_A; c >= 1 && !pa; c >>= 1)
         if (t->na % c == 0 && 32 % c == 0 && t->nbs % (32 / c) == 0) pa = c;
+    const int n_patches = (int)(n_rays / 32);
+    WarpLists warps{st};
+    if ((r = warps.get((const void *)k_trace_hemi, HEMI_THREADS, n_patches)) != RGS_OK) return r;
     for (int attempt = 0; attempt < 2; ++attempt) {
         if (want > t->cap_slots) {
             if ((r = dev_alloc(&t->rec_ja, (size_t)want, &t->device_bytes)) != RGS_OK) return r;
@@ -291,8 +257,8 @@ rgs_status rgs_trace_impl(rgs_transport *t, const rgs_lights *L, const rgs_trace
         RGS_CUDA(cudaMemsetAsync(t->flags, 0, sizeof(int) * FLAG_COUNT, st));
         RGS_CUDA(cudaMemsetAsync(t->src_cnt, 0, sizeof(int) * n, st));
         RaysDev rd = t->rays();
-        const int TB = 128;
-        { ProfScope ps_("k_trace_hemi", st); k_trace_hemi<<<(unsigned)((n_rays + TB - 1) / TB), TB, 0, st>>>(sd, rd, (int)n_rays, t->cap_slots, t->counter, t->rec_ja, t->off, t->cnt, t->dir, t->src_cnt, t->flags, pa); }
+        RGS_CUDA(cudaMemsetAsync(warps.work, 0, sizeof(unsigned), st));
+        { ProfScope ps_("k_trace_hemi", st); k_trace_hemi<<<warps.blocks, HEMI_THREADS, 0, st>>>(sd, rd, n_patches, t->cap_slots, t->counter, warps.work, t->rec_ja, t->off, t->cnt, t->dir, t->src_cnt, t->flags, pa, warps.lists); }
         RGS_LAUNCH("trace_hemi");
         unsigned long long used = 0;
         int flags[FLAG_COUNT];
