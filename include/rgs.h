@@ -491,7 +491,8 @@ rgs_status rgs_mc_groups(rgs_transport *t, int32_t groups, int32_t *assign, void
  * once no unshot radiance is left the remaining shots do nothing.  The remaining problem
  * B^r = dB + K B^r is again the full transport, so B = Bhat + B^r - dB exactly: running
  * rgs_mc_solve with S_in = dB and combining gives the paper's hybrid solver.  Bhat_out,
- * dB_out: device [N][nc][C].  Three launches per shot.  Errors: RGS_ERR_ARG (NULL t or
+ * dB_out: device [N][nc][C].  Few receivers per shot: one launch for many shots, else two
+ * launches per shot.  Errors: RGS_ERR_ARG (NULL t or
  * output, shots < 0, a hemisphere transport), RGS_ERR_STATE, RGS_ERR_OOM, RGS_ERR_CUDA. */
 rgs_status rgs_prog_refine(rgs_transport *t, const float *E, int32_t shots, float *Bhat_out, float *dB_out,
                            void *stream);

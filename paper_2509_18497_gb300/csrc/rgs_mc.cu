@@ -24,6 +24,8 @@
 // receiver selection, 1000 + k the k-th candidate, draw q + 2^30 for the group stage -- so a
 // draw is reproducible from its key alone.  K-means (Lloyd's iterations on centre and normal,
 // FP64) runs once per (transport, group count) and is cached.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <vector>
 
@@ -501,104 +503,335 @@ __global__ void k_mc_visits(int n, const int *__restrict__ uid, const double *__
 // caller index) and sends it to every receiver that has it as a source:
 // dB_a += K_a,best dB_best, Bhat_a += the same, then dB_best = 0.
 constexpr int PR_T = 256;
+constexpr int PR_FIRE_BLOCKS = 608;              // 4 blocks of 8 warps per SM
+constexpr int SHOOT_LAUNCH = 4096;                // shots per launch of the cluster form
+constexpr size_t SHOOT_MAX_SMEM = 160 * 1024;     // a row and a block's share of the luminances, cluster form
+constexpr long long SHOOT_CLUSTER_ROWS = 160000;  // see prog_refine_nc
+// A luminance is a non-negative double, held as its bits: those order like the value, and
+// GB300's FP64 units (2 lanes per clock and SM) took most of a shot when the sums and the
+// search ran on them.
 struct LumIdx {
-    double v;
-    int idx; // caller index (n: none)
+    unsigned long long v;
+    int uid, i; // caller and internal index
 };
-__device__ __forceinline__ LumIdx lum_better(LumIdx a, LumIdx b) {
-    return (b.v > a.v || (b.v == a.v && b.idx < a.idx)) ? b : a;
-}
+#define LUM_NONE (LumIdx{0ull, 0x7fffffff, -1})
+// the brightest of a warp (ties: the lower caller index), in every lane
 __device__ __forceinline__ LumIdx lum_warp(LumIdx x) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        LumIdx y;
-        y.v = __shfl_xor_sync(0xffffffffu, x.v, o);
-        y.idx = __shfl_xor_sync(0xffffffffu, x.idx, o);
-        x = lum_better(x, y);
-    }
-    return x;
+    const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(x.v >> 32));
+    bool in = (unsigned)(x.v >> 32) == hi;
+    const unsigned lo = __reduce_max_sync(0xffffffffu, in ? (unsigned)x.v : 0u);
+    in = in && (unsigned)x.v == lo;
+    const int u = __reduce_min_sync(0xffffffffu, in ? x.uid : 0x7fffffff);
+    in = in && x.uid == u;
+    LumIdx y;
+    y.v = (unsigned long long)hi << 32 | lo;
+    y.uid = u;
+    y.i = __reduce_max_sync(0xffffffffu, in ? x.i : -1);
+    return y;
 }
-__device__ __forceinline__ LumIdx lum_block(LumIdx x, LumIdx *sh) {
+__device__ __forceinline__ LumIdx lum_better(LumIdx a, LumIdx b) {
+    return (b.v > a.v || (b.v == a.v && b.uid < a.uid)) ? b : a;
+}
+// (valid in warp 0; T: the block's threads)
+template <int T> __device__ __forceinline__ LumIdx lum_block(LumIdx x, LumIdx *sh) {
     x = lum_warp(x);
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = x;
     __syncthreads();
-    if (threadIdx.x < 32) {
-        x = threadIdx.x < PR_T / 32 ? sh[threadIdx.x] : LumIdx{0.0, 0x7fffffff};
-        x = lum_warp(x);
-    }
-    return x; // valid in thread 0
+    if (threadIdx.x < 32) x = lum_warp(threadIdx.x < T / 32 ? sh[threadIdx.x] : LUM_NONE);
+    return x;
 }
-// per-block brightest unshot surfel (luminance > 0 only)
-__global__ void __launch_bounds__(PR_T) k_pr_argmax(int n, int C, int NC, const int *__restrict__ uid,
-                                                   const float *__restrict__ dB, LumIdx *part) {
-    __shared__ LumIdx sh[PR_T / 32];
-    LumIdx best{0.0, 0x7fffffff};
-    const int i = blockIdx.x * PR_T + threadIdx.x;
-    if (i < n) {
-        double l = 0.0;
-        const float *x = dB + (size_t)i * C * NC;
-        for (int e = 0; e < C * NC; ++e) l += (double)lum_w(e / NC) * fabs((double)x[e]);
-        if (l > 0.0) best = LumIdx{l, uid[i]};
-    }
-    best = lum_block(best, sh);
-    if (threadIdx.x == 0) part[blockIdx.x] = best;
+
+// The luminances are kept beside dB: a shot changes the rows of its receivers, whose warps have
+// the new values in hand, so the search for the next shot reads 8 bytes per surfel instead of
+// a row.  The sum of lum(c) |x| over a row is formed in whole numbers, at least as exact as adding
+// in FP64: a column's 24-bit significands, aligned to its largest exponent with 8 bits below,
+// times its weight in units of 2^-27; the columns aligned to the row's largest exponent in 128
+// bits.  It is handed on as the bits of the double it truncates to.
+struct LumSum {
+    unsigned __int128 sum = 0; // in units of 2^(top - 150 - 8 - 27 - LUM_BELOW)
+    int top = 0;
+    unsigned bad = 0; // 1: an infinity, 2: a NaN
+};
+constexpr int LUM_BELOW = 40; // 24 + 4 + 8 + 27 bits of a column, 40 below, 15 for the count of columns
+__device__ __forceinline__ void lum_align(LumSum &s, int top) {
+    const int d = top - s.top;
+    s.sum = d > 127 ? 0 : s.sum >> d;
+    s.top = top;
 }
-// the shot: the brightest surfel (internal index to *shot_i, -1 if nothing is left), its
-// unshot radiance copied to shot and cleared in dB
-__global__ void __launch_bounds__(PR_T) k_pr_pick(int nparts, int R, const int *__restrict__ inv,
-                                                 const LumIdx *__restrict__ part, float *dB, float *shot, int *shot_i) {
-    __shared__ LumIdx sh[PR_T / 32];
-    __shared__ int sel;
-    LumIdx best{0.0, 0x7fffffff};
-    for (int b = threadIdx.x; b < nparts; b += PR_T) best = lum_better(best, part[b]);
-    best = lum_block(best, sh);
-    if (threadIdx.x == 0) {
-        sel = best.v > 0.0 ? inv[best.idx] : -1;
-        *shot_i = sel;
+// adds column c of a row
+template <int NC> __device__ __forceinline__ void lum_column(LumSum &s, const float (&x)[NC], int c) {
+    int ex[NC], top = 0;
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+        const unsigned b = __float_as_uint(x[k]) & 0x7fffffffu;
+        if (b >= 0x7f800000u) s.bad |= b > 0x7f800000u ? 2u : 1u;
+        ex[k] = max((int)(b >> 23), 1);
+        top = max(top, ex[k]);
     }
-    __syncthreads();
-    if (sel < 0) return;
-    for (int e = threadIdx.x; e < R; e += PR_T) {
-        shot[e] = dB[(size_t)sel * R + e];
-        dB[(size_t)sel * R + e] = 0.f;
+    unsigned long long t = 0ull; // 24 + 8 + 4 bits
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+        const unsigned b = __float_as_uint(x[k]) & 0x7fffffffu;
+        const unsigned m = (b & 0x7fffffu) | (b >= 0x800000u ? 0x800000u : 0u);
+        const int d = top - ex[k];
+        t += d > 31 ? 0u : (m << 8) >> d;
+    }
+    const unsigned w27 = (unsigned)(lum_w(c) * 134217728.f); // (exact)
+    const unsigned __int128 p = (unsigned __int128)(t * w27) << LUM_BELOW; // 63 bits before the shift
+    if (top > s.top) lum_align(s, top);
+    const int d = s.top - top;
+    if (d <= 127) s.sum += p >> d;
+}
+// the row's luminance from the sums of its m lanes base .. base + m - 1 (the whole warp calls)
+__device__ __forceinline__ unsigned long long lum_bits(const LumSum &s, int base, int m) {
+    LumSum t;
+    for (int q = 0; q < m; ++q) {
+        const int src = min(base + q, 31);
+        LumSum x;
+        x.top = __shfl_sync(0xffffffffu, s.top, src);
+        x.bad = __shfl_sync(0xffffffffu, s.bad, src);
+        const unsigned long long lo = __shfl_sync(0xffffffffu, (unsigned long long)s.sum, src);
+        const unsigned long long hi = __shfl_sync(0xffffffffu, (unsigned long long)(s.sum >> 64), src);
+        x.sum = (unsigned __int128)hi << 64 | lo;
+        const int top = max(t.top, x.top);
+        lum_align(t, top);
+        lum_align(x, top);
+        t.sum += x.sum;
+        t.bad |= x.bad;
+    }
+    if (t.bad) return t.bad & 2u ? 0ull : 0x7ff0000000000000ull; // a NaN is never the brightest
+    if (!t.sum) return 0ull;
+    const unsigned long long hi = (unsigned long long)(t.sum >> 64);
+    const int z = hi ? __clzll((long long)hi) : 64 + __clzll((long long)(unsigned long long)t.sum);
+    const int e = 1023 + (127 - z) + t.top - 150 - 8 - 27 - LUM_BELOW; // > 0: floats are far above FP64's least
+    const unsigned long long lead = (unsigned long long)((t.sum << z) >> 64);
+    return (unsigned long long)e << 52 | (lead << 1) >> 12;
+}
+// column c of a row, past the L1 (other SMs update the rows in other shots)
+template <int NC> __device__ __forceinline__ void ldcg_col(const float *p, float (&v)[NC]) {
+    if constexpr (NC % 4 == 0) {
+#pragma unroll
+        for (int q = 0; q < NC / 4; ++q) {
+            const float4 f = __ldcg(reinterpret_cast<const float4 *>(p) + q);
+            v[4 * q] = f.x;
+            v[4 * q + 1] = f.y;
+            v[4 * q + 2] = f.z;
+            v[4 * q + 3] = f.w;
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < NC; ++k) v[k] = __ldcg(p + k);
     }
 }
-// a warp per receiver of the shot's source: dB_a += K_a,j shot, Bhat_a += the same
+template <int NC> __device__ __forceinline__ void stcg_col(float *p, const float (&v)[NC]) {
+    if constexpr (NC % 4 == 0) {
+#pragma unroll
+        for (int q = 0; q < NC / 4; ++q)
+            __stcg(reinterpret_cast<float4 *>(p) + q, make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]));
+    } else {
+#pragma unroll
+        for (int k = 0; k < NC; ++k) __stcg(p + k, v[k]);
+    }
+}
+// Rows go to the lanes of a warp column by column: 32 / C whole rows of up to 32 columns, or one
+// row 32 columns at a time.
+__device__ __forceinline__ int rows_per_warp(int C) { return C <= 32 ? 32 / C : 1; }
+
 template <int NC>
-__global__ void __launch_bounds__(PR_T) k_pr_scatter(SceneDev sc, int C, const long long *__restrict__ src_off,
-                                                    const int2 *__restrict__ tr, const int *__restrict__ shot_i,
-                                                    const float *__restrict__ shot, float *dB, float *Bhat) {
-    const int j = *shot_i;
-    if (j < 0) return;
-    const long long e0 = src_off[j], e1 = src_off[j + 1];
-    const int lane = threadIdx.x & 31;
-    const long long warps = (long long)gridDim.x * (PR_T / 32);
-    const float3 pj = f3(sc.P[j]);
-    for (long long e = e0 + blockIdx.x * (PR_T / 32) + (threadIdx.x >> 5); e < e1; e += warps) {
-        const int2 iv = tr[e];
-        const int a = iv.x;
+__global__ void __launch_bounds__(PR_T) k_pr_lum(int n, int C, const float *__restrict__ dB, unsigned long long *lum) {
+    const int rows = rows_per_warp(C), m = min(C, 32), lane = threadIdx.x & 31;
+    const int i = (int)((blockIdx.x * (size_t)PR_T + threadIdx.x) >> 5) * rows + lane / m;
+    const bool live = lane < rows * m && i < n;
+    LumSum s;
+    for (int c = lane % m; live && c < C; c += 32) {
+        float x[NC];
+        ldcg_col<NC>(dB + ((size_t)i * C + c) * NC, x);
+        lum_column<NC>(s, x, c);
+    }
+    const unsigned long long v = lum_bits(s, lane / m * m, m);
+    if (live && lane % m == 0) lum[i] = v;
+}
+// rows_per_warp(C) receivers of the shot (entries e, e + 1, .. below e1 of its source's
+// transposed list) by a warp, a lane per receiver and column: dB_a += K_a,j shot, Bhat_a += the
+// same; put(a, luminance) by one lane of each.
+template <int NC, class Put>
+__device__ __forceinline__ void shoot_entries(const SceneDev &sc, int C, const int2 *__restrict__ tr, long long e, long long e1,
+                                              float3 pj, const float *shot, float *dB, float *Bhat, Put &&put) {
+    const int rows = rows_per_warp(C), m = min(C, 32), lane = threadIdx.x & 31;
+    e += lane / m;
+    const bool live = lane < rows * m && e < e1;
+    LumSum s;
+    int a = 0;
+    if (live) {
+        const int2 iv = __ldg(&tr[e]);
+        a = iv.x;
         const float V = __int_as_float(iv.y);
-        const float3 pa = f3(sc.P[a]), na = f3(sc.N4[a]);
-        float3 d = make_float3(pj.x - pa.x, pj.y - pa.y, pj.z - pa.z);
+        const float4 Pa = __ldg(&sc.P[a]), Na = __ldg(&sc.N4[a]);
+        float3 d = make_float3(pj.x - Pa.x, pj.y - Pa.y, pj.z - Pa.z);
         d = (1.f / sqrtf(dot3(d, d))) * d;
-        float Yo[NC], Yi[NC];
-        sh_eval<NC>(neg3(d), Yo);
-        sh_eval<NC>(reflect_n(na, d), Yi);
-        const float oa = alpha_center(sc, a);
-        for (int c = lane; c < C; c += 32) {
+        const float oa = alpha_of(sc, Pa.w, 1.f);
+        for (int c = lane % m; c < C; c += 32) {
+            const size_t row = ((size_t)a * C + c) * NC;
+            float x[NC], y[NC], w[NC];
+            ldcg_col<NC>(dB + row, x);
+            ldcg_col<NC>(Bhat + row, y);
+            sh_eval<NC>(neg3(d), w);
             float sv = 0.f;
 #pragma unroll
-            for (int k = 0; k < NC; ++k) sv += Yo[k] * shot[c * NC + k];
-            const float x = V * sv;
+            for (int k = 0; k < NC; ++k) sv += w[k] * shot[c * NC + k];
+            sv *= V;
+            sh_eval<NC>(reflect_n(f3(Na), d), w);
 #pragma unroll
             for (int k = 0; k < NC; ++k) {
-                const size_t idx = ((size_t)a * C + c) * NC + k;
-                const float v = oa * sc.cl[(size_t)a * 12 + band_of(k) * 3 + (c % 3)] * Yi[k] * x;
-                dB[idx] += v;
-                Bhat[idx] += v;
+                const float v = oa * __ldg(&sc.cl[(size_t)a * 12 + band_of(k) * 3 + (c % 3)]) * w[k] * sv;
+                x[k] += v;
+                y[k] += v;
             }
+            stcg_col<NC>(dB + row, x);
+            stcg_col<NC>(Bhat + row, y);
+            lum_column<NC>(s, x, c);
         }
     }
+    const unsigned long long v = lum_bits(s, lane / m * m, m);
+    if (live && lane % m == 0) put(a, v);
+}
+
+// Many shots by one cluster of up to 16 blocks: a shot is two cluster barriers (the pick; the
+// rows it changed) and no launch.  The luminances live in the blocks' shared memory (surfel i
+// with block i mod nb), where the receivers' warps put the new ones.
+constexpr int SHOOT_T = 512; // (measured: 256 and 1024 threads are slower by 3-24 %)
+template <int NC>
+__global__ void __launch_bounds__(SHOOT_T, 1) k_pr_shoot(SceneDev sc, int n, int C, const int *__restrict__ uid,
+                                                        const long long *__restrict__ src_off,
+                                                        const int2 *__restrict__ tr, int shots, unsigned long long *lum,
+                                                        float *dB, float *Bhat) {
+    extern __shared__ __align__(16) unsigned char shoot_smem[];
+    __shared__ LumIdx sh[SHOOT_T / 32], slots[16];
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank(), nb = (int)cluster.num_blocks();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int R = C * NC;
+    unsigned long long *mine = reinterpret_cast<unsigned long long *>(shoot_smem); // [ceil(n / nb)]
+    float *shot = reinterpret_cast<float *>(mine + (n + nb - 1) / nb);             // the shot's row
+    for (int i = rank + nb * (int)threadIdx.x; i < n; i += nb * SHOOT_T) mine[i / nb] = lum[i];
+    cluster.sync();
+    const int first = rank + nb * (int)threadIdx.x;
+    const int uid0 = first < n ? uid[first] : 0x7fffffff;
+    int prev = -1;
+    // the last shot's row is cleared by the block that searches it, once every block has read it
+    auto clear = [&]() {
+        if (prev < 0 || prev % nb != rank) return;
+        for (int e = threadIdx.x; e < R; e += SHOOT_T) __stcg(&dB[(size_t)prev * R + e], 0.f);
+        if (threadIdx.x == 0) mine[prev / nb] = 0ull;
+    };
+    for (int m = 0; m < shots; ++m) {
+        clear();
+        __syncthreads();
+        LumIdx best = LUM_NONE;
+        if (first < n && mine[threadIdx.x]) best = LumIdx{mine[threadIdx.x], uid0, first};
+        for (int i = first + nb * SHOOT_T; i < n; i += nb * SHOOT_T)
+            if (mine[i / nb]) best = lum_better(best, LumIdx{mine[i / nb], __ldg(&uid[i]), i});
+        best = lum_block<SHOOT_T>(best, sh);
+        if (threadIdx.x < (unsigned)nb) cluster.map_shared_rank(slots, threadIdx.x)[rank] = best;
+        cluster.sync();
+        const int j = prev = lum_warp(lane < nb ? slots[lane] : LUM_NONE).i;
+        if (j < 0) break; // nothing left to shoot (the same in every block)
+        const long long e0 = src_off[j], e1 = src_off[j + 1];
+        const float3 pj = f3(sc.P[j]);
+        for (int e = threadIdx.x; e < R; e += SHOOT_T) shot[e] = __ldcg(&dB[(size_t)j * R + e]);
+        __syncthreads();
+        const int rows = rows_per_warp(C);
+        for (long long e = e0 + rows * (rank + nb * warp); e < e1; e += rows * nb * (SHOOT_T / 32))
+            shoot_entries<NC>(sc, C, tr, e, e1, pj, shot, dB, Bhat, [&](int a, unsigned long long v) {
+                cluster.map_shared_rank(mine, a % nb)[a / nb] = v;
+            });
+        cluster.sync();
+    }
+    clear();
+    cluster.sync();
+    for (int i = rank + nb * (int)threadIdx.x; i < n; i += nb * SHOOT_T) lum[i] = mine[i / nb]; // for the next launch
+}
+
+// The same shot by shot over the whole chip, two launches each, where one cluster's SMs would
+// take longer than the launches: the search (which first clears the last shot's row) ...
+__global__ void __launch_bounds__(PR_T) k_pr_argmax(int n, int R, const int *__restrict__ uid, const int *__restrict__ shot_i,
+                                                   unsigned long long *lum, float *dB, LumIdx *part) {
+    __shared__ LumIdx sh[PR_T / 32];
+    const int prev = *shot_i, chunk = blockIdx.x * PR_T;
+    if (prev >= chunk && prev < chunk + PR_T) {
+        for (int e = threadIdx.x; e < R; e += PR_T) dB[(size_t)prev * R + e] = 0.f;
+        if (threadIdx.x == 0) lum[prev] = 0ull;
+    }
+    __syncthreads();
+    const int i = chunk + threadIdx.x;
+    const LumIdx best = lum_block<PR_T>(i < n && lum[i] ? LumIdx{lum[i], uid[i], i} : LUM_NONE, sh);
+    if (threadIdx.x == 0) part[blockIdx.x] = best;
+}
+// ... and the shot itself, every block finding the pick from the search's parts
+template <int NC>
+__global__ void __launch_bounds__(PR_T) k_pr_fire(SceneDev sc, int nparts, int C, const LumIdx *__restrict__ part,
+                                                 const long long *__restrict__ src_off, const int2 *__restrict__ tr,
+                                                 int *shot_i, unsigned long long *lum, float *dB, float *Bhat) {
+    __shared__ LumIdx sh[PR_T / 32];
+    __shared__ int sel;
+    LumIdx best = LUM_NONE;
+    for (int b = threadIdx.x; b < nparts; b += PR_T) best = lum_better(best, part[b]);
+    best = lum_block<PR_T>(best, sh);
+    if (threadIdx.x == 0) {
+        sel = best.i;
+        if (blockIdx.x == 0) *shot_i = best.i;
+    }
+    __syncthreads();
+    const int j = sel;
+    if (j < 0) return;
+    const float3 pj = f3(sc.P[j]);
+    const long long e1 = src_off[j + 1];
+    const int rows = rows_per_warp(C);
+    const long long step = (long long)rows * gridDim.x * (PR_T / 32);
+    for (long long e = src_off[j] + rows * (blockIdx.x * (PR_T / 32) + (threadIdx.x >> 5)); e < e1; e += step)
+        shoot_entries<NC>(sc, C, tr, e, e1, pj, dB + (size_t)j * C * NC, dB, Bhat,
+                          [&](int a, unsigned long long v) { lum[a] = v; });
+}
+
+// `shots` shots by one cluster; *done = false where the device grants no cluster of this shape
+template <int NC>
+rgs_status cluster_shots(rgs_transport *t, const int2 *tr, int shots, unsigned long long *lum, float *dB, float *Bhat,
+                         bool *done,
+                         cudaStream_t st) {
+    *done = false;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    cfg.blockDim = dim3(SHOOT_T);
+    cfg.dynamicSmemBytes = sizeof(float) * (size_t)t->C * NC + 8 * (((size_t)t->n + 7) / 8);
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    const void *fn = (const void *)k_pr_shoot<NC>;
+    if (cfg.dynamicSmemBytes > SHOOT_MAX_SMEM) return RGS_OK;
+    RGS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes));
+    RGS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    int fit = 0;
+    unsigned blocks = 16;
+    for (; blocks >= 8 && fit < 1; blocks /= 2) { // 16 is the opt-in size, 8 the portable one
+        cfg.gridDim = dim3(blocks);
+        attr[0].val.clusterDim.x = blocks;
+        if (cudaOccupancyMaxActiveClusters(&fit, fn, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            fit = 0;
+        }
+    }
+    if (fit < 1) return RGS_OK;
+    const SceneDev sd = t->sc->dev();
+    for (int m = 0; m < shots; m += SHOOT_LAUNCH) {
+        ProfScope ps_("k_pr_shoot", st);
+        RGS_CUDA(cudaLaunchKernelEx(&cfg, k_pr_shoot<NC>, sd, t->n, t->C, (const int *)t->sc->uid,
+                                    (const long long *)t->src_off, tr, std::min(SHOOT_LAUNCH, shots - m), lum, dB, Bhat));
+    }
+    *done = true;
+    return RGS_OK;
 }
 
 inline unsigned nblk(size_t m, int b) { return (unsigned)((m + b - 1) / b); }
@@ -853,11 +1086,12 @@ rgs_status prog_refine_nc(rgs_transport *t, const float *E, int shots, float *Bh
     const size_t M = t->arr();
     const int nparts = (int)nblk(n, PR_T);
     Scratch s{st};
-    float *dB, *Bhat, *shot;
+    float *dB, *Bhat;
+    unsigned long long *lum;
     LumIdx *part;
     int *shot_i;
     int2 *tr;
-    if ((r = s.get(&dB, M)) != RGS_OK || (r = s.get(&Bhat, M)) != RGS_OK || (r = s.get(&shot, (size_t)R)) != RGS_OK ||
+    if ((r = s.get(&dB, M)) != RGS_OK || (r = s.get(&Bhat, M)) != RGS_OK || (r = s.get(&lum, (size_t)n)) != RGS_OK ||
         (r = s.get(&part, (size_t)nparts)) != RGS_OK || (r = s.get(&shot_i, 1)) != RGS_OK ||
         (r = s.get(&tr, (size_t)std::max(t->n_pairs, 1ll))) != RGS_OK)
         return r;
@@ -865,14 +1099,29 @@ rgs_status prog_refine_nc(rgs_transport *t, const float *E, int shots, float *Bh
     { ProfScope ps_("k_mc_make_S", st); k_mc_make_S<NC><<<nblk(M, 256), 256, 0, st>>>(n, C, t->sc->uid, E, t->D, Bhat); }
     RGS_LAUNCH("shooting source");
     RGS_CUDA(cudaMemcpyAsync(dB, Bhat, sizeof(float) * M, cudaMemcpyDeviceToDevice, st));
-    const SceneDev sd = t->sc->dev();
-    for (int m = 0; m < shots; ++m) {
-        { ProfScope ps_("k_pr_argmax", st); k_pr_argmax<<<nparts, PR_T, 0, st>>>(n, C, NC, t->sc->uid, dB, part); }
-        RGS_LAUNCH("shooting argmax");
-        { ProfScope ps_("k_pr_pick", st); k_pr_pick<<<1, PR_T, 0, st>>>(nparts, R, t->sc->inv, part, dB, shot, shot_i); }
-        RGS_LAUNCH("shooting pick");
-        { ProfScope ps_("k_pr_scatter", st); k_pr_scatter<NC><<<256, PR_T, 0, st>>>(sd, C, t->src_off, tr, shot_i, shot, dB, Bhat); }
-        RGS_LAUNCH("shooting scatter");
+    if (shots > 0) {
+        { ProfScope ps_("k_pr_lum", st); k_pr_lum<NC><<<nblk(nblk(n, C <= 32 ? 32 / C : 1) * 32ull, PR_T), PR_T, 0, st>>>(n, C, dB, lum); }
+        RGS_LAUNCH("shooting luminances");
+        bool done = false;
+        // The values a shot updates (its receivers' rows) decide the form.  Measured, us per shot,
+        // cluster / launches (three launches over FP64 luminances before): 2,500 surfels x 27
+        // values a row (33 k values) 6.3 / 12.4 (22.9), 5,000 x 48 (119 k) 9.1 / 12.0 (32.4),
+        // 10,000 x 48 (237 k) 16.2 / 12.1 (38.8), 2,500 x 384 (470 k) 21.5 / 13.9 (78.9).
+        if ((long long)(t->n_pairs / n) * R <= SHOOT_CLUSTER_ROWS &&
+            (r = cluster_shots<NC>(t, tr, shots, lum, dB, Bhat, &done, st)) != RGS_OK)
+            return r;
+        if (!done) {
+            const SceneDev sd = t->sc->dev();
+            RGS_CUDA(cudaMemsetAsync(shot_i, 0xff, sizeof(int), st)); // -1
+            for (int m = 0; m < shots; ++m) {
+                { ProfScope ps_("k_pr_argmax", st); k_pr_argmax<<<nparts, PR_T, 0, st>>>(n, R, t->sc->uid, shot_i, lum, dB, part); }
+                RGS_LAUNCH("shooting search");
+                { ProfScope ps_("k_pr_fire", st); k_pr_fire<NC><<<PR_FIRE_BLOCKS, PR_T, 0, st>>>(sd, nparts, C, part, t->src_off, tr, shot_i, lum, dB, Bhat); }
+                RGS_LAUNCH("shooting shot");
+            }
+            { ProfScope ps_("k_pr_argmax", st); k_pr_argmax<<<nparts, PR_T, 0, st>>>(n, R, t->sc->uid, shot_i, lum, dB, part); } // clears the last row
+            RGS_LAUNCH("shooting end");
+        }
     }
     { ProfScope ps_("k_mc_to_user", st); k_mc_to_user<NC><<<nblk(M, 256), 256, 0, st>>>(n, C, t->sc->uid, Bhat, Bhat_out); }
     { ProfScope ps_("k_mc_to_user", st); k_mc_to_user<NC><<<nblk(M, 256), 256, 0, st>>>(n, C, t->sc->uid, dB, dB_out); }
