@@ -29,18 +29,18 @@ template <int NC> __device__ __forceinline__ void load_col(const float *__restri
         for (int k = 0; k < NC; ++k) v[k] = __ldg(p + k);
     }
 }
+// (BF16 rows of 9 or 16 coefficients are padded to 32 bytes: one request a lane.  As two
+// 16-byte requests at a 32-byte stride a warp's kilobyte took the L1 twice the wavefronts.)
 template <int NC> __device__ __forceinline__ void load_col(const __nv_bfloat16 *__restrict__ p, float *v) {
-    if constexpr (NC >= 9) { // padded to 16
+    if constexpr (NC >= 9) {
+        float4 a, b;
+        ld_rec32(p, a, b);
+        const float f[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const uint4 w = __ldg(reinterpret_cast<const uint4 *>(p) + q);
-            const unsigned u[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-            for (int m = 0; m < 4; ++m) {
-                const int k0 = 8 * q + 2 * m;
-                if (k0 < NC) v[k0] = __uint_as_float(u[m] << 16);
-                if (k0 + 1 < NC) v[k0 + 1] = __uint_as_float(u[m] & 0xffff0000u);
-            }
+        for (int m = 0; m < 8; ++m) {
+            const unsigned u = __float_as_uint(f[m]);
+            if (2 * m < NC) v[2 * m] = __uint_as_float(u << 16);
+            if (2 * m + 1 < NC) v[2 * m + 1] = __uint_as_float(u & 0xffff0000u);
         }
     } else {
 #pragma unroll
@@ -52,54 +52,39 @@ template <int NC, class T> constexpr int row_stride() {
 }
 
 // Dot products of Y with the 32 columns of one FP32 source row tile (nc = 16: 64 B per
-// column, 2 KB per tile), read as four contiguous 512-B warp requests, a lane taking 16 B
-// (a quarter of one column).  Each lane forms its partial dot products with its quarter of
-// Y, and a reduce-scatter over the 4 lanes holding each column leaves lane l with the
-// whole dot product of tile column own(l).  A 64-B column row per lane at a 64-B stride
-// costs the L1 about twice the wavefronts for the same bytes (measured: the FP32 form of
-// the 300- and 1,536-column workloads 6 % and 25 % faster).  For BF16 rows (32 B per
-// column) the same scheme measured 3-7 % slower than a row per lane and is not used.
+// column, 2 KB per tile), read as two contiguous 1-KB warp requests, a lane taking 32 B (half
+// of one column).  Each lane forms its partial dot products with its half of Y, and one
+// exchange between the 2 lanes holding each column leaves lane l with the whole dot product
+// of tile column own(l).  A 64-B column row per lane at a 64-B stride costs the L1 about
+// twice the wavefronts for the same bytes.
 // Columns past the tile's `ncols` live ones read the last live column (their results are
 // not used).  All 32 lanes take part (the shuffles use the full mask).
 template <class T, int NC> struct TileDot;
 
 template <int NC> struct TileDot<float, NC> {
     static_assert(NC == 16, "FP32 tiles of 16 coefficients per column");
-    static constexpr int KPL = 4;
-    __device__ static int own(int lane) {
-        const int g = lane & 3;
-        return 8 * (2 * (g & 1) + (g >> 1)) + (lane >> 2);
-    }
+    static constexpr int KPL = 8;
+    __device__ static int own(int lane) { return 16 * (lane & 1) + (lane >> 1); }
     __device__ static void pick(const float *Y, int lane, float (&y)[KPL]) {
-        const int g = lane & 3;
 #pragma unroll
-        for (int m = 0; m < KPL; ++m) {
-            float v = Y[m];
-            v = g == 1 ? Y[4 + m] : v;
-            v = g == 2 ? Y[8 + m] : v;
-            v = g == 3 ? Y[12 + m] : v;
-            y[m] = v;
-        }
+        for (int m = 0; m < KPL; ++m) y[m] = lane & 1 ? Y[8 + m] : Y[m];
     }
     // tile: the tile's first column in source row j; ncols: its live columns (1..32)
     __device__ static float dot(const float *__restrict__ tile, int ncols, int lane, const float (&y)[KPL]) {
-        const int g = lane & 3, a = lane >> 2;
-        float p[4];
+        const int g = lane & 1, a = lane >> 1;
+        float p[2];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int c = min(8 * q + a, ncols - 1);
-            const float4 f = __ldg(reinterpret_cast<const float4 *>(tile + c * 16) + g);
+        for (int q = 0; q < 2; ++q) {
+            const int c = min(16 * q + a, ncols - 1);
+            float4 f, h;
+            ld_rec32(tile + c * 16 + 8 * g, f, h);
             p[q] = y[0] * f.x + y[1] * f.y + y[2] * f.z + y[3] * f.w;
+            p[q] += y[4] * h.x + y[5] * h.y + y[6] * h.z + y[7] * h.w;
         }
-        const bool b0 = (g & 1) != 0, b1 = (g & 2) != 0;
-        const float r0 = __shfl_xor_sync(0xffffffffu, b0 ? p[0] : p[2], 1);
-        const float r1 = __shfl_xor_sync(0xffffffffu, b0 ? p[1] : p[3], 1);
-        const float s0 = (b0 ? p[2] : p[0]) + r0, s1 = (b0 ? p[3] : p[1]) + r1;
-        const float r = __shfl_xor_sync(0xffffffffu, b1 ? s0 : s1, 2);
-        return (b1 ? s1 : s0) + r;
+        const float r = __shfl_xor_sync(0xffffffffu, g ? p[0] : p[1], 1);
+        return (g ? p[1] : p[0]) + r;
     }
 };
-
 
 template <int NC, int CT, class SL>
 __device__ __forceinline__ void bounce_epilogue(const SceneDev &sc, int C, const float (&acc)[SL::KPL][CT], float w,

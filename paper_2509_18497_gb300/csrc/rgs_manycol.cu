@@ -135,7 +135,7 @@ __global__ void RGS_MC_LB k_opacity_g_mc(SceneDev sc, RaysDev rays, int C, int c
         }
     }
     const long long base = rays.off[r];
-    [[maybe_unused]] float ys[4]; // this lane's quarter of Y(-d) (TileDot)
+    [[maybe_unused]] float ys[8]; // this lane's half of Y(-d) (TileDot)
     if constexpr (COOP) TileDot<T, NC>::pick(Yo, lane, ys);
     for (int h = 0; h < cnt; ++h) {
         const int j = __ldg(&rays.rec_ja[base + h]).x;

@@ -87,9 +87,9 @@ __device__ __forceinline__ void shade_pixel(const int4 *hits, int n, float3 d, i
         return;
     }
     if constexpr (NC == 16) {
-        // 32-column tiles of each source row read as four contiguous 512-B warp requests, every
+        // 32-column tiles of each source row read as two contiguous 1-KB warp requests, every
         // lane ending with the dot product of one tile column (TileDot)
-        float ys[4];
+        float ys[8];
         TileDot<float, 16>::pick(Yo, lane, ys);
         const int own = TileDot<float, 16>::own(lane);
         for (int c0 = 0; c0 < C; c0 += 32) {
