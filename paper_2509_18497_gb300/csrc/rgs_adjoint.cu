@@ -71,40 +71,57 @@ __global__ void __launch_bounds__(32 * ROW_WARPS) k_pair_accum(int n, int C, con
     }
 }
 
-// Per ray r of receiver i (column tile col0..col0+2):
+// Per ray r of receiver i, for a tile of CT columns:
 //   y_r[c] = (pi/nd) o_i sum_k' c_{i,l(k'),ch} Y_k'(R_i d_r) v_i[c][k']
-// stored next to the ray's direction for the by-source gather.
-template <int NC>
+// in one record with the ray's direction for the by-source gather: 8 floats (d, 0, y[0..2], 0)
+// for 3 columns, 16 (d, 0, y[0..11]) for 12 (columns past C are zero).  With d and y in arrays of
+// their own each entry touched two cache lines, and at 3 columns a tile 48 columns took 16
+// passes: the gather held the L1 data pipe at 80 % of peak with lookups.  60,000 surfels, 128
+// rays, 48 columns, four bounces: the gather 71 -> 28.5 ms.
+template <int CT> constexpr int adj_rec() { return CT == 3 ? 8 : 16; }
+template <int NC, int CT>
 __global__ void __launch_bounds__(256) k_adj_ray(SceneDev sc, RaysDev rays, int C, int col0,
-                                                 const float *__restrict__ vin, float4 *dy) {
+                                                 const float *__restrict__ vin, float *__restrict__ rec) {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= sc.n * rays.nd) return;
     const int i = r / rays.nd;
     const float3 n = f3(sc.N4[i]);
     const float3 d = f3(rays.dir[r]);
-    float Yi[NC];
+    float Yi[NC], cy[NC]; // cy: c_{i,l(k),ch} Y_k of one channel
     sh_eval<NC>(reflect_n(n, d), Yi);
     const float oi = alpha_center(sc, i) * (3.14159265358979f / (float)rays.nd);
     const float *vi = vin + ((size_t)i * C + col0) * NC;
-    float y[3];
+    float y[CT];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const int ch = (col0 + c) % 3;
-        float s = 0.f;
+    for (int ch = 0; ch < 3; ++ch) {
 #pragma unroll
-        for (int k = 0; k < NC; ++k) s += __ldg(&sc.cl[(size_t)i * 12 + band_of(k) * 3 + ch]) * Yi[k] * __ldg(&vi[c * NC + k]);
-        y[c] = oi * s;
+        for (int k = 0; k < NC; ++k) cy[k] = __ldg(&sc.cl[(size_t)i * 12 + band_of(k) * 3 + ch]) * Yi[k];
+#pragma unroll
+        for (int c = ch; c < CT; c += 3) { // (col0 is a multiple of 3)
+            float s = 0.f;
+            if (CT == 3 || col0 + c < C) {
+#pragma unroll
+                for (int k = 0; k < NC; ++k) s += cy[k] * __ldg(&vi[c * NC + k]);
+            }
+            y[c] = oi * s;
+        }
     }
-    dy[r] = make_float4(y[0], y[1], y[2], 0.f);
+    float4 *out = reinterpret_cast<float4 *>(rec + (size_t)r * adj_rec<CT>());
+    out[0] = make_float4(d.x, d.y, d.z, 0.f);
+#pragma unroll
+    for (int q = 0; q < adj_rec<CT>() / 4 - 1; ++q)
+        out[q + 1] = make_float4(y[(4 * q) % CT], y[(4 * q + 1) % CT], y[(4 * q + 2) % CT],
+                                 4 * q + 3 < CT ? y[(4 * q + 3) % CT] : 0.f);
 }
 
 // (K^T v)_j[c][k] = sum_{entries e on j} a_e Y_k(-d_e) y_e[c]; one CTA per source j.
+// 3 columns: a thread per entry.
 template <int NC>
-__global__ void RGS_ADJ_LB k_adj_src(RaysDev rays, int C, int col0, const long long *__restrict__ src_off,
-                                                        const int2 *__restrict__ tr, const float4 *__restrict__ dy,
+__global__ void RGS_ADJ_LB k_adj_src(int C, int col0, const long long *__restrict__ src_off,
+                                                        const int2 *__restrict__ tr, const float *__restrict__ rec,
                                                         float *__restrict__ vout, float *__restrict__ u, int j0,
                                                         long long ebase) {
-    constexpr int CT = 3;
+    constexpr int CT = 3, RS = adj_rec<CT>();
     const int j = j0 + blockIdx.x; // sources j0 .. of this index part; its entries start at ebase
     float acc[NC][CT];
 #pragma unroll
@@ -115,8 +132,8 @@ __global__ void RGS_ADJ_LB k_adj_src(RaysDev rays, int C, int col0, const long l
     for (long long e = e0 + threadIdx.x; e < e1; e += ADJ_THREADS) {
         const int2 ent = __ldg(&tr[e]);
         const float a = __int_as_float(ent.y);
-        const float4 d4 = __ldg(&rays.dir[ent.x]);
-        const float4 y4 = __ldg(&dy[ent.x]);
+        float4 d4, y4;
+        ld_rec32(rec + (size_t)ent.x * RS, d4, y4);
         float Yo[NC];
         sh_eval<NC>(make_float3(-d4.x, -d4.y, -d4.z), Yo);
         const float y[3] = {a * y4.x, a * y4.y, a * y4.z};
@@ -141,6 +158,120 @@ __global__ void RGS_ADJ_LB k_adj_src(RaysDev rays, int C, int col0, const long l
         float v = 0.f;
         for (int q = 0; q < ADJ_THREADS / 32; ++q) v += red[q][e];
         const int k = e / CT, c = e - k * CT;
+        const size_t idx = ((size_t)j * C + col0 + c) * NC + k;
+        vout[idx] = v;
+        u[idx] += v;
+    }
+}
+
+// 12 columns: the entries' records are copied into shared memory 128 at a time (asynchronously,
+// the next batch while this one is used: their latency, not the arithmetic, is what bounds
+// the gather), a thread evaluates the SH of one entry, and G lanes per entry, each KPL
+// coefficients, multiply: 48 FMAs per 4 shared-memory reads.  60,000 surfels, 128 rays, 48
+// columns: 1.78 ms a launch (an entry per thread at 3 columns: 1.1 ms for a quarter of them).
+constexpr int ADJ_STRIDE = 20; // floats of a record in shared memory (16-byte rows without conflicts)
+template <int NC> struct AdjLanes {
+    static constexpr int G = NC >= 9 ? 4 : 1, KPL = (NC + G - 1) / G;
+};
+template <int NC> struct AdjTile {
+    __align__(16) float rec[2][ADJ_THREADS][ADJ_STRIDE];
+    __align__(16) float Y[ADJ_THREADS][ADJ_STRIDE]; // a Y(-d)
+    float a[2][ADJ_THREADS];
+};
+__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src));
+}
+template <int NC>
+__global__ void __launch_bounds__(ADJ_THREADS, 7) k_adj_src_tile(int C, int col0, const long long *__restrict__ src_off,
+                                                               const int2 *__restrict__ tr, const float *__restrict__ rec,
+                                                               float *__restrict__ vout, float *__restrict__ u, int j0,
+                                                               long long ebase) {
+    constexpr int CT = 12, RS = adj_rec<CT>(), G = AdjLanes<NC>::G, KPL = AdjLanes<NC>::KPL;
+    __shared__ AdjTile<NC> s;
+    const int j = j0 + blockIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, g = tid % G;
+    float acc[KPL][CT];
+#pragma unroll
+    for (int k = 0; k < KPL; ++k)
+#pragma unroll
+        for (int c = 0; c < CT; ++c) acc[k][c] = 0.f;
+    const long long e0 = src_off[j] - ebase, e1 = src_off[j + 1] - ebase;
+    const int batches = (int)((e1 - e0 + ADJ_THREADS - 1) / ADJ_THREADS);
+    auto entry = [&](int b) { // this thread's entry of batch b (ray -1: none)
+        const long long e = e0 + (long long)b * ADJ_THREADS + tid;
+        return e < e1 ? __ldg(&tr[e]) : make_int2(-1, 0);
+    };
+    auto fetch = [&](int st, int2 ent) { // four lanes copy a record
+        s.a[st][tid] = __int_as_float(ent.y);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int from = 8 * q + (lane >> 2), ray = __shfl_sync(0xffffffffu, ent.x, from);
+            if (ray >= 0)
+                cp_async16(&s.rec[st][(tid & ~31) + from][4 * (lane & 3)], rec + (size_t)ray * RS + 4 * (lane & 3));
+        }
+        asm volatile("cp.async.commit_group;");
+    };
+    int2 ent = entry(0);
+    if (batches > 0) fetch(0, ent);
+    ent = entry(1);
+    for (int b = 0; b < batches; ++b) {
+        const int st = b & 1;
+        if (b + 1 < batches) {
+            fetch(st ^ 1, ent);
+            ent = entry(b + 2);
+            asm volatile("cp.async.wait_group 1;");
+        } else {
+            asm volatile("cp.async.wait_group 0;");
+        }
+        __syncthreads();
+        const int m = (int)min((long long)ADJ_THREADS, e1 - e0 - (long long)b * ADJ_THREADS);
+        if (tid < m) {
+            const float4 d = *reinterpret_cast<const float4 *>(s.rec[st][tid]);
+            const float a = s.a[st][tid];
+            float Yo[NC];
+            sh_eval<NC>(make_float3(-d.x, -d.y, -d.z), Yo);
+#pragma unroll
+            for (int k = 0; k < G * KPL; ++k) s.Y[tid][k] = k < NC ? a * Yo[k < NC ? k : 0] : 0.f;
+        }
+        __syncthreads();
+#pragma unroll 2
+        for (int x = tid / G; x < m; x += ADJ_THREADS / G) {
+            float w[KPL], y[CT];
+#pragma unroll
+            for (int k = 0; k < KPL; ++k) w[k] = s.Y[x][KPL * g + k];
+#pragma unroll
+            for (int q = 0; q < CT / 4; ++q) {
+                const float4 f = *reinterpret_cast<const float4 *>(&s.rec[st][x][4 + 4 * q]);
+                y[4 * q] = f.x;
+                y[4 * q + 1] = f.y;
+                y[4 * q + 2] = f.z;
+                y[4 * q + 3] = f.w;
+            }
+#pragma unroll
+            for (int k = 0; k < KPL; ++k)
+#pragma unroll
+                for (int c = 0; c < CT; ++c) acc[k][c] += w[k] * y[c];
+        }
+        __syncthreads(); // the tables are rewritten
+    }
+    float *red = &s.rec[0][0][0]; // [warp][G KPL CT]
+    constexpr int OUT = G * KPL * CT;
+    static_assert(ADJ_THREADS / 32 * OUT <= 2 * ADJ_THREADS * ADJ_STRIDE, "the sums fit the records' place");
+#pragma unroll
+    for (int k = 0; k < KPL; ++k)
+#pragma unroll
+        for (int c = 0; c < CT; ++c) {
+            float v = acc[k][c];
+#pragma unroll
+            for (int off = 16; off >= G; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+            if (lane < G) red[(tid >> 5) * OUT + (KPL * lane + k) * CT + c] = v;
+        }
+    __syncthreads();
+    for (int e = tid; e < NC * CT; e += ADJ_THREADS) {
+        const int c = e / NC, k = e - c * NC;
+        if (col0 + c >= C) continue;
+        float v = 0.f;
+        for (int q = 0; q < ADJ_THREADS / 32; ++q) v += red[q * OUT + k * CT + c];
         const size_t idx = ((size_t)j * C + col0 + c) * NC + k;
         vout[idx] = v;
         u[idx] += v;
@@ -708,7 +839,6 @@ rgs_status run_adjoint(rgs_transport *t, const float *g, float *dE, float *dad, 
     const size_t A = t->arr();
     const size_t A16 = (size_t)n * C * bf16_stride<NC>();
     const bool bf16 = t->prec_last != RGS_FP32;
-    const bool mc = wide_adjoint(C);
     SceneDev sd = t->sc->dev();
     RaysDev rd = t->rays();
     const unsigned ga = (unsigned)((A + 255) / 256);
@@ -745,13 +875,16 @@ rgs_status run_adjoint(rgs_transport *t, const float *g, float *dE, float *dad, 
             if (j1 <= j0) continue;
             const long long eb = part_base[p];
             if (parts.size() > 2 && (q = build_index(t, j0, j1, eb, st)) != RGS_OK) return q;
-            if (mc) {
-                if ((q = mc_adjoint_bounce<NC>(t, sd, rd, vp(a - 1), vp(a), j0, j1, eb, st)) != RGS_OK) return q;
-                continue;
-            }
-            for (int col0 = 0; col0 < C; col0 += 3) {
-                { ProfScope ps_("k_adj_ray", st); k_adj_ray<NC><<<gr, 256, 0, st>>>(sd, rd, C, col0, vp(a - 1), t->dy); }
-                { ProfScope ps_("k_adj_src", st); k_adj_src<NC><<<j1 - j0, ADJ_THREADS, 0, st>>>(rd, C, col0, t->src_off, t->tr, t->dy, vp(a), t->u, j0, eb); }
+            for (int col0 = 0; col0 < C;) {
+                if (t->dy_cols == 12 && C - col0 > 3) {
+                    { ProfScope ps_("k_adj_ray", st); k_adj_ray<NC, 12><<<gr, 256, 0, st>>>(sd, rd, C, col0, vp(a - 1), t->dy); }
+                    { ProfScope ps_("k_adj_src_tile", st); k_adj_src_tile<NC><<<j1 - j0, ADJ_THREADS, 0, st>>>(C, col0, t->src_off, t->tr, t->dy, vp(a), t->u, j0, eb); }
+                    col0 += 12;
+                    continue;
+                }
+                { ProfScope ps_("k_adj_ray", st); k_adj_ray<NC, 3><<<gr, 256, 0, st>>>(sd, rd, C, col0, vp(a - 1), t->dy); }
+                { ProfScope ps_("k_adj_src", st); k_adj_src<NC><<<j1 - j0, ADJ_THREADS, 0, st>>>(C, col0, t->src_off, t->tr, t->dy, vp(a), t->u, j0, eb); }
+                col0 += 3;
             }
             RGS_LAUNCH("adjoint bounce");
         }
@@ -947,7 +1080,6 @@ rgs_status rgs_adjoint_impl(rgs_transport *t, const float *g, float *dE, float *
             pool_release(t->u, st);
             pool_release(t->tr, st);
             pool_release(t->dy, st);
-            pool_release(t->dy_mc, st);
             pool_release(t->gh, st);
             pool_release(geo.dp, st);
             pool_release(geo.ds, st);
@@ -955,7 +1087,6 @@ rgs_status rgs_adjoint_impl(rgs_transport *t, const float *g, float *dE, float *
         }
         RgsGeoAcc geo;
     } scratch{t, st, {}};
-    const bool mc = wide_adjoint(t->C);
     const bool want_gh = (dop || want_geo) && nb >= 1;
     // the last solve ran on the tensor cores: so do the transposed bounces (source tiles
     // instead of the transposed hit index and the per-ray adjoint values)
@@ -974,11 +1105,15 @@ rgs_status rgs_adjoint_impl(rgs_transport *t, const float *g, float *dE, float *
     const int n_v = t->stride ? t->stride + 1 : nb + 1;
     if ((r = pool_alloc(&t->v, A * n_v, st)) != RGS_OK) return r;
     if ((r = pool_alloc(&t->u, A, st)) != RGS_OK) return r;
-    if (tcp) {
-    } else if (mc) {
-        if ((r = pool_alloc(&t->dy_mc, (size_t)n_rays * 32, st)) != RGS_OK) return r;
-    } else {
-        if ((r = pool_alloc(&t->dy, (size_t)n_rays, st)) != RGS_OK) return r;
+    if (!tcp) {
+        // records of 12-column tiles (64 bytes a ray) unless they do not fit, or 3 are all there are
+        t->dy_cols = t->C > 3 ? 12 : 3;
+        r = pool_alloc(&t->dy, (size_t)n_rays * (t->dy_cols == 12 ? 16 : 8), st);
+        if (r == RGS_ERR_OOM && t->dy_cols == 12) {
+            t->dy_cols = 3;
+            r = pool_alloc(&t->dy, (size_t)n_rays * 8, st);
+        }
+        if (r != RGS_OK) return r;
     }
     if (want_gh && (r = pool_alloc(&t->gh, (size_t)t->n_slots, st)) != RGS_OK) return r;
     // The transposed index in one part when it fits next to the segment scratch of a
@@ -989,7 +1124,7 @@ rgs_status rgs_adjoint_impl(rgs_transport *t, const float *g, float *dE, float *
     const double tr_all = 8.0 * (double)t->n_hits;
     double avail = 0.92 * (double)pool_available_bytes() - seg;
     if (t->mem_budget > 0) {
-        const double scratch = 4.0 * A * (n_v + 1) + (mc ? 128.0 : 16.0) * n_rays + (want_gh ? 4.0 * t->n_slots : 0.0);
+        const double scratch = 4.0 * A * (n_v + 1) + (t->dy_cols == 12 ? 64.0 : 32.0) * n_rays + (want_gh ? 4.0 * t->n_slots : 0.0);
         avail = std::min(avail, (double)t->mem_budget - (double)t->device_bytes - scratch - seg);
     }
     int P = 1;

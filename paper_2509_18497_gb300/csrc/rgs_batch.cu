@@ -357,6 +357,7 @@ rgs_status rgs_solve_batched_impl(rgs_transport *const *tsp, int count, const fl
         key.push_back((const void *)(size_t)ts[s]->C);
         key.push_back(ts[s]->sc->P);
         key.push_back(ts[s]->sc->nodes);
+        key.push_back(ts[s]->sc->rec);
         key.push_back(ts[s]->off);
         key.push_back(ts[s]->dir);
         key.push_back(ts[s]->Q);
@@ -364,9 +365,7 @@ rgs_status rgs_solve_batched_impl(rgs_transport *const *tsp, int count, const fl
         key.push_back(ts[s]->iters16);
         key.push_back(ts[s]->rec_ja);
         key.push_back((const void *)(size_t)nbs[s]);
-        key.push_back(E ? E[s] : nullptr);
-        key.push_back(B_out ? B_out[s] : nullptr);
-    }
+    } // (E and B_out are read and written outside the captured launches)
     std::lock_guard<std::mutex> lk(g_plan_mu);
     Plan *P = g_plans.count(key) ? g_plans[key] : nullptr;
     const bool fresh = (P == nullptr);

@@ -636,10 +636,10 @@ struct rgs_transport {
     unsigned *ray_ctr = nullptr; // persistent trace: next ray to fetch
     int num_sms = 0;
     float4 *dir = nullptr; // per-ray direction
-    // adjoint scratch (dy, dy_mc, tr, v, u, gh): taken from the workspace pool at the start
+    // adjoint scratch (dy, tr, v, u, gh): taken from the workspace pool at the start
     // of rgs_adjoint and returned at its end; null outside that call
-    float4 *dy = nullptr;  // adjoint: per-ray (y[0..2], 0) for the current column tile
-    float *dy_mc = nullptr; // adjoint, many columns: per-ray y of one 32-column tile
+    float *dy = nullptr;    // adjoint: per-ray (direction, y) records of one column tile
+    int dy_cols = 3;        // its columns: 3 (8 floats a record) or 12 (16)
     long long rays_cap = 0;
     unsigned long long *counter = nullptr;
     int *flags = nullptr;
@@ -786,19 +786,13 @@ template <class T> void pool_release(T *&p, cudaStream_t st) {
 // 32-column tile but leave lanes idle when C is not a multiple of 32, and load a full
 // column row per lane (32 bytes BF16, 64 bytes FP32).  Crossovers measured on GB300 with
 // SH degree 3 and 50,000 surfels: the bounce on BF16 rows from 18 columns, on FP32 rows
-// from 64; the opacity gather on BF16 rows from 12, on FP32 rows from 64; the adjoint
-// (FP32) when one 32-column tile costs less than 26.5 three-column passes would.
+// from 64; the opacity gather on BF16 rows from 12, on FP32 rows from 64.
 __host__ __device__ inline bool wide_bounce(int C, bool rows16) { return C >= (rows16 ? 18 : 64); }
 __host__ __device__ inline bool wide_opacity(int C, bool rows16) { return C >= (rows16 ? 12 : 64); }
-__host__ __device__ inline bool wide_adjoint(int C) { return 2 * C > 53 * ((C + 31) / 32); }
 template <int NC>
 rgs_status mc_bounce(const rgs_transport *t, SceneDev sd, RaysDev rd, bool rows16, const float *Bprev,
                      const __nv_bfloat16 *Bprev16, const float *S, float *Q, float *Bout, __nv_bfloat16 *Bout16,
                      double *norm2, cudaStream_t st);
-// K^T for the sources j0 .. j1-1, whose transposed entries start at ebase in t->tr
-template <int NC>
-rgs_status mc_adjoint_bounce(rgs_transport *t, SceneDev sd, RaysDev rd, const float *vin, float *vout, int j0, int j1,
-                             long long ebase, cudaStream_t st);
 // per-launch set of up to NA adjoint iterates v^(a) and the matching B^(n-1-a) (FP32 or BF16)
 template <class T, int NA> struct OpaSet {
     const float *v[NA];

@@ -5,8 +5,8 @@
 // hit record once per 3-column tile; here a warp takes one ray (or one transposed entry) at
 // a time and its 32 lanes take 32 consecutive columns, so each hit is read once per
 // 32-column tile and every row load is one contiguous 512-byte (BF16) or 1-KiB (FP32)
-// warp access.  Which layout a launch uses is decided per kernel family by wide_bounce,
-// wide_opacity and wide_adjoint (rgs_internal.cuh).
+// warp access.  Which layout a launch uses is decided per kernel family by wide_bounce and
+// wide_opacity (rgs_internal.cuh).
 #include "rgs_bounce_body.cuh"
 
 namespace {
@@ -22,77 +22,6 @@ __global__ void RGS_MCB_LB k_bounce_mc(SceneDev sc, RaysDev rays, int C, const T
 }
 
 // ------------------------------------------------------------------ adjoint
-// y_r[c] = (pi/nd) o_i sum_k' c_{i,l(k'),ch} Y_k'(R_i d_r) v_i[c][k'] for the 32 columns of
-// tile `ct`, stored as dy[r*32 + lane]
-template <int NC>
-__global__ void __launch_bounds__(MC_THREADS) k_adj_ray_mc(SceneDev sc, RaysDev rays, int C, int ct,
-                                                          const float *__restrict__ vin, float *dy) {
-    const int i = blockIdx.x;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int col = ct * 32 + lane;
-    const bool live = col < C;
-    const int nd = rays.nd;
-    const float3 n = f3(sc.N4[i]);
-    float cv[NC]; // c_{i,l(k),ch(col)} * v_i[col][k] * o_i pi/nd
-    {
-        const float oi = alpha_center(sc, i) * (3.14159265358979f / (float)nd);
-        float v[NC];
-        if (live) load_col<NC>(vin + ((size_t)i * C + col) * NC, v);
-#pragma unroll
-        for (int k = 0; k < NC; ++k)
-            cv[k] = live ? oi * __ldg(&sc.cl[(size_t)i * 12 + band_of(k) * 3 + col % 3]) * v[k] : 0.f;
-    }
-    for (int q = warp; q < nd; q += MC_WARPS) {
-        const long long r = (long long)i * nd + q;
-        const float3 d = f3(rays.dir[r]);
-        float Yi[NC];
-        sh_eval<NC>(reflect_n(n, d), Yi);
-        float y = 0.f;
-#pragma unroll
-        for (int k = 0; k < NC; ++k) y += cv[k] * Yi[k];
-        dy[r * 32 + lane] = y;
-    }
-}
-
-// (K^T v)_j[c][k] = sum_{entries e on j} a_e Y_k(-d_e) y_e[c], one CTA per source j
-template <int NC>
-__global__ void RGS_MC_LB k_adj_src_mc(RaysDev rays, int C, int ct,
-                                                          const long long *__restrict__ src_off,
-                                                          const int2 *__restrict__ tr, const float *__restrict__ dy,
-                                                          float *__restrict__ vout, float *__restrict__ u, int j0,
-                                                          long long ebase) {
-    const int j = j0 + blockIdx.x; // sources j0 .. of this index part; its entries start at ebase
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float acc[NC];
-#pragma unroll
-    for (int k = 0; k < NC; ++k) acc[k] = 0.f;
-    const long long e0 = src_off[j] - ebase, e1 = src_off[j + 1] - ebase;
-    for (long long e = e0 + warp; e < e1; e += MC_WARPS) {
-        const int2 ent = __ldg(&tr[e]);
-        const float4 d4 = __ldg(&rays.dir[ent.x]);
-        float Yo[NC];
-        sh_eval<NC>(make_float3(-d4.x, -d4.y, -d4.z), Yo);
-        const float y = __int_as_float(ent.y) * __ldg(&dy[(long long)ent.x * 32 + lane]);
-#pragma unroll
-        for (int k = 0; k < NC; ++k) acc[k] += Yo[k] * y;
-    }
-    __shared__ float red[MC_WARPS][NC][32];
-#pragma unroll
-    for (int k = 0; k < NC; ++k) red[warp][k][lane] = acc[k];
-    __syncthreads();
-    for (int e = threadIdx.x; e < NC * 32; e += MC_THREADS) {
-        const int k = e >> 5, c = e & 31;
-        const int cc = ct * 32 + c;
-        if (cc >= C) continue;
-        float v = 0.f;
-#pragma unroll
-        for (int q = 0; q < MC_WARPS; ++q) v += red[q][k][c];
-        const size_t idx = ((size_t)j * C + cc) * NC + k;
-        vout[idx] = v;
-        u[idx] += v;
-    }
-}
-
 // opacity backward: per hit g_h (partial over this column tile and iterate chunk)
 // accumulated into gh[slot]; a warp per ray, lanes over columns
 template <int NC, int NA, class T>
@@ -181,17 +110,6 @@ rgs_status mc_bounce(const rgs_transport *t, SceneDev sd, RaysDev rd, bool rows1
 }
 
 template <int NC>
-rgs_status mc_adjoint_bounce(rgs_transport *t, SceneDev sd, RaysDev rd, const float *vin, float *vout, int j0, int j1,
-                             long long ebase, cudaStream_t st) {
-    for (int ct = 0; ct * 32 < t->C; ++ct) {
-        { ProfScope ps_("k_adj_ray_mc", st); k_adj_ray_mc<NC><<<t->n, MC_THREADS, 0, st>>>(sd, rd, t->C, ct, vin, t->dy_mc); }
-        { ProfScope ps_("k_adj_src_mc", st); k_adj_src_mc<NC><<<j1 - j0, MC_THREADS, 0, st>>>(rd, t->C, ct, t->src_off, t->tr, t->dy_mc, vout, t->u, j0, ebase); }
-    }
-    RGS_LAUNCH("adjoint bounce mc");
-    return RGS_OK;
-}
-
-template <int NC>
 rgs_status mc_opacity(rgs_transport *t, SceneDev sd, RaysDev rd, int na, const float *const *v, const float *const *Bf,
                       const __nv_bfloat16 *const *Bh, bool first, cudaStream_t st) {
     constexpr int NA = 4;
@@ -221,8 +139,6 @@ rgs_status mc_opacity(rgs_transport *t, SceneDev sd, RaysDev rd, int na, const f
     template rgs_status mc_bounce<NC>(const rgs_transport *, SceneDev, RaysDev, bool, const float *,                   \
                                       const __nv_bfloat16 *, const float *, float *, float *, __nv_bfloat16 *,         \
                                       double *, cudaStream_t);                                                         \
-    template rgs_status mc_adjoint_bounce<NC>(rgs_transport *, SceneDev, RaysDev, const float *, float *, int, int,    \
-                                              long long, cudaStream_t);                                                \
     template rgs_status mc_opacity<NC>(rgs_transport *, SceneDev, RaysDev, int, const float *const *,                 \
                                        const float *const *, const __nv_bfloat16 *const *, bool, cudaStream_t);
 RGS_MC_INSTANTIATE(1)

@@ -172,7 +172,7 @@ int rgs_auto_stride(const rgs_transport *t, int nb, int precision) {
     const double A16 = precision != RGS_FP32 ? 2.0 * t->n * t->C * bf16_row(t->nc) : 0.0;
     const double rays = (double)t->n * t->nd;
     const double fwd = (nb + 1) * (A + A16) + nb * A;
-    const double adj = (nb + 2) * A + 8.0 * t->n_hits + 4.0 * t->n_slots + rays * (wide_adjoint(t->C) ? 128 : 16);
+    const double adj = (nb + 2) * A + 8.0 * t->n_hits + 4.0 * t->n_slots + rays * (t->C > 3 ? 64 : 32);
     const double held = t->iters_cap * A + t->q_cap * A + t->iters16_cap * A16;
     double room = 0.95 * ((double)pool_available_bytes() + held);
     if (t->mem_budget > 0) room = std::min(room, (double)t->mem_budget - ((double)t->device_bytes - held));
