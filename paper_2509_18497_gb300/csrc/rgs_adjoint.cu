@@ -802,7 +802,7 @@ rgs_status build_index(rgs_transport *t, int j0, int j1, long long ebase, cudaSt
 template <int NC>
 rgs_status opacity_group(rgs_transport *t, SceneDev sd, RaysDev rd, int na, const float *const *v,
                          const float *const *Bf, const __nv_bfloat16 *const *Bh, bool first, cudaStream_t st) {
-    if (wide_opacity(t->C, Bh != nullptr)) return mc_opacity<NC>(t, sd, rd, na, v, Bf, Bh, first, st);
+    if (wide_opacity(NC, t->C, Bh != nullptr)) return mc_opacity<NC>(t, sd, rd, na, v, Bf, Bh, first, st);
     constexpr int NA = 4;
     const long long n_rays = (long long)t->n * t->nd;
     const unsigned gg = (unsigned)((n_rays * Slice<NC>::G + 255) / 256);

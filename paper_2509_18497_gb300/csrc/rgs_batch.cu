@@ -171,7 +171,7 @@ struct Plan {
 
 std::mutex g_plan_mu;
 std::map<std::vector<const void *>, Plan *> g_plans;
-bool policy_wide(int pol, int C, bool rows16);
+bool policy_wide(int pol, int nc, int C, bool rows16);
 std::vector<int32_t> g_last_plan; // the plan of the last rgs_solve_batched call (rgs_batch_last_plan)
 
 void note_plan(const Plan &P) {
@@ -187,8 +187,8 @@ void note_plan(const Plan &P) {
         g_last_plan.push_back(P.bkey[k][2]);
         g_last_plan.push_back(P.pol16[k]);
         g_last_plan.push_back(P.pol32[k]);
-        g_last_plan.push_back(policy_wide(P.pol16[k], C, true) ? 32 : 3);
-        g_last_plan.push_back(policy_wide(P.pol32[k], C, false) ? 32 : 3);
+        g_last_plan.push_back(policy_wide(P.pol16[k], P.bkey[k][0], C, true) ? 32 : 3);
+        g_last_plan.push_back(policy_wide(P.pol32[k], P.bkey[k][0], C, false) ? 32 : 3);
     }
 }
 
@@ -198,8 +198,8 @@ void enqueue_make_S(rgs_transport *t, const float *E, cudaStream_t st, bool bf16
 // columns from which policy 2 gives a scene 32-column items
 constexpr int kWideMinCols = 6;
 
-bool policy_wide(int pol, int C, bool rows16) {
-    return pol == 0 ? false : (pol == 1 ? wide_bounce(C, rows16) : C >= kWideMinCols);
+bool policy_wide(int pol, int nc, int C, bool rows16) {
+    return pol == 0 ? false : (pol == 1 ? wide_bounce(nc, C, rows16) : C >= kWideMinCols);
 }
 
 // item shapes of every scene under the plan's policies, the level offsets they imply, and
@@ -208,8 +208,8 @@ rgs_status upload_shape(Plan &P, cudaStream_t st, bool force32 = false) {
     const int count = P.count;
     for (int s = 0; s < count; ++s) {
         BatchSceneDev &b = P.host[s];
-        b.wide16 = policy_wide(P.pol16[P.bucket[s]], b.C, true) ? 1 : 0;
-        b.wide32 = policy_wide(P.pol32[P.bucket[s]], b.C, false) ? 1 : 0;
+        b.wide16 = policy_wide(P.pol16[P.bucket[s]], b.nc, b.C, true) ? 1 : 0;
+        b.wide32 = policy_wide(P.pol32[P.bucket[s]], b.nc, b.C, false) ? 1 : 0;
         b.tiles16 = b.wide16 ? (b.C + 31) / 32 : b.C / 3;
         b.tiles32 = b.wide32 ? (b.C + 31) / 32 : b.C / 3;
     }

@@ -1,6 +1,6 @@
 // Bounce gather/projection for one receiver and one column tile (the body of k_bounce and
-// of the persistent batch kernel): CTA-wide, BOUNCE_THREADS threads, red = shared scratch of
-// (BOUNCE_THREADS/32) * G * KPL * CT floats.
+// of the persistent batch kernel): CTA-wide, up to BOUNCE_THREADS threads, red = shared scratch
+// of (BOUNCE_THREADS/32) * G * KPL * CT floats.
 #pragma once
 #include "rgs_internal.cuh"
 
@@ -100,8 +100,8 @@ __device__ __forceinline__ void bounce_receiver(const SceneDev &sc, const RaysDe
                                                 float *__restrict__ Bout, __nv_bfloat16 *__restrict__ Bout16,
                                                 double *norm2, int i, int col0, float *red) {
 
-    constexpr int G = SL::G, KPL = SL::KPL, GROUPS = BOUNCE_THREADS / G, RS = SL::STRIDE;
-    const int nd = rays.nd;
+    constexpr int G = SL::G, KPL = SL::KPL, RS = SL::STRIDE;
+    const int nd = rays.nd, groups = blockDim.x / G;
     const int grp = threadIdx.x / G, g = threadIdx.x % G;
     const float3 n = f3(sc.N4[i]);
     float acc[KPL][CT];
@@ -110,7 +110,7 @@ __device__ __forceinline__ void bounce_receiver(const SceneDev &sc, const RaysDe
 #pragma unroll
         for (int c = 0; c < CT; ++c) acc[m][c] = 0.f;
 
-    for (int q = grp; q < nd; q += GROUPS) {
+    for (int q = grp; q < nd; q += groups) {
         const long long r = (long long)i * nd + q;
         const float3 d = f3(rays.dir[r]);
         float yo[KPL], yi[KPL];
@@ -175,7 +175,7 @@ __device__ __forceinline__ void bounce_epilogue(const SceneDev &sc, int C, const
         }
     __syncthreads();
     double dsq = 0.0;
-    for (int e = threadIdx.x; e < NC * CT; e += BOUNCE_THREADS) {
+    for (int e = threadIdx.x; e < NC * CT; e += blockDim.x) {
         const int k = e / CT, c = e - k * CT;
         int gg = 0, mm = 0;
 #pragma unroll
@@ -187,7 +187,7 @@ __device__ __forceinline__ void bounce_epilogue(const SceneDev &sc, int C, const
                     mm = m2;
                 }
         float v = 0.f;
-        for (int q = 0; q < BOUNCE_THREADS / 32; ++q) v += red[(q * G + gg) * (KPL * CT) + mm * CT + c];
+        for (int q = 0; q < blockDim.x / 32; ++q) v += red[(q * G + gg) * (KPL * CT) + mm * CT + c];
         const int col = col0 + c;
         const float Q = w * v;
         const size_t idx = ((size_t)i * C + col) * NC + k;
@@ -208,16 +208,16 @@ __device__ __forceinline__ void bounce_epilogue(const SceneDev &sc, int C, const
 
 // Lane-per-column bounce for one receiver and one 32-column tile (the body of k_bounce_mc and
 // of the persistent batch kernel's wide items); red = shared scratch of MC_WARPS * NC * 32 floats.
-template <int NC, class T>
+template <int NC, class T, bool HALF>
 __device__ __forceinline__ void bounce_receiver_mc(const SceneDev &sc, const RaysDev &rays, int C,
                                                    const T *__restrict__ Bg, const float *__restrict__ Bprev,
                                                    const float *__restrict__ S, float *__restrict__ Qout,
                                                    float *__restrict__ Bout, __nv_bfloat16 *__restrict__ Bout16,
                                                    double *norm2, int i, int tile, float *red) {
     constexpr int RS = row_stride<NC, T>();
-    constexpr bool COOP = sizeof(T) == 4 && NC == 16; // whole-tile reads (TileDot)
+    constexpr bool COOP = sizeof(T) == 4 && NC == 16 && !HALF; // whole-tile reads (TileDot)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int own = lane; // the tile column whose sums this lane keeps
+    int own = HALF ? lane & 15 : lane; // the tile column whose sums this lane keeps
     if constexpr (COOP) own = TileDot<T, NC>::own(lane);
     const int col = tile * 32 + own;
     const bool live = col < C;
@@ -228,41 +228,45 @@ __device__ __forceinline__ void bounce_receiver_mc(const SceneDev &sc, const Ray
     float acc[NC];
 #pragma unroll
     for (int k = 0; k < NC; ++k) acc[k] = 0.f;
-    for (int q = warp; q < nd; q += MC_WARPS) {
-        const long long r = (long long)i * nd + q;
+    for (int rq = warp; rq < nd; rq += MC_WARPS) {
+        const long long r = (long long)i * nd + rq;
         const float3 d = f3(rays.dir[r]);
         float Yo[NC];
         sh_eval<NC>(neg3(d), Yo);
         const int cnt = rays.cnt[r];
         const long long base = rays.off[r];
         float x = 0.f;
-        if constexpr (COOP) {
-            float ys[TileDot<T, NC>::KPL];
-            TileDot<T, NC>::pick(Yo, lane, ys);
-#pragma unroll 2
-            for (int h = 0; h < cnt; ++h) {
-                const int2 ja = __ldg(&rays.rec_ja[base + h]);
-                x += __int_as_float(ja.y) * TileDot<T, NC>::dot(Bg + ((size_t)ja.x * C + tile * 32) * RS, ncols, lane, ys);
-            }
-        } else {
-#pragma unroll 2
-            for (int h = 0; h < cnt; ++h) {
-                const int2 ja = __ldg(&rays.rec_ja[base + h]);
-                float v[NC];
-                load_col<NC>(Bg + ((size_t)ja.x * C + colc) * RS, v);
-                float s = 0.f;
+        [[maybe_unused]] float ys[8]; // this lane's half of Y(-d) (TileDot)
+        if constexpr (COOP) TileDot<T, NC>::pick(Yo, lane, ys);
+        for (int h0 = 0; h0 < cnt; h0 += 32) { // the lanes hold 32 records; four rows are requested together
+            const int m = min(32, cnt - h0);
+            const int2 rec = lane < m ? __ldg(&rays.rec_ja[base + h0 + lane]) : make_int2(0, 0);
+#pragma unroll 4
+            for (int q = 0; q < m; q += HALF ? 2 : 1) { // HALF: the upper 16 lanes take the next hit
+                const int h = HALF ? q + (lane >> 4) : q, hc = HALF ? min(h, m - 1) : h;
+                const int j = __shfl_sync(0xffffffffu, rec.x, hc);
+                const float aw = __int_as_float(__shfl_sync(0xffffffffu, rec.y, hc));
+                const float a = HALF && h >= m ? 0.f : aw;
+                if constexpr (COOP) {
+                    x += a * TileDot<T, NC>::dot(Bg + ((size_t)j * C + tile * 32) * RS, ncols, lane, ys);
+                } else {
+                    float v[NC];
+                    load_col<NC>(Bg + ((size_t)j * C + colc) * RS, v);
+                    float s = 0.f;
 #pragma unroll
-                for (int k = 0; k < NC; ++k) s += Yo[k] * v[k];
-                x += __int_as_float(ja.y) * s;
+                    for (int k = 0; k < NC; ++k) s += Yo[k] * v[k];
+                    x += a * s;
+                }
             }
         }
+        if constexpr (HALF) x += __shfl_xor_sync(0xffffffffu, x, 16);
         float Yi[NC];
         sh_eval<NC>(reflect_n(n, d), Yi);
 #pragma unroll
         for (int k = 0; k < NC; ++k) acc[k] += Yi[k] * x;
     }
 #pragma unroll
-    for (int k = 0; k < NC; ++k) red[(warp * NC + k) * 32 + own] = acc[k];
+    for (int k = 0; k < NC; ++k) red[(warp * NC + k) * 32 + own] = acc[k]; // (HALF: both halves the same)
     __syncthreads();
     double dsq = 0.0;
     const float w = 3.14159265358979f / (float)nd;
@@ -286,4 +290,16 @@ __device__ __forceinline__ void bounce_receiver_mc(const SceneDev &sc, const Ray
     for (int off = 16; off > 0; off >>= 1) dsq += __shfl_xor_sync(0xffffffffu, dsq, off);
     if (lane == 0) atomicAdd(norm2, dsq);
     __syncthreads(); // red is reused by the caller's next receiver
+}
+// the same, a tile of up to 16 columns taken two hits at a time
+template <int NC, class T>
+__device__ __forceinline__ void bounce_receiver_mc(const SceneDev &sc, const RaysDev &rays, int C,
+                                                   const T *__restrict__ Bg, const float *__restrict__ Bprev,
+                                                   const float *__restrict__ S, float *__restrict__ Qout,
+                                                   float *__restrict__ Bout, __nv_bfloat16 *__restrict__ Bout16,
+                                                   double *norm2, int i, int tile, float *red) {
+    if (half_tile(NC, C - tile * 32, sizeof(T) == 2))
+        bounce_receiver_mc<NC, T, true>(sc, rays, C, Bg, Bprev, S, Qout, Bout, Bout16, norm2, i, tile, red);
+    else
+        bounce_receiver_mc<NC, T, false>(sc, rays, C, Bg, Bprev, S, Qout, Bout, Bout16, norm2, i, tile, red);
 }

@@ -25,9 +25,9 @@
 // is sized for that many resident blocks per SM (these latency-bound kernels gain from more
 // resident warps as long as nothing spills); undefined, the compiler's default budget.
 // Build-time knobs, set from measurements on GB300 (50,000-surfel bowl, 1 and 16 lights):
-// 5 blocks for the 3-column bounce (-9 %, despite a few spilled registers) and 4 for the
-// lane-per-column bounce (-18 %); the opacity and adjoint gathers keep the default (tighter
-// budgets measured slower).
+// 5 blocks for the 3-column bounce (-9 %, despite a few spilled registers), 4 for the
+// lane-per-column bounce (-18 %) and opacity gather (-5 %); the 3-column opacity gather keeps
+// the default (tighter budgets measured slower).
 #define RGS_LB_(threads, minb) __launch_bounds__(threads, minb)
 #ifndef RGS_BOUNCE_MINB
 #define RGS_BOUNCE_MINB 5
@@ -56,11 +56,10 @@
 #else
 #define RGS_ADJ_LB __launch_bounds__(128)
 #endif
-#ifdef RGS_MC_MINB
-#define RGS_MC_LB RGS_LB_(256, RGS_MC_MINB)
-#else
-#define RGS_MC_LB __launch_bounds__(256)
+#ifndef RGS_MC_MINB
+#define RGS_MC_MINB 4
 #endif
+#define RGS_MC_LB RGS_LB_(256, RGS_MC_MINB)
 
 // ------------------------------------------------------------------ error flags
 enum {
@@ -783,12 +782,22 @@ template <class T> void pool_release(T *&p, cudaStream_t st) {
 // Column layout of the gathers.  The 3-column kernels (4 lanes share a ray, each lane a
 // slice of the coefficients of 3 columns) re-read the hit records and re-evaluate the SH
 // per 3-column tile; the lane-per-column kernels (rgs_manycol.cu) read them once per
-// 32-column tile but leave lanes idle when C is not a multiple of 32, and load a full
-// column row per lane (32 bytes BF16, 64 bytes FP32).  Crossovers measured on GB300 with
-// SH degree 3 and 50,000 surfels: the bounce on BF16 rows from 18 columns, on FP32 rows
-// from 64; the opacity gather on BF16 rows from 12, on FP32 rows from 64.
-__host__ __device__ inline bool wide_bounce(int C, bool rows16) { return C >= (rows16 ? 18 : 64); }
-__host__ __device__ inline bool wide_opacity(int C, bool rows16) { return C >= (rows16 ? 12 : 64); }
+// 32-column tile but leave lanes idle when C is not a multiple of 16 (a half tile takes two
+// hits at a time) or 32.  Crossovers measured on GB300 (20,000 surfels, 64 rays, 3 to 60
+// columns), e.g. at 16 coefficients: the bounce on FP32 rows, 6.1 against 6.2 ms at 18 columns
+// and 8.2 against 6.3 at 24; on BF16 rows 2.8 against 3.2 ms at 9 and 3.7 against 3.2 at 12; the
+// opacity gather on FP32 rows 4.2 against 4.7 ms at 9 and 5.6 against 4.8 at 12, on BF16 rows
+// 1.1 against 2.1 ms at 3 and 2.4 against 2.2 at 6.
+__host__ __device__ inline bool wide_bounce(int nc, int C, bool rows16) {
+    return C >= (rows16 ? 12 : (nc == 16 ? 18 : (nc == 9 ? 9 : 12)));
+}
+__host__ __device__ inline bool wide_opacity(int nc, int C, bool rows16) {
+    return C >= (nc < 9 ? 9 : (nc == 16 && !rows16 ? 12 : 6));
+}
+// Half tiles give a lane a whole column row; FP32 rows of 16 coefficients are read faster as
+// whole tiles (TileDot) once they are more than half full (9 columns: 4.8 against 5.6 ms, 15:
+// 6.6 against 5.8).
+__host__ __device__ inline bool half_tile(int nc, int cols, bool rows16) { return cols <= (nc == 16 && !rows16 ? 9 : 16); }
 template <int NC>
 rgs_status mc_bounce(const rgs_transport *t, SceneDev sd, RaysDev rd, bool rows16, const float *Bprev,
                      const __nv_bfloat16 *Bprev16, const float *S, float *Q, float *Bout, __nv_bfloat16 *Bout16,

@@ -23,12 +23,17 @@ __global__ void RGS_MCB_LB k_bounce_mc(SceneDev sc, RaysDev rays, int C, const T
 
 // ------------------------------------------------------------------ adjoint
 // opacity backward: per hit g_h (partial over this column tile and iterate chunk)
-// accumulated into gh[slot]; a warp per ray, lanes over columns
-template <int NC, int NA, class T>
+// accumulated into gh[slot]; a warp per ray, lanes over columns.  The lanes hold 32 of the ray's
+// records at a time, four hits' rows are requested together, and their four sums over the
+// columns share one reduction: with a hit, its row and a five-step reduction at a time every
+// hit waited for the last, and lane 0's stores took a request each (60,000 surfels, 128 rays, 48
+// columns, two launches: 103 -> 85 ms).  HALF: a tile of up to 16 columns, the upper 16 lanes
+// take every other hit (85 -> 75 ms).
+template <int NC, int NA, class T, bool HALF>
 __global__ void RGS_MC_LB k_opacity_g_mc(SceneDev sc, RaysDev rays, int C, int ct, int na,
                                                             OpaSet<T, NA> it, float *gh, bool first) {
     constexpr int RS = row_stride<NC, T>();
-    constexpr bool COOP = sizeof(T) == 4 && NC == 16; // whole-tile reads (TileDot)
+    constexpr bool COOP = sizeof(T) == 4 && NC == 16 && !HALF; // whole-tile reads (TileDot)
     const int warp_g = (int)((blockIdx.x * (size_t)MC_THREADS + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
     const int n_rays = sc.n * rays.nd;
@@ -36,7 +41,7 @@ __global__ void RGS_MC_LB k_opacity_g_mc(SceneDev sc, RaysDev rays, int C, int c
     const int r = warp_g;
     const int cnt = rays.cnt[r];
     if (cnt == 0) return;
-    int own = lane; // the tile column whose terms this lane forms
+    int own = HALF ? lane & 15 : lane; // the tile column whose terms this lane forms
     if constexpr (COOP) own = TileDot<T, NC>::own(lane);
     const int col = ct * 32 + own;
     const bool live = col < C;
@@ -66,27 +71,55 @@ __global__ void RGS_MC_LB k_opacity_g_mc(SceneDev sc, RaysDev rays, int C, int c
     const long long base = rays.off[r];
     [[maybe_unused]] float ys[8]; // this lane's half of Y(-d) (TileDot)
     if constexpr (COOP) TileDot<T, NC>::pick(Yo, lane, ys);
-    for (int h = 0; h < cnt; ++h) {
-        const int j = __ldg(&rays.rec_ja[base + h]).x;
-        float acc = 0.f;
+    constexpr int U = 4;
+    for (int h0 = 0; h0 < cnt; h0 += 32) {
+        const int m = min(32, cnt - h0);
+        const int jl = lane < m ? __ldg(&rays.rec_ja[base + h0 + lane]).x : 0;
+        float mine = 0.f; // g of hit h0 + lane
+        const int half = HALF ? lane >> 4 : 0;
+        for (int q = 0; q < m; q += HALF ? 2 * U : U) {
+            int j[U];
+            float acc[U];
 #pragma unroll
-        for (int aa = 0; aa < NA; ++aa) {
-            if (aa < na) {
-                float s = 0.f;
-                if constexpr (COOP) {
-                    s = TileDot<T, NC>::dot(it.b[aa] + ((size_t)j * C + ct * 32) * RS, ncols, lane, ys);
-                } else {
-                    float v[NC];
-                    load_col<NC>(it.b[aa] + ((size_t)j * C + colc) * RS, v);
-#pragma unroll
-                    for (int k = 0; k < NC; ++k) s += Yo[k] * v[k];
-                }
-                acc += y[aa] * s;
+            for (int u = 0; u < U; ++u) {
+                j[u] = __shfl_sync(0xffffffffu, jl, min(HALF ? q + 2 * u + half : q + u, m - 1));
+                acc[u] = 0.f;
             }
-        }
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-        if (lane == 0) gh[base + h] = first ? acc : gh[base + h] + acc;
+            for (int aa = 0; aa < NA; ++aa) {
+                if (aa < na) {
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        float s = 0.f;
+                        if constexpr (COOP) {
+                            s = TileDot<T, NC>::dot(it.b[aa] + ((size_t)j[u] * C + ct * 32) * RS, ncols, lane, ys);
+                        } else {
+                            float v[NC];
+                            load_col<NC>(it.b[aa] + ((size_t)j[u] * C + colc) * RS, v);
+#pragma unroll
+                            for (int k = 0; k < NC; ++k) s += Yo[k] * v[k];
+                        }
+                        acc[u] += y[aa] * s;
+                    }
+                }
+            }
+            // the four sums over the (half) warp at once: its two top lane bits come to select the hit
+            constexpr int B1 = HALF ? 8 : 16, B2 = B1 / 2;
+            const bool b1 = lane & B1, b2 = lane & B2;
+            const float s01 = (b1 ? acc[1] : acc[0]) + __shfl_xor_sync(0xffffffffu, b1 ? acc[0] : acc[1], B1);
+            const float s23 = (b1 ? acc[3] : acc[2]) + __shfl_xor_sync(0xffffffffu, b1 ? acc[2] : acc[3], B1);
+            float s = (b2 ? s23 : s01) + __shfl_xor_sync(0xffffffffu, b2 ? s01 : s23, B2);
+#pragma unroll
+            for (int off = B2 / 2; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+            const int d = lane - q, u = HALF ? d >> 1 : d;
+            const int from = (u & 1 ? B1 : 0) | (u & 2 ? B2 : 0) | (HALF && (d & 1) ? 16 : 0);
+            s = __shfl_sync(0xffffffffu, s, from);
+            if (d >= 0 && u < U) mine = s;
+        }
+        if (lane < m) {
+            const long long slot = base + h0 + lane;
+            gh[slot] = first ? mine : gh[slot] + mine;
+        }
     }
 }
 
@@ -125,10 +158,16 @@ rgs_status mc_opacity(rgs_transport *t, SceneDev sd, RaysDev rd, int na, const f
     for (int ct = 0; ct * 32 < t->C; ++ct) {
         if (Bh) {
             ProfScope ps_("k_opacity_g_mc", st);
-            k_opacity_g_mc<NC, NA, __nv_bfloat16><<<grid, MC_THREADS, 0, st>>>(sd, rd, t->C, ct, na, sh, t->gh, first && ct == 0);
+            if (half_tile(NC, t->C - ct * 32, true))
+                k_opacity_g_mc<NC, NA, __nv_bfloat16, true><<<grid, MC_THREADS, 0, st>>>(sd, rd, t->C, ct, na, sh, t->gh, first && ct == 0);
+            else
+                k_opacity_g_mc<NC, NA, __nv_bfloat16, false><<<grid, MC_THREADS, 0, st>>>(sd, rd, t->C, ct, na, sh, t->gh, first && ct == 0);
         } else {
             ProfScope ps_("k_opacity_g_mc", st);
-            k_opacity_g_mc<NC, NA, float><<<grid, MC_THREADS, 0, st>>>(sd, rd, t->C, ct, na, sf, t->gh, first && ct == 0);
+            if (half_tile(NC, t->C - ct * 32, false))
+                k_opacity_g_mc<NC, NA, float, true><<<grid, MC_THREADS, 0, st>>>(sd, rd, t->C, ct, na, sf, t->gh, first && ct == 0);
+            else
+                k_opacity_g_mc<NC, NA, float, false><<<grid, MC_THREADS, 0, st>>>(sd, rd, t->C, ct, na, sf, t->gh, first && ct == 0);
         }
     }
     RGS_LAUNCH("opacity mc");

@@ -57,12 +57,17 @@ rgs_status launch_bounce(const rgs_transport *t, SceneDev sd, RaysDev rd, bool b
                          const __nv_bfloat16 *Bprev16, const float *S, float *Q, float *Bout, __nv_bfloat16 *Bout16,
                          double *norm2, cudaStream_t st) {
     dim3 grid(t->n, t->C / 3);
+    // A block of a few rays per lane group: with 256 threads whatever the SH degree and ray count,
+    // most of a block had no ray (4 coefficients, a thread per ray, 64 rays: 1.81 -> 0.56 ms on
+    // 20,000 surfels; 16 coefficients, 32 rays: 1.06 -> 0.55), and at 256 rays the block waited for
+    // its slowest of 4 rays a group instead of 8 (3.94 -> 3.78).
+    const int threads = Slice<NC>::G > 1 ? (t->nd >= 128 ? 128 : 64) : (t->nd >= 64 ? 64 : 32);
     if (bf16_rows) {
         ProfScope ps_("k_bounce", st);
-        k_bounce<NC, 3, SliceH<NC>><<<grid, BOUNCE_THREADS, 0, st>>>(sd, rd, t->C, Bprev16, Bprev, S, Q, Bout, Bout16, norm2);
+        k_bounce<NC, 3, SliceH<NC>><<<grid, threads, 0, st>>>(sd, rd, t->C, Bprev16, Bprev, S, Q, Bout, Bout16, norm2);
     } else {
         ProfScope ps_("k_bounce", st);
-        k_bounce<NC, 3, Slice<NC>><<<grid, BOUNCE_THREADS, 0, st>>>(sd, rd, t->C, Bprev, Bprev, S, Q, Bout, Bout16, norm2);
+        k_bounce<NC, 3, Slice<NC>><<<grid, threads, 0, st>>>(sd, rd, t->C, Bprev, Bprev, S, Q, Bout, Bout16, norm2);
     }
     RGS_LAUNCH("bounce");
     return RGS_OK;
@@ -126,7 +131,7 @@ rgs_status run_solve(rgs_transport *t, const float *E, int nb, int precision, cu
             r = pairs_bounce<NC>(t, rows16, t->iters + A * sp, bf16 ? I16 + A16 * sp : nullptr, t->iters,
                                  t->Q + A * (b - 1), t->iters + A * so, bf16 ? I16 + A16 * so : nullptr, t->norm2 + b, st);
         else
-            r = (wide_bounce(t->C, rows16) ? mc_bounce<NC> : launch_bounce<NC>)(
+            r = (wide_bounce(NC, t->C, rows16) ? mc_bounce<NC> : launch_bounce<NC>)(
                 t, sd, rd, rows16, t->iters + A * sp, bf16 ? I16 + A16 * sp : nullptr, t->iters,
                 t->Q + A * (t->stride ? 0 : b - 1), t->iters + A * so, bf16 ? I16 + A16 * so : nullptr, t->norm2 + b, st);
         if (r != RGS_OK) return r;
@@ -147,7 +152,7 @@ rgs_status run_recompute(rgs_transport *t, int c, int e, float *const *B, __nv_b
         const int k = b - c - 1;
         const float *Bp = k == 0 ? t->iters + A * t->slot(c) : B[k - 1];
         const __nv_bfloat16 *Bp16 = !bf16 ? nullptr : (k == 0 ? t->iters16 + A16 * t->slot(c) : B16[k - 1]);
-        rgs_status r = (wide_bounce(t->C, rows16) ? mc_bounce<NC> : launch_bounce<NC>)(
+        rgs_status r = (wide_bounce(NC, t->C, rows16) ? mc_bounce<NC> : launch_bounce<NC>)(
             t, sd, rd, rows16, Bp, Bp16, t->iters, Q[k], B[k], bf16 ? B16[k] : nullptr, norm2 + b, st);
         if (r != RGS_OK) return r;
     }
