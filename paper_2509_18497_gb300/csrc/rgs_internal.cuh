@@ -615,7 +615,7 @@ struct rgs_transport {
     float *lpos = nullptr, *lint = nullptr;
     int lcap = 0;
     // center-to-center pairs: receiver i's pairs at pair_off[i] .. pair_off[i+1], each
-    // (source j, bits of V_ji); chunk_off: first pair of each (receiver, 256-source chunk)
+    // (source j, bits of V_ji); chunk_off: first pair of each (receiver, source chunk)
     long long *pair_off = nullptr;
     int2 *pair_rec = nullptr;
     long long pair_cap = 0, n_pairs = 0;

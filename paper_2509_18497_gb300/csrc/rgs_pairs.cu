@@ -13,7 +13,7 @@
 // Storage: the pairs of receiver i are contiguous (pair_off[i] .. pair_off[i+1]), each one
 // record (j, bits of V_ji), sources in increasing internal (Morton) index, so that a warp's 32
 // segments leave one centre towards neighbouring sources.  A count pass sizes
-// every (receiver, 256-source chunk) block exactly; the fill pass traces each front pair's
+// every (receiver, source chunk) block exactly; the fill pass traces each front pair's
 // segment and writes its record at the chunk's offset plus its rank in the block.
 #include <algorithm>
 #include <type_traits>
@@ -24,7 +24,15 @@
 
 namespace {
 
-constexpr int PCH = 256;      // sources per block of the count / fill passes
+// Sources per block of the count, fill and gradient passes, and the threads of the last two:
+// a warp takes 32 of the block's front sources (about half of all) at a time.  A thread per
+// source left half of each block's warps without one while the block held their registers and
+// shared memory (23 % of the warp slots active).  4,000 surfels: fill 20.5 -> 17.4 ms, gradient
+// 23.0 -> 19.6 ms.  Where there are few blocks, smaller ones end more evenly (fill, 256 against
+// 512 sources: 500 surfels 0.41 and 0.58 ms, 1,500 2.70 and 2.85, 2,500 7.76 and 7.48).
+constexpr int PCH = 512; // at most
+int pair_chunk(int n) { return n < 2048 ? 256 : 512; }
+constexpr int PT = 128;
 constexpr int PAIR_THREADS = 128;
 
 // Ein(x) = int_0^x (1 - e^{-y}) / y dy in FP32: for x <= 2 its power series
@@ -98,23 +106,33 @@ __device__ __forceinline__ bool pair_occludes(const SceneDev &sc, int k, int j, 
     return fabsf(e) > eps;
 }
 
-// The front sources of a (receiver, 256-source chunk) block in increasing order, packed so that
-// the first warps hold them all and no lane idles beside a source behind the receiver.
+// The front sources of a (receiver, source chunk) block in increasing order, packed: the
+// block's warps take 32 of them at a time, and no lane idles beside a source behind the receiver.
 struct PairChunk {
     int base[PCH / 32];
     int j[PCH];
 };
-__device__ __forceinline__ int pack_front(PairChunk &s, bool front, int j) {
+__device__ __forceinline__ int pack_front(PairChunk &s, const SceneDev &sc, int n, int i, int c, int pch, float3 pi,
+                                          float3 ni, float eps) {
+    constexpr int R = PCH / PT;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const unsigned bal = __ballot_sync(WT_FULL, front);
-    if (lane == 0) s.base[warp] = __popc(bal);
+    unsigned bal[R];
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+        const int j = c * pch + q * PT + threadIdx.x;
+        float3 dv;
+        bal[q] = __ballot_sync(WT_FULL, q * PT < pch && j < n && j != i && pair_front(sc, pi, ni, j, eps, dv));
+        if (lane == 0) s.base[q * (PT / 32) + warp] = __popc(bal[q]);
+    }
     __syncthreads();
-    int base = 0, total = 0;
+    int total = 0;
+#pragma unroll
     for (int w = 0; w < PCH / 32; ++w) {
-        if (w < warp) base += s.base[w];
+        const int q = w / (PT / 32);
+        if (w % (PT / 32) == warp && (bal[q] >> lane & 1u))
+            s.j[total + __popc(bal[q] & ((1u << lane) - 1u))] = c * pch + q * PT + threadIdx.x;
         total += s.base[w];
     }
-    if (front) s.j[base + __popc(bal & ((1u << lane) - 1u))] = j;
     __syncthreads();
     return total;
 }
@@ -122,7 +140,7 @@ __device__ __forceinline__ int pack_front(PairChunk &s, bool front, int j) {
 __global__ void __launch_bounds__(PCH) k_pair_count(SceneDev sc, int n, int chunks, int *chunk_cnt, int *src_cnt) {
     const int blk = blockIdx.x;
     const int i = blk / chunks, c = blk - i * chunks;
-    const int j = c * PCH + threadIdx.x;
+    const int j = c * blockDim.x + threadIdx.x;
     const float eps = *sc.eps_plane;
     const float3 pi = f3(sc.P[i]), ni = f3(sc.N4[i]);
     float3 dv;
@@ -138,8 +156,8 @@ struct PairWarp {
     WarpOcclusion w;
     float4 pj[32]; // the segment's end and its source
 };
-constexpr size_t PAIR_FILL_SMEM = sizeof(PairChunk) + (PCH / 32) * sizeof(PairWarp);
-__global__ void __launch_bounds__(PCH, 3) k_pair_fill(SceneDev sc, int n, int chunks, const long long *__restrict__ chunk_off,
+constexpr size_t PAIR_FILL_SMEM = sizeof(PairChunk) + (PT / 32) * sizeof(PairWarp);
+__global__ void __launch_bounds__(PT, 6) k_pair_fill(SceneDev sc, int n, int chunks, int pch, const long long *__restrict__ chunk_off,
                                                    const float *__restrict__ lam, const float *__restrict__ aarea,
                                                    int2 *rec, int *flags) {
     extern __shared__ __align__(16) unsigned char pair_smem[];
@@ -149,30 +167,30 @@ __global__ void __launch_bounds__(PCH, 3) k_pair_fill(SceneDev sc, int n, int ch
     const int i = blk / chunks, c = blk - i * chunks;
     const float eps = *sc.eps_plane;
     const float3 pi = f3(sc.P[i]), ni = f3(sc.N4[i]);
-    float3 dv;
-    const int own = c * PCH + threadIdx.x;
-    const int total = pack_front(ck, own < n && own != i && pair_front(sc, pi, ni, own, eps, dv), own);
-    const int rank = threadIdx.x, lane = threadIdx.x & 31;
-    if (rank - lane >= total) return; // whole warps
-    const bool live = rank < total;
-    const int j = ck.j[live ? rank : rank - lane];
-    const float4 Pj = __ldg(&sc.P[j]);
-    dv = make_float3(__fsub_rn(Pj.x, pi.x), __fsub_rn(Pj.y, pi.y), __fsub_rn(Pj.z, pi.z));
-    float r, T;
-    const float3 d = unit_dir(dv, r);
-    sm.pj[lane] = make_float4(Pj.x, Pj.y, Pj.z, __int_as_float(j));
-    int nzero;
-    const bool ok = warp_transmittance(sc, sm.w, pi, d, r, i, live, eps, T, nzero, [&](int k, int ray) {
-        const float4 e = sm.pj[ray];
-        return pair_occludes(sc, k, __float_as_int(e.w), f3(e), eps);
-    });
-    if (!ok) atomicAdd(&flags[FLAG_STACK], 1);
-    if (!live) return;
-    if (nzero) T = 0.f;
-    const float3 nj = f3(sc.N4[j]);
-    const float geo = fabsf(dot3(ni, d)) * fabsf(dot3(nj, d)) / (r * r);
-    const float V = __ldg(&lam[j]) * __ldg(&aarea[j]) * T * geo;
-    rec[chunk_off[blk] + rank] = make_int2(j, __float_as_int(V));
+    const int lane = threadIdx.x & 31;
+    const int total = pack_front(ck, sc, n, i, c, pch, pi, ni, eps);
+    for (int at = threadIdx.x - lane; at < total; at += PT) { // a warp's 32 segments
+        const int rank = at + lane;
+        const bool live = rank < total;
+        const int j = ck.j[live ? rank : at];
+        const float4 Pj = __ldg(&sc.P[j]);
+        float r, T;
+        const float3 d = unit_dir(make_float3(__fsub_rn(Pj.x, pi.x), __fsub_rn(Pj.y, pi.y), __fsub_rn(Pj.z, pi.z)), r);
+        sm.pj[lane] = make_float4(Pj.x, Pj.y, Pj.z, __int_as_float(j));
+        int nzero;
+        const bool ok = warp_transmittance(sc, sm.w, pi, d, r, i, live, eps, T, nzero, [&](int k, int ray) {
+            const float4 e = sm.pj[ray];
+            return pair_occludes(sc, k, __float_as_int(e.w), f3(e), eps);
+        });
+        if (!ok) atomicAdd(&flags[FLAG_STACK], 1);
+        if (live) {
+            if (nzero) T = 0.f;
+            const float3 nj = f3(sc.N4[j]);
+            const float geo = fabsf(dot3(ni, d)) * fabsf(dot3(nj, d)) / (r * r);
+            const float V = __ldg(&lam[j]) * __ldg(&aarea[j]) * T * geo;
+            rec[chunk_off[blk] + rank] = make_int2(j, __float_as_int(V));
+        }
+    }
 }
 
 __global__ void k_pair_off(const long long *chunk_off, int chunks, int n, long long *pair_off) {
@@ -393,7 +411,7 @@ __global__ void __launch_bounds__(PAIR_THREADS) k_pair_g(SceneDev sc, int C, int
 }
 
 // Source-side gradients of every pair, laid out as the fill pass (one block per receiver
-// and 256-source chunk, the front sources packed, a lane per source):
+// and source chunk, the front sources packed, a lane per source):
 //   dL/dlambda_j += g A_j T geo,  dL/do_j += g lambda_j (A_j/o_j) T geo,
 //   dL/do_k += -g lambda_j A_j geo prod_{m != k}(1 - alpha_m) G_k for the segment's occluders.
 // T is V / (lambda_j A_j geo) from the pair's record, so the segment is traced once, for its
@@ -414,9 +432,9 @@ struct PairGeoWarp {
     float gp[32][3], gd[32][3];
 };
 template <bool GEO>
-constexpr size_t PAIR_GRAD_SMEM = sizeof(PairChunk) + (PCH / 32) * (GEO ? sizeof(PairGeoWarp) : sizeof(PairGradWarp));
+constexpr size_t PAIR_GRAD_SMEM = sizeof(PairChunk) + (PT / 32) * (GEO ? sizeof(PairGeoWarp) : sizeof(PairGradWarp));
 template <bool GEO>
-__global__ void __launch_bounds__(PCH, 2) k_pair_grad(SceneDev sc, int n, int chunks, const long long *__restrict__ chunk_off,
+__global__ void __launch_bounds__(PT, 7) k_pair_grad(SceneDev sc, int n, int chunks, int pch, const long long *__restrict__ chunk_off,
                                                    const int2 *__restrict__ rec, const float *__restrict__ lam,
                                                    const float *__restrict__ aarea, const float *__restrict__ daarea,
                                                    const float *__restrict__ gpair, const float4 *__restrict__ gq,
@@ -430,132 +448,132 @@ __global__ void __launch_bounds__(PCH, 2) k_pair_grad(SceneDev sc, int n, int ch
     const int i = blk / chunks, c = blk - i * chunks;
     const float eps = *sc.eps_plane;
     const float3 pi = f3(sc.P[i]), ni = f3(sc.N4[i]);
-    float3 dv;
-    const int own = c * PCH + threadIdx.x;
-    const int total = pack_front(ck, own < n && own != i && pair_front(sc, pi, ni, own, eps, dv), own);
-    const int rank = threadIdx.x, lane = threadIdx.x & 31;
-    if (rank - lane >= total) return; // whole warps
-    const bool have = rank < total;
-    const int j = ck.j[have ? rank : rank - lane];
-    const long long e = chunk_off[blk] + (have ? rank : rank - lane);
-    const float g = have ? gpair[e] : 0.f;
-    const float4 gs = GEO && have ? gq[e] : make_float4(0.f, 0.f, 0.f, 0.f);
-    const bool live = g != 0.f || gs.x != 0.f || gs.y != 0.f || gs.z != 0.f;
-    const float4 Pj = __ldg(&sc.P[j]);
-    dv = make_float3(__fsub_rn(Pj.x, pi.x), __fsub_rn(Pj.y, pi.y), __fsub_rn(Pj.z, pi.z));
-    float r;
-    const float3 d = unit_dir(dv, r);
-    const float3 nj = f3(sc.N4[j]);
-    const float Aj = __ldg(&aarea[j]), dAj = __ldg(&daarea[j]), lj = __ldg(&lam[j]);
-    const float nid = dot3(ni, d), njd = dot3(nj, d);
-    const float geo = fabsf(nid) * fabsf(njd) / (r * r);
-    sm.p.pj[lane] = make_float4(Pj.x, Pj.y, Pj.z, __int_as_float(j));
-    auto occ = [&](int k, int ray) {
-        const float4 x = sm.p.pj[ray];
-        return pair_occludes(sc, k, __float_as_int(x.w), f3(x), eps);
-    };
-    // T from the record; a record of (nearly) 0 says too little about it
-    const float V = __int_as_float(__ldg(&rec[e].y)), den = lj * Aj * geo;
-    const bool known = fabsf(V) > 1e-30f && fabsf(den) > 1e-30f;
-    float Tnz = known ? V / den : 0.f;
-    int nzero = 0;
-    if (__any_sync(WT_FULL, live && !known)) {
-        float T1;
-        int nz1;
-        if (!warp_transmittance(sc, sm.p.w, pi, d, r, i, live && !known, eps, T1, nz1, occ)) atomicAdd(&flags[FLAG_STACK], 1);
-        if (!known) {
-            Tnz = T1;
-            nzero = nz1;
+    const int lane = threadIdx.x & 31;
+    const int total = pack_front(ck, sc, n, i, c, pch, pi, ni, eps);
+    for (int at = threadIdx.x - lane; at < total; at += PT) { // a warp's 32 segments
+        const int rank = at + lane;
+        const bool have = rank < total;
+        const int j = ck.j[have ? rank : at];
+        const long long e = chunk_off[blk] + (have ? rank : at);
+        const float g = have ? gpair[e] : 0.f;
+        const float4 gs = GEO && have ? gq[e] : make_float4(0.f, 0.f, 0.f, 0.f);
+        const bool live = g != 0.f || gs.x != 0.f || gs.y != 0.f || gs.z != 0.f;
+        const float4 Pj = __ldg(&sc.P[j]);
+        float r;
+        const float3 d = unit_dir(make_float3(__fsub_rn(Pj.x, pi.x), __fsub_rn(Pj.y, pi.y), __fsub_rn(Pj.z, pi.z)), r);
+        const float3 nj = f3(sc.N4[j]);
+        const float Aj = __ldg(&aarea[j]), dAj = __ldg(&daarea[j]), lj = __ldg(&lam[j]);
+        const float nid = dot3(ni, d), njd = dot3(nj, d);
+        const float geo = fabsf(nid) * fabsf(njd) / (r * r);
+        sm.p.pj[lane] = make_float4(Pj.x, Pj.y, Pj.z, __int_as_float(j));
+        auto occ = [&](int k, int ray) {
+            const float4 x = sm.p.pj[ray];
+            return pair_occludes(sc, k, __float_as_int(x.w), f3(x), eps);
+        };
+        // T from the record; a record of (nearly) 0 says too little about it
+        const float V = __int_as_float(__ldg(&rec[e].y)), den = lj * Aj * geo;
+        const bool known = fabsf(V) > 1e-30f && fabsf(den) > 1e-30f;
+        float Tnz = known ? V / den : 0.f;
+        int nzero = 0;
+        if (__any_sync(WT_FULL, live && !known)) {
+            float T1;
+            int nz1;
+            if (!warp_transmittance(sc, sm.p.w, pi, d, r, i, live && !known, eps, T1, nz1, occ)) atomicAdd(&flags[FLAG_STACK], 1);
+            if (!known) {
+                Tnz = T1;
+                nzero = nz1;
+            }
         }
-    }
-    const float T = nzero ? 0.f : Tnz;
-    float3 gd = make_float3(gs.x, gs.y, gs.z), gpi = make_float3(0.f, 0.f, 0.f);
-    // the receiver's own position and normal terms are summed over the warp (all 32 lanes
-    // share receiver i) and added once per warp
-    float3 dpi = make_float3(0.f, 0.f, 0.f), gni = make_float3(0.f, 0.f, 0.f);
-    float gr = 0.f;
-    if (live) {
-        if (dlam) atomicAdd(&dlam[j], g * Aj * T * geo);
-        if (dop && T != 0.f) atomicAdd(&dop[j], g * lj * dAj * T * geo);
-        if constexpr (GEO) {
-            const float f = g * lj * Aj * T / (r * r), sj = njd >= 0.f ? 1.f : -1.f;
-            gd = gd + f * (fabsf(njd) * ni + (fabsf(nid) * sj) * nj);
-            gr = g * lj * Aj * T * (-2.f * geo / r);
-            const float fs = g * lj * T * geo * Aj;
-            geo_add2(ds + 2 * (size_t)j, fs * __ldg(&sc.FU[j].w), fs * __ldg(&sc.FV[j].w));
-            // normals through geo: d geo/d n_i = |n_j.d| d / r^2, d geo/d n_j = (n_i.d) sgn(n_j.d) d / r^2
-            const float fi = f * fabsf(njd), fj = f * fabsf(nid) * sj;
-            gni = gni + fi * d;
-            geo_add3(gF + GEO_GF * (size_t)j + GEO_N, fj * d);
+        const float T = nzero ? 0.f : Tnz;
+        float3 gd = make_float3(gs.x, gs.y, gs.z), gpi = make_float3(0.f, 0.f, 0.f);
+        // the receiver's own position and normal terms are summed over the warp (all 32 lanes
+        // share receiver i) and added once per warp
+        float3 dpi = make_float3(0.f, 0.f, 0.f), gni = make_float3(0.f, 0.f, 0.f);
+        float gr = 0.f;
+        if (live) {
+            if (dlam) atomicAdd(&dlam[j], g * Aj * T * geo);
+            if (dop && T != 0.f) atomicAdd(&dop[j], g * lj * dAj * T * geo);
+            if constexpr (GEO) {
+                const float f = g * lj * Aj * T / (r * r), sj = njd >= 0.f ? 1.f : -1.f;
+                gd = gd + f * (fabsf(njd) * ni + (fabsf(nid) * sj) * nj);
+                gr = g * lj * Aj * T * (-2.f * geo / r);
+                const float fs = g * lj * T * geo * Aj;
+                geo_add2(ds + 2 * (size_t)j, fs * __ldg(&sc.FU[j].w), fs * __ldg(&sc.FV[j].w));
+                // normals through geo: d geo/d n_i = |n_j.d| d / r^2, d geo/d n_j = (n_i.d) sgn(n_j.d) d / r^2
+                const float fi = f * fabsf(njd), fj = f * fabsf(nid) * sj;
+                gni = gni + fi * d;
+                geo_add3(gF + GEO_GF * (size_t)j + GEO_N, fj * d);
+            }
         }
-    }
-    const bool second = live && (dop || GEO) && nzero <= 1 && g != 0.f;
-    if (__any_sync(WT_FULL, second)) {
-        sm.q[lane] = -g * lj * Aj * geo;
-        sm.T[lane] = Tnz;
-        sm.nz[lane] = nzero;
-        sm.p.w.d[lane] = make_float4(d.x, d.y, d.z, r);
-        sm.p.w.own.who[lane] = 0u;
-        __syncwarp();
-        auto test = [&](int k, int ray, bool valid) {
-            bool terms = false;
-            if (valid) {
-                const float4 rd = sm.p.w.d[ray];
-                const float3 dd = f3(rd);
-                float t, gk, ok;
-                if (hit_surfel(sc, k, i, pi, dd, rd.w, eps, t, gk, ok) && occ(k, ray)) {
-                    const float om = 1.f - alpha_of(sc, ok, gk);
-                    const float others = sm.nz[ray] == 0 ? sm.T[ray] / om : (om == 0.f ? sm.T[ray] : 0.f);
-                    if (others != 0.f) {
-                        const float q = sm.q[ray];
-                        if (dop) atomicAdd(&dop[k], q * others * dalpha_do(sc, ok, gk));
-                        if constexpr (GEO) {
-                            const float coef = q * others * dalpha_dq(sc, ok, gk);
-                            if (coef != 0.f) {
-                                terms = true;
-                                float uu, vv;
-                                const float3 pw = crossing_pw(sc, k, pi, dd, t, uu, vv);
-                                smw.gp[lane][0] = coef * pw.x;
-                                smw.gp[lane][1] = coef * pw.y;
-                                smw.gp[lane][2] = coef * pw.z;
-                                smw.gd[lane][0] = (coef * t) * pw.x;
-                                smw.gd[lane][1] = (coef * t) * pw.y;
-                                smw.gd[lane][2] = (coef * t) * pw.z;
-                                geo_add3(dp + GEO_DP * (size_t)k, (-coef) * pw);
-                                geo_add2(ds + 2 * (size_t)k, coef * (-2.f * uu * uu * __ldg(&sc.FU[k].w)),
-                                         coef * (-2.f * vv * vv * __ldg(&sc.FV[k].w)));
-                                occluder_frame_grad(sc, k, pi, dd, t, uu, vv, coef, gF);
+        const bool second = live && (dop || GEO) && nzero <= 1 && g != 0.f;
+        if (__any_sync(WT_FULL, second)) {
+            sm.q[lane] = -g * lj * Aj * geo;
+            sm.T[lane] = Tnz;
+            sm.nz[lane] = nzero;
+            sm.p.w.d[lane] = make_float4(d.x, d.y, d.z, r);
+            sm.p.w.own.who[lane] = 0u;
+            __syncwarp();
+            auto test = [&](int k, int ray, bool valid) {
+                bool terms = false;
+                if (valid) {
+                    const float4 rd = sm.p.w.d[ray];
+                    const float3 dd = f3(rd);
+                    float t, gk, ok;
+                    if (hit_surfel(sc, k, i, pi, dd, rd.w, eps, t, gk, ok) && occ(k, ray)) {
+                        const float om = 1.f - alpha_of(sc, ok, gk);
+                        const float others = sm.nz[ray] == 0 ? sm.T[ray] / om : (om == 0.f ? sm.T[ray] : 0.f);
+                        if (others != 0.f) {
+                            const float q = sm.q[ray];
+                            if (dop) atomicAdd(&dop[k], q * others * dalpha_do(sc, ok, gk));
+                            if constexpr (GEO) {
+                                const float coef = q * others * dalpha_dq(sc, ok, gk);
+                                if (coef != 0.f) {
+                                    terms = true;
+                                    float uu, vv;
+                                    const float3 pw = crossing_pw(sc, k, pi, dd, t, uu, vv);
+                                    smw.gp[lane][0] = coef * pw.x;
+                                    smw.gp[lane][1] = coef * pw.y;
+                                    smw.gp[lane][2] = coef * pw.z;
+                                    smw.gd[lane][0] = (coef * t) * pw.x;
+                                    smw.gd[lane][1] = (coef * t) * pw.y;
+                                    smw.gd[lane][2] = (coef * t) * pw.z;
+                                    geo_add3(dp + GEO_DP * (size_t)k, (-coef) * pw);
+                                    geo_add2(ds + 2 * (size_t)k, coef * (-2.f * uu * uu * __ldg(&sc.FU[k].w)),
+                                             coef * (-2.f * vv * vv * __ldg(&sc.FV[k].w)));
+                                    occluder_frame_grad(sc, k, pi, dd, t, uu, vv, coef, gF);
+                                }
                             }
                         }
                     }
                 }
+                if constexpr (GEO)
+                    warp_owner_loop(sm.p.w.own, terms, ray, [&](int b) {
+                        gpi = gpi + make_float3(smw.gp[b][0], smw.gp[b][1], smw.gp[b][2]);
+                        gd = gd + make_float3(smw.gd[b][0], smw.gd[b][1], smw.gd[b][2]);
+                    });
+            };
+            if (!warp_traverse<false>(sc, pi, d, r, second, sm.p.w.q, test, [](float m) { return m; })) atomicAdd(&flags[FLAG_STACK], 1);
+        }
+        if constexpr (GEO) {
+            if (live) {
+                const float dd = dot3(d, gd);
+                const float3 gp = make_float3((gd.x - d.x * dd) / r + d.x * gr, (gd.y - d.y * dd) / r + d.y * gr,
+                                              (gd.z - d.z * dd) / r + d.z * gr);
+                geo_add3(dp + GEO_DP * (size_t)j, gp);
+                dpi = gpi - gp;
             }
-            if constexpr (GEO)
-                warp_owner_loop(sm.p.w.own, terms, ray, [&](int b) {
-                    gpi = gpi + make_float3(smw.gp[b][0], smw.gp[b][1], smw.gp[b][2]);
-                    gd = gd + make_float3(smw.gd[b][0], smw.gd[b][1], smw.gd[b][2]);
-                });
-        };
-        if (!warp_traverse<false>(sc, pi, d, r, second, sm.p.w.q, test, [](float m) { return m; })) atomicAdd(&flags[FLAG_STACK], 1);
-    }
-    if constexpr (!GEO) return;
-    if (live) {
-        const float dd = dot3(d, gd);
-        const float3 gp = make_float3((gd.x - d.x * dd) / r + d.x * gr, (gd.y - d.y * dd) / r + d.y * gr,
-                                      (gd.z - d.z * dd) / r + d.z * gr);
-        geo_add3(dp + GEO_DP * (size_t)j, gp);
-        dpi = gpi - gp;
-    }
-    float red[6] = {dpi.x, dpi.y, dpi.z, gni.x, gni.y, gni.z};
+            float red[6] = {dpi.x, dpi.y, dpi.z, gni.x, gni.y, gni.z};
 #pragma unroll
-    for (int q = 0; q < 6; ++q)
+            for (int q = 0; q < 6; ++q)
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) red[q] += __shfl_xor_sync(0xffffffffu, red[q], off);
-    if (lane == 0) {
+                for (int off = 16; off > 0; off >>= 1) red[q] += __shfl_xor_sync(0xffffffffu, red[q], off);
+            if (lane == 0) {
 #pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            if (red[q] != 0.f) atomicAdd(&dp[GEO_DP * (size_t)i + q], red[q]);
-            if (red[3 + q] != 0.f) atomicAdd(&gF[GEO_GF * (size_t)i + GEO_N + q], red[3 + q]);
+                for (int q = 0; q < 3; ++q) {
+                    if (red[q] != 0.f) atomicAdd(&dp[GEO_DP * (size_t)i + q], red[q]);
+                    if (red[3 + q] != 0.f) atomicAdd(&gF[GEO_GF * (size_t)i + GEO_N + q], red[3 + q]);
+                }
+            }
         }
     }
 }
@@ -618,7 +636,7 @@ rgs_status rgs_trace_pairs_impl(rgs_transport *t, const rgs_lights *L, const flo
     t->nd = 0;
     if ((r = rgs_transport_common(t, L, st)) != RGS_OK) return r;
     const int n = t->n;
-    const int chunks = (n + PCH - 1) / PCH;
+    const int pch = pair_chunk(n), chunks = (n + pch - 1) / pch;
     const long long nchunk = (long long)n * chunks;
     if (nchunk >= (1ll << 31)) {
         rgs_set_error("rgs_trace_pairs: %d surfels give too many (receiver, source-chunk) blocks", n);
@@ -643,7 +661,7 @@ rgs_status rgs_trace_pairs_impl(rgs_transport *t, const rgs_lights *L, const flo
     { ProfScope ps_("k_alpha_area", st); k_alpha_area<<<(n + 255) / 256, 256, 0, st>>>(sd, t->aarea, t->daarea); }
     RGS_CUDA(cudaMemsetAsync(t->flags, 0, sizeof(int) * FLAG_COUNT, st));
     RGS_CUDA(cudaMemsetAsync(t->src_cnt, 0, sizeof(int) * n, st));
-    { ProfScope ps_("k_pair_count", st); k_pair_count<<<(unsigned)nchunk, PCH, 0, st>>>(sd, n, chunks, t->chunk_cnt, t->src_cnt); }
+    { ProfScope ps_("k_pair_count", st); k_pair_count<<<(unsigned)nchunk, pch, 0, st>>>(sd, n, chunks, t->chunk_cnt, t->src_cnt); }
     RGS_LAUNCH("pair count");
     if ((r = rgs_scan_counts(t->chunk_cnt, t->chunk_off, (int)nchunk, t->chunk_tmp, t->chunk_tmp_cap, st)) != RGS_OK)
         return r;
@@ -659,7 +677,7 @@ rgs_status rgs_trace_pairs_impl(rgs_transport *t, const rgs_lights *L, const flo
     t->n_slots = total;
     t->n_full = 0;
     RGS_CUDA(cudaFuncSetAttribute(k_pair_fill, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PAIR_FILL_SMEM));
-    { ProfScope ps_("k_pair_fill", st); k_pair_fill<<<(unsigned)nchunk, PCH, PAIR_FILL_SMEM, st>>>(sd, n, chunks, t->chunk_off, t->lam, t->aarea, t->pair_rec, t->flags); }
+    { ProfScope ps_("k_pair_fill", st); k_pair_fill<<<(unsigned)nchunk, PT, PAIR_FILL_SMEM, st>>>(sd, n, chunks, pch, t->chunk_off, t->lam, t->aarea, t->pair_rec, t->flags); }
     { ProfScope ps_("k_pair_off", st); k_pair_off<<<(n + 256) / 256, 256, 0, st>>>(t->chunk_off, chunks, n, t->pair_off); }
     RGS_LAUNCH("pair fill");
     if ((r = rgs_direct_term(t, st)) != RGS_OK) return r;
@@ -731,7 +749,7 @@ rgs_status run_adjoint_pairs(rgs_transport *t, const float *g, float *dE, float 
     }
     if ((r = rgs_shadow_backward(t, NC, st, geo.dp, geo.ds, geo.gF)) != RGS_OK) return r;
     if (nb >= 1 && (dopo || dlam_acc || geo.dp)) {
-        const int chunks = (n + PCH - 1) / PCH;
+        const int pch = pair_chunk(n), chunks = (n + pch - 1) / pch;
         if (geo.dp) {
             ProfScope ps_("k_pair_g", st);
             k_pair_g<NC, true><<<n, PAIR_THREADS, 0, st>>>(sd, C, nb, t->pair_off, t->pair_rec, A, t->v, t->iters, t->gh, geo.gq, geo.gF);
@@ -742,11 +760,11 @@ rgs_status run_adjoint_pairs(rgs_transport *t, const float *g, float *dE, float 
         if (geo.dp) {
             RGS_CUDA(cudaFuncSetAttribute(k_pair_grad<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PAIR_GRAD_SMEM<true>));
             ProfScope ps_("k_pair_grad", st);
-            k_pair_grad<true><<<(unsigned)((long long)n * chunks), PCH, PAIR_GRAD_SMEM<true>, st>>>(sd, n, chunks, t->chunk_off, t->pair_rec, t->lam, t->aarea, t->daarea, t->gh, geo.gq, dopo ? t->dop : nullptr, dlam_acc, geo.dp, geo.ds, geo.gF, t->flags);
+            k_pair_grad<true><<<(unsigned)((long long)n * chunks), PT, PAIR_GRAD_SMEM<true>, st>>>(sd, n, chunks, pch, t->chunk_off, t->pair_rec, t->lam, t->aarea, t->daarea, t->gh, geo.gq, dopo ? t->dop : nullptr, dlam_acc, geo.dp, geo.ds, geo.gF, t->flags);
         } else {
             RGS_CUDA(cudaFuncSetAttribute(k_pair_grad<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PAIR_GRAD_SMEM<false>));
             ProfScope ps_("k_pair_grad", st);
-            k_pair_grad<false><<<(unsigned)((long long)n * chunks), PCH, PAIR_GRAD_SMEM<false>, st>>>(sd, n, chunks, t->chunk_off, t->pair_rec, t->lam, t->aarea, t->daarea, t->gh, nullptr, dopo ? t->dop : nullptr, dlam_acc, nullptr, nullptr, nullptr, t->flags);
+            k_pair_grad<false><<<(unsigned)((long long)n * chunks), PT, PAIR_GRAD_SMEM<false>, st>>>(sd, n, chunks, pch, t->chunk_off, t->pair_rec, t->lam, t->aarea, t->daarea, t->gh, nullptr, dopo ? t->dop : nullptr, dlam_acc, nullptr, nullptr, nullptr, t->flags);
         }
         RGS_LAUNCH("pair backward");
     }

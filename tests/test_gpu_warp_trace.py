@@ -45,6 +45,42 @@ def test_small_trees(n, pairs):
     _check(scenes.random_cluster(n=n, seed=n, L=2, nd=32, nb=2, n_lights=2), pairs)
 
 
+@pytest.mark.parametrize("n", [255, 256, 513])
+def test_pairs_source_chunks(n):
+    """Blocks of 256 sources, full and with one over."""
+    _check(scenes.random_cluster(n=n, seed=n, L=1, nd=32, nb=1, n_lights=1), True)
+
+
+@pytest.mark.parametrize("n", [2048, 2561])
+def test_pairs_large_source_chunks(n):
+    """Blocks of 512 sources: surfels of opacity 0 inside the cloud change nothing for the others."""
+    m = 150
+    sc = scenes.with_emission(scenes.random_cluster(n=m, seed=7, L=1, nd=32, nb=2, n_lights=1), seed=3)
+    W = np.random.default_rng(2).normal(size=(m, 4, 3))
+    o = run_oracle(sc, W=W, pairs=True)
+    rng = np.random.default_rng(n)
+    src = rng.integers(0, m, size=n - m)
+    big = dict(sc, n=n)
+    for key, v in sc.items():
+        if isinstance(v, np.ndarray) and v.ndim and v.shape[0] == m:
+            big[key] = np.concatenate([v, v[src]])
+    lo, hi = sc["p"].min(0), sc["p"].max(0)
+    big["p"][m:] = (lo + (hi - lo) * rng.uniform(0.3, 0.7, size=(n - m, 3))).astype(np.float32)
+    big["s"][m:] *= 0.1
+    big["o"][m:] = 0.0
+    big["E"][m:] = 0.0
+    at = rng.permutation(n)  # the caller's order mixes the two
+    for key, v in big.items():
+        if isinstance(v, np.ndarray) and v.ndim and v.shape[0] == n:
+            big[key] = v[at]
+    real = np.argsort(at)[:m]
+    Wb = np.zeros((n, 4, 3))
+    Wb[real] = W
+    g = run_gpu(big, W=Wb, pairs=True)
+    for key in ("B", "dE", "dad", "dop", "dlam"):
+        assert rel_l2(g[key][real], o[key]) <= TOL, (key, rel_l2(g[key][real], o[key]))
+
+
 def _overlapping(n, o_lo, o_hi, seed=5):
     """A cloud whose surfels all cover each other: about half of them on every ray."""
     sc = scenes.random_cluster(n=n, seed=seed, L=1, nd=32, nb=2, n_lights=1)
