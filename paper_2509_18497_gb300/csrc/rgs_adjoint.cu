@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(SHADOW_THREADS) k_shadow_bwd(SceneDev sc, int 
     const float eps = *sc.eps_plane;
     float Tnz;
     int nzero;
-    warp_transmittance(sc, sm.w, o, w, r, i, lit, eps, Tnz, nzero, [](int, int) { return true; });
+    warp_transmittance<false>(sc, sm.w, o, w, r, i, lit, eps, Tnz, nzero, [](int, const SurfelRec &, int) { return true; });
     float qv = 0.f, H = 0.f;
     const float T = nzero ? 0.f : Tnz;
     float3 gw = make_float3(0.f, 0.f, 0.f), gpi = make_float3(0.f, 0.f, 0.f);

@@ -464,13 +464,10 @@ __device__ __forceinline__ float plane_den(const SurfelRec &s, float3 d) {
     return __fmaf_rn(s.N.z, d.z, __fmaf_rn(s.N.y, d.y, __fmul_rn(s.N.x, d.x)));
 }
 
-// Ray o + t d against the plane of surfel j (Eq. G). Returns true with t and r2 when the
-// hit is accepted: j != self, |n_j.(p_j - o)| > eps, 0 < t < tmax, inside the cutoff; op is
-// then its opacity parameter.
-__device__ __forceinline__ bool hit_surfel_t(const SceneDev &sc, int j, int self, float3 o, float3 d, float tmax,
-                                             float eps, float &t_out, float &r2_out, float &op) {
-    if (j == self) return false;
-    const SurfelRec s = ld_surfel(sc, j);
+// Ray o + t d against the plane of a surfel (Eq. G). Returns true with t and r2 when the
+// hit is accepted: |n_j.(p_j - o)| > eps, 0 < t < tmax, inside the cutoff.
+__device__ __forceinline__ bool hit_rec(const SceneDev &sc, const SurfelRec &s, float3 o, float3 d, float tmax, float eps,
+                                        float &t_out, float &r2_out) {
     const float den = plane_den(s, d);
     if (fabsf(den) < 1e-12f) return false;
     const float h = plane_h(s, o);
@@ -481,8 +478,15 @@ __device__ __forceinline__ bool hit_surfel_t(const SceneDev &sc, int j, int self
     if (r2 > sc.cutoff2) return false;
     t_out = t;
     r2_out = r2;
-    op = s.P.w;
     return true;
+}
+// the same for surfel j of the scene, unless it is the ray's own; op: its opacity parameter
+__device__ __forceinline__ bool hit_surfel_t(const SceneDev &sc, int j, int self, float3 o, float3 d, float tmax,
+                                             float eps, float &t_out, float &r2_out, float &op) {
+    if (j == self) return false;
+    const SurfelRec s = ld_surfel(sc, j);
+    op = s.P.w;
+    return hit_rec(sc, s, o, d, tmax, eps, t_out, r2_out);
 }
 
 // t, u^2 + v^2 and the opacity parameter of a hit that the trace has accepted (ray o + t d on

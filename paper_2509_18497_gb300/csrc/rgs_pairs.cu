@@ -98,12 +98,8 @@ __device__ __forceinline__ float3 unit_dir(float3 dv, float &r) {
 
 // a hit on surfel k of the segment i -> j occludes it if k is not the source and k's plane is
 // more than eps from the source's centre
-__device__ __forceinline__ bool pair_occludes(const SceneDev &sc, int k, int j, float3 pj, float eps) {
-    if (k == j) return false;
-    const float4 Nk = __ldg(&sc.N4[k]);
-    const float4 Pk = __ldg(&sc.P[k]);
-    const float e = Nk.x * (pj.x - Pk.x) + Nk.y * (pj.y - Pk.y) + Nk.z * (pj.z - Pk.z);
-    return fabsf(e) > eps;
+__device__ __forceinline__ bool pair_occludes(int k, const SurfelRec &s, int j, float3 pj, float eps) {
+    return k != j && fabsf(plane_h(s, pj)) > eps;
 }
 
 // The front sources of a (receiver, source chunk) block in increasing order, packed: the
@@ -178,9 +174,9 @@ __global__ void __launch_bounds__(PT, 6) k_pair_fill(SceneDev sc, int n, int chu
         const float3 d = unit_dir(make_float3(__fsub_rn(Pj.x, pi.x), __fsub_rn(Pj.y, pi.y), __fsub_rn(Pj.z, pi.z)), r);
         sm.pj[lane] = make_float4(Pj.x, Pj.y, Pj.z, __int_as_float(j));
         int nzero;
-        const bool ok = warp_transmittance(sc, sm.w, pi, d, r, i, live, eps, T, nzero, [&](int k, int ray) {
+        const bool ok = warp_transmittance<true>(sc, sm.w, pi, d, r, i, live, eps, T, nzero, [&](int k, const SurfelRec &s, int ray) {
             const float4 e = sm.pj[ray];
-            return pair_occludes(sc, k, __float_as_int(e.w), f3(e), eps);
+            return pair_occludes(k, s, __float_as_int(e.w), f3(e), eps);
         });
         if (!ok) atomicAdd(&flags[FLAG_STACK], 1);
         if (live) {
@@ -466,9 +462,9 @@ __global__ void __launch_bounds__(PT, 7) k_pair_grad(SceneDev sc, int n, int chu
         const float nid = dot3(ni, d), njd = dot3(nj, d);
         const float geo = fabsf(nid) * fabsf(njd) / (r * r);
         sm.p.pj[lane] = make_float4(Pj.x, Pj.y, Pj.z, __int_as_float(j));
-        auto occ = [&](int k, int ray) {
+        auto occ = [&](int k, const SurfelRec &s, int ray) {
             const float4 x = sm.p.pj[ray];
-            return pair_occludes(sc, k, __float_as_int(x.w), f3(x), eps);
+            return pair_occludes(k, s, __float_as_int(x.w), f3(x), eps);
         };
         // T from the record; a record of (nearly) 0 says too little about it
         const float V = __int_as_float(__ldg(&rec[e].y)), den = lj * Aj * geo;
@@ -478,7 +474,7 @@ __global__ void __launch_bounds__(PT, 7) k_pair_grad(SceneDev sc, int n, int chu
         if (__any_sync(WT_FULL, live && !known)) {
             float T1;
             int nz1;
-            if (!warp_transmittance(sc, sm.p.w, pi, d, r, i, live && !known, eps, T1, nz1, occ)) atomicAdd(&flags[FLAG_STACK], 1);
+            if (!warp_transmittance<true>(sc, sm.p.w, pi, d, r, i, live && !known, eps, T1, nz1, occ)) atomicAdd(&flags[FLAG_STACK], 1);
             if (!known) {
                 Tnz = T1;
                 nzero = nz1;
@@ -515,11 +511,13 @@ __global__ void __launch_bounds__(PT, 7) k_pair_grad(SceneDev sc, int n, int chu
             __syncwarp();
             auto test = [&](int k, int ray, bool valid) {
                 bool terms = false;
-                if (valid) {
+                if (valid && k != i) {
                     const float4 rd = sm.p.w.d[ray];
                     const float3 dd = f3(rd);
-                    float t, gk, ok;
-                    if (hit_surfel(sc, k, i, pi, dd, rd.w, eps, t, gk, ok) && occ(k, ray)) {
+                    const SurfelRec s = ld_surfel(sc, k);
+                    float t, r2;
+                    if (hit_rec(sc, s, pi, dd, rd.w, eps, t, r2) && occ(k, s, ray)) {
+                        const float gk = surfel_G(sc, r2), ok = s.P.w;
                         const float om = 1.f - alpha_of(sc, ok, gk);
                         const float others = sm.nz[ray] == 0 ? sm.T[ray] / om : (om == 0.f ? sm.T[ray] : 0.f);
                         if (others != 0.f) {

@@ -120,8 +120,8 @@ __global__ void __launch_bounds__(DIRECT_THREADS) k_direct(SceneDev sc, int nl, 
     const bool lit = live && cs > 0.f;
     float T;
     int nzero;
-    if (!warp_transmittance(sc, sm[threadIdx.x >> 5], o, w, r, i, lit, *sc.eps_plane, T, nzero,
-                            [](int, int) { return true; }))
+    if (!warp_transmittance<false>(sc, sm[threadIdx.x >> 5], o, w, r, i, lit, *sc.eps_plane, T, nzero,
+                            [](int, const SurfelRec &, int) { return true; }))
         atomicAdd(&flags[FLAG_STACK], 1);
     if (!live) return;
     float *Dout = D + ((size_t)i * C + lt * 3) * NC;

@@ -157,14 +157,14 @@ struct __align__(16) WarpOcclusion {
     WarpOwners own;
 };
 // T = prod (1 - alpha_k) over the surfels k that the lane's ray (o, d, t < tmax, not `self`)
-// meets, the factors that are exactly 0 counted in nzero instead; occluder(k, lane of the ray)
-// may reject a hit.  All lanes call.
-template <class Occ>
+// meets, the factors that are exactly 0 counted in nzero instead; occluder(surfel, its record,
+// lane of the ray) may reject a hit.  ONE: all rays have this origin and own surfel.  All lanes call.
+template <bool ONE, class Occ>
 __device__ __forceinline__ bool warp_transmittance(const SceneDev &sc, WarpOcclusion &s, float3 o, float3 d, float tmax,
                                                    int self, bool active, float eps, float &T, int &nzero,
                                                    Occ &&occluder) {
     const int lane = threadIdx.x & 31;
-    s.o[lane] = make_float4(o.x, o.y, o.z, __int_as_float(self));
+    if constexpr (!ONE) s.o[lane] = make_float4(o.x, o.y, o.z, __int_as_float(self));
     s.d[lane] = make_float4(d.x, d.y, d.z, tmax);
     s.own.who[lane] = 0u;
     T = 1.f;
@@ -172,11 +172,13 @@ __device__ __forceinline__ bool warp_transmittance(const SceneDev &sc, WarpOcclu
     __syncwarp();
     auto test = [&](int k, int ray, bool valid) {
         bool hit = false;
-        if (valid) {
-            const float4 ro = s.o[ray], rd = s.d[ray];
-            float t, g, op;
-            hit = hit_surfel(sc, k, __float_as_int(ro.w), f3(ro), f3(rd), rd.w, eps, t, g, op) && occluder(k, ray);
-            if (hit) s.om[lane] = 1.f - alpha_of(sc, op, g);
+        const float4 ro = ONE ? make_float4(o.x, o.y, o.z, __int_as_float(self)) : s.o[ray];
+        if (valid && k != __float_as_int(ro.w)) {
+            const float4 rd = s.d[ray];
+            const SurfelRec rec = ld_surfel(sc, k);
+            float t, r2;
+            hit = hit_rec(sc, rec, f3(ro), f3(rd), rd.w, eps, t, r2) && occluder(k, rec, ray);
+            if (hit) s.om[lane] = 1.f - alpha_of(sc, rec.P.w, surfel_G(sc, r2));
         }
         warp_owner_loop(s.own, hit, ray, [&](int b) {
             const float om = s.om[b];
