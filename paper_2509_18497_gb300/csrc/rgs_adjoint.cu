@@ -116,31 +116,94 @@ __global__ void __launch_bounds__(256) k_adj_ray(SceneDev sc, RaysDev rays, int 
 
 // (K^T v)_j[c][k] = sum_{entries e on j} a_e Y_k(-d_e) y_e[c]; one CTA per source j.
 // 3 columns: a thread per entry.
-template <int NC>
+// OPA: the opacity backward's per-hit sums as well, which need the same two things of an entry,
+//   g_e (+)= sum_c y_e[c] Y(-d_e) . B_j[c],
+// B the iterate paired with v.  By source its row is read once per CTA; the ray-wise gather
+// reads a row per hit, at the ~10 TB/s the L2 gives (192 bytes a hit and iterate for 3 FP32
+// columns, 1.5 KB for 48 BF16 ones).  Both passes, 20,000 surfels, 128 rays, 16 coefficients,
+// three pairings: 3 columns 4.2 -> 1.7 ms, 12 columns 15.3 -> 4.9; 60,000 surfels, 48 BF16
+// columns, four pairings: 104 -> 66 ms.
+struct AdjOpa {
+    const float *Bf;         // B^(b), FP32 rows
+    const __nv_bfloat16 *Bh; // its BF16 rows (the batched modes), or NULL
+    float *gt;               // per entry of the index
+    bool first;              // write instead of add
+};
+template <int NC> __device__ __forceinline__ float adj_opa_row(const AdjOpa &o, size_t jc, int k) {
+    return o.Bh ? __bfloat162float(o.Bh[jc * bf16_stride<NC>() + k]) : __ldg(&o.Bf[jc * NC + k]);
+}
+template <int NC, bool OPA>
 __global__ void RGS_ADJ_LB k_adj_src(int C, int col0, const long long *__restrict__ src_off,
                                                         const int2 *__restrict__ tr, const float *__restrict__ rec,
                                                         float *__restrict__ vout, float *__restrict__ u, int j0,
-                                                        long long ebase) {
+                                                        long long ebase, AdjOpa opa) {
     constexpr int CT = 3, RS = adj_rec<CT>();
     const int j = j0 + blockIdx.x; // sources j0 .. of this index part; its entries start at ebase
+    constexpr int NQ = (NC + 3) / 4;
+    __shared__ float4 Bj[OPA ? CT * NQ : 1];
+    if constexpr (OPA) {
+        if (threadIdx.x < CT * NQ * 4) {
+            const int c = threadIdx.x / (NQ * 4), k = threadIdx.x % (NQ * 4);
+            reinterpret_cast<float *>(Bj)[threadIdx.x] = k < NC ? adj_opa_row<NC>(opa, (size_t)j * C + col0 + c, k) : 0.f;
+        }
+        __syncthreads();
+    }
     float acc[NC][CT];
 #pragma unroll
     for (int k = 0; k < NC; ++k)
 #pragma unroll
         for (int c = 0; c < CT; ++c) acc[k][c] = 0.f;
     const long long e0 = src_off[j] - ebase, e1 = src_off[j + 1] - ebase;
-    for (long long e = e0 + threadIdx.x; e < e1; e += ADJ_THREADS) {
-        const int2 ent = __ldg(&tr[e]);
-        const float a = __int_as_float(ent.y);
-        float4 d4, y4;
+    // the next entry's record and sum are requested before this one is worked on, the entry
+    // after it before that
+    auto entry = [&](long long e) { return e < e1 ? __ldg(&tr[e]) : make_int2(0, 0); };
+    long long e = e0 + threadIdx.x;
+    int2 ent = entry(e), ent1 = entry(e + ADJ_THREADS);
+    float4 d4 = make_float4(0.f, 0.f, 0.f, 0.f), y4 = d4;
+    float old = 0.f, old1 = 0.f;
+    if (e < e1) {
         ld_rec32(rec + (size_t)ent.x * RS, d4, y4);
+        if (OPA && !opa.first) old = opa.gt[e];
+    }
+    for (; e < e1; e += ADJ_THREADS) {
+        const float a = __int_as_float(ent.y);
+        const long long en = e + ADJ_THREADS;
+        float4 d41 = d4, y41 = y4;
+        if (en < e1) {
+            ld_rec32(rec + (size_t)ent1.x * RS, d41, y41);
+            if (OPA && !opa.first) old1 = opa.gt[en];
+        }
+        const int2 ent2 = entry(en + ADJ_THREADS);
         float Yo[NC];
         sh_eval<NC>(make_float3(-d4.x, -d4.y, -d4.z), Yo);
+        if constexpr (OPA) {
+            const float yc[3] = {y4.x, y4.y, y4.z};
+            float g = old;
+#pragma unroll
+            for (int c = 0; c < CT; ++c) {
+                float t = 0.f;
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) {
+                    const float4 b = Bj[c * NQ + q];
+                    const float bk[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        if (4 * q + k < NC) t += Yo[4 * q + k < NC ? 4 * q + k : 0] * bk[k];
+                }
+                g += yc[c] * t;
+            }
+            opa.gt[e] = g;
+        }
         const float y[3] = {a * y4.x, a * y4.y, a * y4.z};
 #pragma unroll
         for (int k = 0; k < NC; ++k)
 #pragma unroll
             for (int c = 0; c < CT; ++c) acc[k][c] += Yo[k] * y[c];
+        ent = ent1;
+        ent1 = ent2;
+        d4 = d41;
+        y4 = y41;
+        old = old1;
     }
     __shared__ float red[ADJ_THREADS / 32][NC * CT];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -167,7 +230,9 @@ __global__ void RGS_ADJ_LB k_adj_src(int C, int col0, const long long *__restric
 // 12 columns: the entries' records are copied into shared memory 128 at a time (asynchronously,
 // the next batch while this one is used: their latency, not the arithmetic, is what bounds
 // the gather), a thread evaluates the SH of one entry, and G lanes per entry, each KPL
-// coefficients, multiply: 48 FMAs per 4 shared-memory reads.  60,000 surfels, 128 rays, 48
+// coefficients, multiply: 48 FMAs (two to an instruction) per 4 shared-memory reads, 108 with the
+// opacity sums (OPA), whose partial results are copied ahead with the records (read where they
+// are added to, the 12-column pass took 86 ms for 66).  60,000 surfels, 128 rays, 48
 // columns: 1.78 ms a launch (an entry per thread at 3 columns: 1.1 ms for a quarter of them).
 constexpr int ADJ_STRIDE = 20; // floats of a record in shared memory (16-byte rows without conflicts)
 template <int NC> struct AdjLanes {
@@ -175,34 +240,50 @@ template <int NC> struct AdjLanes {
 };
 template <int NC> struct AdjTile {
     __align__(16) float rec[2][ADJ_THREADS][ADJ_STRIDE];
-    __align__(16) float Y[ADJ_THREADS][ADJ_STRIDE]; // a Y(-d)
-    float a[2][ADJ_THREADS];
+    __align__(16) float Y[ADJ_THREADS][ADJ_STRIDE]; // Y(-d)
+    float a[2][ADJ_THREADS], g[2][ADJ_THREADS]; // weights; opacity sums so far
 };
 __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src));
 }
-template <int NC>
-__global__ void __launch_bounds__(ADJ_THREADS, 7) k_adj_src_tile(int C, int col0, const long long *__restrict__ src_off,
+__device__ __forceinline__ void cp_async4(void *dst, const void *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src));
+}
+template <int NC, bool OPA>
+__global__ void __launch_bounds__(ADJ_THREADS, OPA ? 4 : 6) k_adj_src_tile(int C, int col0, const long long *__restrict__ src_off,
                                                                const int2 *__restrict__ tr, const float *__restrict__ rec,
                                                                float *__restrict__ vout, float *__restrict__ u, int j0,
-                                                               long long ebase) {
+                                                               long long ebase, AdjOpa opa) {
     constexpr int CT = 12, RS = adj_rec<CT>(), G = AdjLanes<NC>::G, KPL = AdjLanes<NC>::KPL;
     __shared__ AdjTile<NC> s;
     const int j = j0 + blockIdx.x;
     const int tid = threadIdx.x, lane = tid & 31, g = tid % G;
-    float acc[KPL][CT];
+    constexpr int CP = CT / 2; // pairs of columns
+    uint64_t acc[KPL][CP];
 #pragma unroll
     for (int k = 0; k < KPL; ++k)
 #pragma unroll
-        for (int c = 0; c < CT; ++c) acc[k][c] = 0.f;
+        for (int c = 0; c < CP; ++c) acc[k][c] = 0ull;
+    uint64_t Bj[OPA ? CP : 1][OPA ? KPL : 1]; // this lane's coefficients of the source's paired row
+    if constexpr (OPA) {
+        auto el = [&](int c, int k) {
+            return col0 + c < C && KPL * g + k < NC ? adj_opa_row<NC>(opa, (size_t)j * C + col0 + c, KPL * g + k) : 0.f;
+        };
+#pragma unroll
+        for (int c = 0; c < CP; ++c)
+#pragma unroll
+            for (int k = 0; k < KPL; ++k) Bj[c][k] = pack2(el(2 * c, k), el(2 * c + 1, k));
+    }
     const long long e0 = src_off[j] - ebase, e1 = src_off[j + 1] - ebase;
     const int batches = (int)((e1 - e0 + ADJ_THREADS - 1) / ADJ_THREADS);
     auto entry = [&](int b) { // this thread's entry of batch b (ray -1: none)
         const long long e = e0 + (long long)b * ADJ_THREADS + tid;
         return e < e1 ? __ldg(&tr[e]) : make_int2(-1, 0);
     };
-    auto fetch = [&](int st, int2 ent) { // four lanes copy a record
+    auto fetch = [&](int b, int2 ent) { // batch b: four lanes copy a record
+        const int st = b & 1;
         s.a[st][tid] = __int_as_float(ent.y);
+        if (OPA && !opa.first && ent.x >= 0) cp_async4(&s.g[st][tid], opa.gt + e0 + (long long)b * ADJ_THREADS + tid);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int from = 8 * q + (lane >> 2), ray = __shfl_sync(0xffffffffu, ent.x, from);
@@ -217,7 +298,7 @@ __global__ void __launch_bounds__(ADJ_THREADS, 7) k_adj_src_tile(int C, int col0
     for (int b = 0; b < batches; ++b) {
         const int st = b & 1;
         if (b + 1 < batches) {
-            fetch(st ^ 1, ent);
+            fetch(b + 1, ent);
             ent = entry(b + 2);
             asm volatile("cp.async.wait_group 1;");
         } else {
@@ -227,30 +308,53 @@ __global__ void __launch_bounds__(ADJ_THREADS, 7) k_adj_src_tile(int C, int col0
         const int m = (int)min((long long)ADJ_THREADS, e1 - e0 - (long long)b * ADJ_THREADS);
         if (tid < m) {
             const float4 d = *reinterpret_cast<const float4 *>(s.rec[st][tid]);
-            const float a = s.a[st][tid];
             float Yo[NC];
             sh_eval<NC>(make_float3(-d.x, -d.y, -d.z), Yo);
 #pragma unroll
-            for (int k = 0; k < G * KPL; ++k) s.Y[tid][k] = k < NC ? a * Yo[k < NC ? k : 0] : 0.f;
+            for (int k = 0; k < G * KPL; ++k) s.Y[tid][k] = k < NC ? Yo[k < NC ? k : 0] : 0.f;
         }
         __syncthreads();
-#pragma unroll 2
-        for (int x = tid / G; x < m; x += ADJ_THREADS / G) {
-            float w[KPL], y[CT];
+        const int rounds = (m + ADJ_THREADS / G - 1) / (ADJ_THREADS / G); // (all lanes: OPA sums over a group's)
+#pragma unroll 1
+        for (int q0 = 0; q0 < rounds; ++q0) {
+            const int at = q0 * (ADJ_THREADS / G) + tid / G, x = min(at, m - 1);
+            if (!OPA && at >= m) break;
+            float w[KPL];
+            uint64_t y[CP];
 #pragma unroll
             for (int k = 0; k < KPL; ++k) w[k] = s.Y[x][KPL * g + k];
 #pragma unroll
             for (int q = 0; q < CT / 4; ++q) {
-                const float4 f = *reinterpret_cast<const float4 *>(&s.rec[st][x][4 + 4 * q]);
-                y[4 * q] = f.x;
-                y[4 * q + 1] = f.y;
-                y[4 * q + 2] = f.z;
-                y[4 * q + 3] = f.w;
+                const ulonglong2 f = *reinterpret_cast<const ulonglong2 *>(&s.rec[st][x][4 + 4 * q]);
+                y[2 * q] = f.x;
+                y[2 * q + 1] = f.y;
             }
+            if constexpr (OPA) {
+                uint64_t t2 = 0ull, w2[KPL];
 #pragma unroll
-            for (int k = 0; k < KPL; ++k)
+                for (int k = 0; k < KPL; ++k) w2[k] = pack2(w[k], w[k]);
 #pragma unroll
-                for (int c = 0; c < CT; ++c) acc[k][c] += w[k] * y[c];
+                for (int c = 0; c < CP; ++c) {
+                    uint64_t sc = 0ull;
+#pragma unroll
+                    for (int k = 0; k < KPL; ++k) sc = fma2(w2[k], Bj[c][k], sc);
+                    t2 = fma2(y[c], sc, t2);
+                }
+                const float2 tt = unpack2(t2);
+                float t = tt.x + tt.y;
+#pragma unroll
+                for (int off = 1; off < G; off <<= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+                if (g == 0 && at < m)
+                    opa.gt[e0 + (long long)b * ADJ_THREADS + x] = opa.first ? t : s.g[st][x] + t;
+                if (at >= m) break;
+            }
+            const float a = s.a[st][x];
+#pragma unroll
+            for (int k = 0; k < KPL; ++k) {
+                const uint64_t aw = pack2(a * w[k], a * w[k]);
+#pragma unroll
+                for (int c = 0; c < CP; ++c) acc[k][c] = fma2(aw, y[c], acc[k][c]);
+            }
         }
         __syncthreads(); // the tables are rewritten
     }
@@ -261,7 +365,8 @@ __global__ void __launch_bounds__(ADJ_THREADS, 7) k_adj_src_tile(int C, int col0
     for (int k = 0; k < KPL; ++k)
 #pragma unroll
         for (int c = 0; c < CT; ++c) {
-            float v = acc[k][c];
+            const float2 two = unpack2(acc[k][c / 2]);
+            float v = c & 1 ? two.y : two.x;
 #pragma unroll
             for (int off = 16; off >= G; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
             if (lane < G) red[(tid >> 5) * OUT + (KPL * lane + k) * CT + c] = v;
@@ -768,7 +873,7 @@ __global__ void __launch_bounds__(32 * ROW_WARPS) k_finalize(SceneDev sc, int C,
 // transposed index: the records of every ray on a source j0 <= j < j1 scattered into
 // per-source lists of (ray, a), stored from entry ebase = src_off[j0] on
 __global__ void k_src_fill(RaysDev rays, int n_rays, unsigned long long *cursor, int2 *tr, int j0, int j1,
-                           long long ebase) {
+                           long long ebase, unsigned *entry) {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= n_rays) return;
     const long long base = rays.off[r];
@@ -778,6 +883,15 @@ __global__ void k_src_fill(RaysDev rays, int n_rays, unsigned long long *cursor,
         if (ja.x < j0 || ja.x >= j1) continue;
         const unsigned long long pos = atomicAdd(&cursor[ja.x], 1ull);
         tr[(long long)pos - ebase] = make_int2(r, ja.y);
+        if (entry) entry[base + h] = (unsigned)pos; // the record's entry
+    }
+}
+
+// the records' sums from the order of the index: gh[slot] holds the record's entry, then its sum
+__global__ void k_opacity_slots(long long n_slots, unsigned n_hits, const float *__restrict__ gt, float *gh) {
+    for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < n_slots; s += (long long)gridDim.x * blockDim.x) {
+        const unsigned e = __float_as_uint(gh[s]);
+        if (e < n_hits) gh[s] = __ldg(&gt[e]); // (slots between the rays' records hold anything)
     }
 }
 
@@ -787,13 +901,14 @@ __global__ void k_copy_off(const long long *off, unsigned long long *cursor, int
 }
 
 
-// the transposed index of sources j0 .. j1-1 into t->tr (entries from ebase on)
-rgs_status build_index(rgs_transport *t, int j0, int j1, long long ebase, cudaStream_t st) {
+// the transposed index of sources j0 .. j1-1 into t->tr (entries from ebase on); entries: every
+// record's entry into t->gh
+rgs_status build_index(rgs_transport *t, int j0, int j1, long long ebase, bool entries, cudaStream_t st) {
     const int n = t->n;
     const long long n_rays = (long long)n * t->nd;
     RaysDev rd = t->rays();
     { ProfScope ps_("k_copy_off", st); k_copy_off<<<(n + 255) / 256, 256, 0, st>>>(t->src_off, t->cursor, n); }
-    { ProfScope ps_("k_src_fill", st); k_src_fill<<<(unsigned)((n_rays + 255) / 256), 256, 0, st>>>(rd, (int)n_rays, t->cursor, t->tr, j0, j1, ebase); }
+    { ProfScope ps_("k_src_fill", st); k_src_fill<<<(unsigned)((n_rays + 255) / 256), 256, 0, st>>>(rd, (int)n_rays, t->cursor, t->tr, j0, j1, ebase, entries ? reinterpret_cast<unsigned *>(t->gh) : nullptr); }
     RGS_LAUNCH("transposed index");
     return RGS_OK;
 }
@@ -854,7 +969,9 @@ rgs_status run_adjoint(rgs_transport *t, const float *g, float *dE, float *dad, 
     RGS_LAUNCH("adjoint init");
     // v^(a) = K^T v^(a-1), u += v^(a): per part of the transposed index (one part holding
     // every source unless memory asked for more), per column tile
-    auto KT = [&](int a) -> rgs_status {
+    // and, where t->gt is there, g_e of the pairing (v^(a-1), B^(n-a)), B^(n-a) given in FP32 and BF16
+    const bool fused = !tcp && t->gt;
+    auto KT = [&](int a, const float *Bf, const __nv_bfloat16 *Bh) -> rgs_status {
         rgs_status q;
         if (tcp) { // tensor cores over source tiles: y^(a-1) = o c (x) v^(a-1) in BF16 row blocks
             // mode 2: the opacity gather pairs y^(a) with B^(n-1-a) while y^(a) is at hand, per
@@ -874,16 +991,19 @@ rgs_status run_adjoint(rgs_transport *t, const float *g, float *dE, float *dad, 
             const int j0 = parts[p], j1 = parts[p + 1];
             if (j1 <= j0) continue;
             const long long eb = part_base[p];
-            if (parts.size() > 2 && (q = build_index(t, j0, j1, eb, st)) != RGS_OK) return q;
+            if (parts.size() > 2 && (q = build_index(t, j0, j1, eb, false, st)) != RGS_OK) return q;
             for (int col0 = 0; col0 < C;) {
+                const AdjOpa opa{Bf, Bh, t->gt, a == 1 && col0 == 0};
                 if (t->dy_cols == 12 && C - col0 > 3) {
                     { ProfScope ps_("k_adj_ray", st); k_adj_ray<NC, 12><<<gr, 256, 0, st>>>(sd, rd, C, col0, vp(a - 1), t->dy); }
-                    { ProfScope ps_("k_adj_src_tile", st); k_adj_src_tile<NC><<<j1 - j0, ADJ_THREADS, 0, st>>>(C, col0, t->src_off, t->tr, t->dy, vp(a), t->u, j0, eb); }
+                    ProfScope ps_("k_adj_src_tile", st);
+                    (fused ? k_adj_src_tile<NC, true> : k_adj_src_tile<NC, false>)<<<j1 - j0, ADJ_THREADS, 0, st>>>(C, col0, t->src_off, t->tr, t->dy, vp(a), t->u, j0, eb, opa);
                     col0 += 12;
                     continue;
                 }
                 { ProfScope ps_("k_adj_ray", st); k_adj_ray<NC, 3><<<gr, 256, 0, st>>>(sd, rd, C, col0, vp(a - 1), t->dy); }
-                { ProfScope ps_("k_adj_src", st); k_adj_src<NC><<<j1 - j0, ADJ_THREADS, 0, st>>>(C, col0, t->src_off, t->tr, t->dy, vp(a), t->u, j0, eb); }
+                ProfScope ps_("k_adj_src", st);
+                (fused ? k_adj_src<NC, true> : k_adj_src<NC, false>)<<<j1 - j0, ADJ_THREADS, 0, st>>>(C, col0, t->src_off, t->tr, t->dy, vp(a), t->u, j0, eb, opa);
                 col0 += 3;
             }
             RGS_LAUNCH("adjoint bounce");
@@ -944,16 +1064,16 @@ rgs_status run_adjoint(rgs_transport *t, const float *g, float *dE, float *dad, 
         }
         for (int b = hi; b >= lo; --b) {
             const int a = nb - 1 - b;
-            if (a > 0 && (r = KT(a)) != RGS_OK) return r;
             { ProfScope ps_("k_pair_accum", st); k_pair_accum<NC><<<gw, 32 * ROW_WARPS, 0, st>>>(n, C, vp(a), Qb[b - lo], t->Pg); }
             RGS_LAUNCH("pair accum");
+            if ((r = KT(a + 1, Bf[b - lo], Bh[b - lo])) != RGS_OK) return r; // (v^(n) only adds to u)
         }
         if ((dopo || geo) && sddmm) { // g_h as sampled products on the tensor cores
             for (int b = hi; b >= lo; --b) {
                 if ((r = rgs_tc_opacity_sddmm(t, vp(nb - 1 - b), Bf[b - lo], first_g, b == 0, st)) != RGS_OK) return r;
                 first_g = false;
             }
-        } else if ((dopo || geo) && !(tcp && t->tc_mode == 2)) { // g_h over this segment's iterates, four per launch
+        } else if ((dopo || geo) && !fused && !(tcp && t->tc_mode == 2)) { // g_h over this segment's iterates, four per launch
             for (int b0 = hi; b0 >= lo; b0 -= 4) {
                 const int na = min(4, b0 - lo + 1);
                 const float *vv[4], *bb[4];
@@ -970,7 +1090,11 @@ rgs_status run_adjoint(rgs_transport *t, const float *g, float *dE, float *dad, 
         }
         hi = lo - 1;
     }
-    if (nb >= 1 && (r = KT(nb)) != RGS_OK) return r; // v^(n) only adds to u
+    if (fused) {
+        ProfScope ps_("k_opacity_slots", st);
+        k_opacity_slots<<<(unsigned)std::min<long long>((t->n_slots + 255) / 256, 8192), 256, 0, st>>>(t->n_slots, (unsigned)t->n_hits, t->gt, t->gh);
+        RGS_LAUNCH("opacity sums to the records");
+    }
     if (t->nl > 0) {
         launch_shadow<NC>(t, st, geo ? geo->dp : nullptr, geo ? geo->ds : nullptr, geo ? geo->gF : nullptr);
         RGS_LAUNCH("shadow backward");
@@ -1081,6 +1205,7 @@ rgs_status rgs_adjoint_impl(rgs_transport *t, const float *g, float *dE, float *
             pool_release(t->tr, st);
             pool_release(t->dy, st);
             pool_release(t->gh, st);
+            pool_release(t->gt, st);
             pool_release(geo.dp, st);
             pool_release(geo.ds, st);
             pool_release(geo.gF, st);
@@ -1151,7 +1276,13 @@ rgs_status rgs_adjoint_impl(rgs_transport *t, const float *g, float *dE, float *
     }
     if (!tcp) {
         if ((r = pool_alloc(&t->tr, (size_t)std::max(biggest, 1ll), st)) != RGS_OK) return r;
-        if (parts.size() == 2 && (r = build_index(t, 0, n, 0, st)) != RGS_OK) return r;
+        // the opacity sums with the transposed bounces where the index is in one part and their
+        // array in its order has room; else ray-wise gathers, over the iterates' rows
+        if (want_gh && parts.size() == 2 && t->n_hits > 0 && t->n_hits < (1ll << 32) && 12.0 * (double)t->n_hits <= avail) {
+            r = pool_alloc(&t->gt, (size_t)t->n_hits, st);
+            if (r != RGS_OK && r != RGS_ERR_OOM) return r;
+        }
+        if (parts.size() == 2 && (r = build_index(t, 0, n, 0, t->gt != nullptr, st)) != RGS_OK) return r;
     }
     switch (t->nc) {
     case 1: r = run_adjoint<1>(t, g, dE, dad, dop, parts, base, st, geop, false); break;

@@ -507,6 +507,23 @@ __device__ __forceinline__ bool hit_surfel(const SceneDev &sc, int j, int self, 
     return true;
 }
 
+// two FP32 numbers in a register pair, multiplied and added at once (each as fmaf)
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
 // A ray as the slab tests use it: 1/d and -o/d.  A direction component of (nearly) zero takes
 // a huge finite reciprocal, so that no product below is 0 * inf.
 struct SlabRay {
@@ -639,7 +656,7 @@ struct rgs_transport {
     unsigned *ray_ctr = nullptr; // persistent trace: next ray to fetch
     int num_sms = 0;
     float4 *dir = nullptr; // per-ray direction
-    // adjoint scratch (dy, tr, v, u, gh): taken from the workspace pool at the start
+    // adjoint scratch (dy, tr, v, u, gh, gt): taken from the workspace pool at the start
     // of rgs_adjoint and returned at its end; null outside that call
     float *dy = nullptr;    // adjoint: per-ray (direction, y) records of one column tile
     int dy_cols = 3;        // its columns: 3 (8 floats a record) or 12 (16)
@@ -689,6 +706,7 @@ struct rgs_transport {
     float *dop = nullptr; // [N]
     int pg_cap = 0;       // surfels allocated in Pg / dop
     float *gh = nullptr;  // per hit-record slot: dL/d(weight) accumulated over the bounces
+    float *gt = nullptr;  // the same in the transposed index's order, while the bounces add to it
     long long device_bytes = 0;
     // tensor-core contraction (batched modes): -1 automatic (many columns), 0 off, 1 always
     int tc_mode = -1;

@@ -7,7 +7,7 @@ import numpy as np
 import pytest
 import torch
 
-from paper_2509_18497_gb300 import rgs, scenes
+from paper_2509_18497_gb300 import api, rgs, scenes
 
 from gpu_helpers import rel_l2, run_gpu, run_oracle
 
@@ -37,3 +37,34 @@ def test_columns_against_the_oracle(lights, L, nd, n):
         assert rel_l2(g["B"], o["B"]) <= tol, (prec, rel_l2(g["B"], o["B"]))
         for key in ("dE", "dad", "dop"):
             assert rel_l2(g[key], o[key]) <= gtol, (prec, key, rel_l2(g[key], o[key]))
+
+
+@pytest.mark.parametrize("lights, L", [(1, 3), (1, 2), (1, 0), (2, 3), (4, 2), (5, 1), (5, 3)])
+@pytest.mark.parametrize("form", ["with the bounces", "index in parts", "no opacity"])
+def test_opacity_sums_against_the_oracle(lights, L, form):
+    """The per-hit opacity sums formed with the transposed bounces, ray by ray where the index
+    comes in parts (no memory for it in one), and the bounces alone."""
+    sc = scenes.random_cluster(n=83, seed=lights + L, L=L, nd=64, nb=4, n_lights=lights)
+    sc = scenes.with_emission(sc, seed=8)
+    W = np.random.default_rng(3).normal(size=(83, (L + 1) ** 2, 3 * lights))
+    o = run_oracle(sc, W=W)
+    g = torch.as_tensor(np.ascontiguousarray(W, np.float32), device="cuda")
+    for prec, (_, tol) in TOL.items():
+        d = api.upload(sc)
+        pipe = api.Pipeline(precision=prec, tensor_cores=0)
+        pipe.build(d)
+        pipe.trace(d)
+        pipe.solve(d["E"], d["nb"])
+        if form == "index in parts":
+            rgs.rgs_set_memory_budget(pipe.transport, rgs.rgs_transport_info_get(pipe.transport)["device_bytes"])
+        rgs.rgs_profile_reset()
+        rgs.rgs_profile_enable(True)
+        want = ("E", "albedo") if form == "no opacity" else ("E", "albedo", "opacity")
+        out = rgs.rgs_adjoint(pipe.transport, g, want=want)
+        torch.cuda.synchronize()
+        rgs.rgs_profile_enable(False)
+        rep = rgs.rgs_profile_report()
+        assert (rep.get("k_opacity_slots", (0, 0))[0] > 0) == (form == "with the bounces")
+        for key, v in zip(("dE", "dad", "dop"), out):
+            if v is not None:
+                assert rel_l2(v.double().cpu().numpy(), o[key]) <= tol, (prec, key)
