@@ -126,7 +126,7 @@ __device__ __forceinline__ void bounce_receiver(const SceneDev &sc, const RaysDe
         float x[CT];
 #pragma unroll
         for (int c = 0; c < CT; ++c) x[c] = 0.f;
-#pragma unroll 4
+#pragma unroll (NC == 16 ? 3 : 4)
         for (int h = 0; h < cnt; ++h) {
             const int2 ja = __ldg(&rays.rec_ja[base + h]);
             const float a = __int_as_float(ja.y);
