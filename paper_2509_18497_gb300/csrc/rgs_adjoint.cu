@@ -121,8 +121,8 @@ __global__ void __launch_bounds__(256) k_adj_ray(SceneDev sc, RaysDev rays, int 
 // B the iterate paired with v.  By source its row is read once per CTA; the ray-wise gather
 // reads a row per hit, at the ~10 TB/s the L2 gives (192 bytes a hit and iterate for 3 FP32
 // columns, 1.5 KB for 48 BF16 ones).  Both passes, 20,000 surfels, 128 rays, 16 coefficients,
-// three pairings: 3 columns 4.2 -> 1.7 ms, 12 columns 15.3 -> 4.9; 60,000 surfels, 48 BF16
-// columns, four pairings: 104 -> 66 ms.
+// three pairings: 3 columns 4.2 -> 1.7 ms, 12 columns 15.3 -> 4.4; 60,000 surfels, 48 BF16
+// columns, four pairings: 104 -> 56 ms.
 struct AdjOpa {
     const float *Bf;         // B^(b), FP32 rows
     const __nv_bfloat16 *Bh; // its BF16 rows (the batched modes), or NULL
@@ -229,14 +229,16 @@ __global__ void RGS_ADJ_LB k_adj_src(int C, int col0, const long long *__restric
 
 // 12 columns: the entries' records are copied into shared memory 128 at a time (asynchronously,
 // the next batch while this one is used: their latency, not the arithmetic, is what bounds
-// the gather), a thread evaluates the SH of one entry, and G lanes per entry, each KPL
-// coefficients, multiply: 48 FMAs (two to an instruction) per 4 shared-memory reads, 108 with the
-// opacity sums (OPA), whose partial results are copied ahead with the records (read where they
-// are added to, the 12-column pass took 86 ms for 66).  60,000 surfels, 128 rays, 48
-// columns: 1.78 ms a launch (an entry per thread at 3 columns: 1.1 ms for a quarter of them).
+// the gather), a thread evaluates the SH of one entry, and G lanes per entry, each CL
+// columns, multiply: 48 FMAs (two coefficients to an instruction), 96 with the opacity sums
+// (OPA), whose partial results are copied ahead with the records (read where they are
+// added to, the pass took a third longer).  A lane takes whole columns, so that the pairs of
+// Y come from shared memory as they are; with a quarter of the coefficients of all 12 each, the
+// duplicated factors were a fifth of the instructions (66 -> 56 ms for the 16 launches of four
+// bounces on 60,000 surfels, 128 rays, 48 columns, opacity sums included).
 constexpr int ADJ_STRIDE = 20; // floats of a record in shared memory (16-byte rows without conflicts)
 template <int NC> struct AdjLanes {
-    static constexpr int G = NC >= 9 ? 4 : 1, KPL = (NC + G - 1) / G;
+    static constexpr int G = NC >= 9 ? 4 : 1, CL = 12 / G; // lanes per entry, columns per lane
 };
 template <int NC> struct AdjTile {
     __align__(16) float rec[2][ADJ_THREADS][ADJ_STRIDE];
@@ -254,25 +256,25 @@ __global__ void __launch_bounds__(ADJ_THREADS, OPA ? 4 : 6) k_adj_src_tile(int C
                                                                const int2 *__restrict__ tr, const float *__restrict__ rec,
                                                                float *__restrict__ vout, float *__restrict__ u, int j0,
                                                                long long ebase, AdjOpa opa) {
-    constexpr int CT = 12, RS = adj_rec<CT>(), G = AdjLanes<NC>::G, KPL = AdjLanes<NC>::KPL;
+    constexpr int CT = 12, RS = adj_rec<CT>(), G = AdjLanes<NC>::G, CL = AdjLanes<NC>::CL;
+    constexpr int NP = (NC + 1) / 2, NY = (NC + 3) / 4; // pairs of coefficients; 16-byte pieces of Y
     __shared__ AdjTile<NC> s;
     const int j = j0 + blockIdx.x;
     const int tid = threadIdx.x, lane = tid & 31, g = tid % G;
-    constexpr int CP = CT / 2; // pairs of columns
-    uint64_t acc[KPL][CP];
+    uint64_t acc[CL][NP];
 #pragma unroll
-    for (int k = 0; k < KPL; ++k)
+    for (int c = 0; c < CL; ++c)
 #pragma unroll
-        for (int c = 0; c < CP; ++c) acc[k][c] = 0ull;
-    uint64_t Bj[OPA ? CP : 1][OPA ? KPL : 1]; // this lane's coefficients of the source's paired row
+        for (int k = 0; k < NP; ++k) acc[c][k] = 0ull;
+    uint64_t Bj[OPA ? CL : 1][OPA ? NP : 1]; // this lane's columns of the source's paired row
     if constexpr (OPA) {
         auto el = [&](int c, int k) {
-            return col0 + c < C && KPL * g + k < NC ? adj_opa_row<NC>(opa, (size_t)j * C + col0 + c, KPL * g + k) : 0.f;
+            return c < C && k < NC ? adj_opa_row<NC>(opa, (size_t)j * C + c, k) : 0.f;
         };
 #pragma unroll
-        for (int c = 0; c < CP; ++c)
+        for (int c = 0; c < CL; ++c)
 #pragma unroll
-            for (int k = 0; k < KPL; ++k) Bj[c][k] = pack2(el(2 * c, k), el(2 * c + 1, k));
+            for (int k = 0; k < NP; ++k) Bj[c][k] = pack2(el(col0 + CL * g + c, 2 * k), el(col0 + CL * g + c, 2 * k + 1));
     }
     const long long e0 = src_off[j] - ebase, e1 = src_off[j + 1] - ebase;
     const int batches = (int)((e1 - e0 + ADJ_THREADS - 1) / ADJ_THREADS);
@@ -311,7 +313,7 @@ __global__ void __launch_bounds__(ADJ_THREADS, OPA ? 4 : 6) k_adj_src_tile(int C
             float Yo[NC];
             sh_eval<NC>(make_float3(-d.x, -d.y, -d.z), Yo);
 #pragma unroll
-            for (int k = 0; k < G * KPL; ++k) s.Y[tid][k] = k < NC ? Yo[k < NC ? k : 0] : 0.f;
+            for (int k = 0; k < 4 * NY; ++k) s.Y[tid][k] = k < NC ? Yo[k < NC ? k : 0] : 0.f;
         }
         __syncthreads();
         const int rounds = (m + ADJ_THREADS / G - 1) / (ADJ_THREADS / G); // (all lanes: OPA sums over a group's)
@@ -319,29 +321,26 @@ __global__ void __launch_bounds__(ADJ_THREADS, OPA ? 4 : 6) k_adj_src_tile(int C
         for (int q0 = 0; q0 < rounds; ++q0) {
             const int at = q0 * (ADJ_THREADS / G) + tid / G, x = min(at, m - 1);
             if (!OPA && at >= m) break;
-            float w[KPL];
-            uint64_t y[CP];
+            uint64_t Y[2 * NY];
+            float y[CL];
 #pragma unroll
-            for (int k = 0; k < KPL; ++k) w[k] = s.Y[x][KPL * g + k];
-#pragma unroll
-            for (int q = 0; q < CT / 4; ++q) {
-                const ulonglong2 f = *reinterpret_cast<const ulonglong2 *>(&s.rec[st][x][4 + 4 * q]);
-                y[2 * q] = f.x;
-                y[2 * q + 1] = f.y;
+            for (int q = 0; q < NY; ++q) {
+                const ulonglong2 f = *reinterpret_cast<const ulonglong2 *>(&s.Y[x][4 * q]);
+                Y[2 * q] = f.x;
+                Y[2 * q + 1] = f.y;
             }
+#pragma unroll
+            for (int c = 0; c < CL; ++c) y[c] = s.rec[st][x][4 + CL * g + c];
             if constexpr (OPA) {
-                uint64_t t2 = 0ull, w2[KPL];
+                float t = 0.f;
 #pragma unroll
-                for (int k = 0; k < KPL; ++k) w2[k] = pack2(w[k], w[k]);
+                for (int c = 0; c < CL; ++c) {
+                    uint64_t two = 0ull;
 #pragma unroll
-                for (int c = 0; c < CP; ++c) {
-                    uint64_t sc = 0ull;
-#pragma unroll
-                    for (int k = 0; k < KPL; ++k) sc = fma2(w2[k], Bj[c][k], sc);
-                    t2 = fma2(y[c], sc, t2);
+                    for (int k = 0; k < NP; ++k) two = fma2(Y[k], Bj[c][k], two);
+                    const float2 sc = unpack2(two);
+                    t += y[c] * (sc.x + sc.y);
                 }
-                const float2 tt = unpack2(t2);
-                float t = tt.x + tt.y;
 #pragma unroll
                 for (int off = 1; off < G; off <<= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
                 if (g == 0 && at < m)
@@ -350,26 +349,26 @@ __global__ void __launch_bounds__(ADJ_THREADS, OPA ? 4 : 6) k_adj_src_tile(int C
             }
             const float a = s.a[st][x];
 #pragma unroll
-            for (int k = 0; k < KPL; ++k) {
-                const uint64_t aw = pack2(a * w[k], a * w[k]);
+            for (int c = 0; c < CL; ++c) {
+                const uint64_t ay = pack2(a * y[c], a * y[c]);
 #pragma unroll
-                for (int c = 0; c < CP; ++c) acc[k][c] = fma2(aw, y[c], acc[k][c]);
+                for (int k = 0; k < NP; ++k) acc[c][k] = fma2(ay, Y[k], acc[c][k]);
             }
         }
         __syncthreads(); // the tables are rewritten
     }
-    float *red = &s.rec[0][0][0]; // [warp][G KPL CT]
-    constexpr int OUT = G * KPL * CT;
+    float *red = &s.rec[0][0][0]; // [warp][NC CT]
+    constexpr int OUT = NC * CT;
     static_assert(ADJ_THREADS / 32 * OUT <= 2 * ADJ_THREADS * ADJ_STRIDE, "the sums fit the records' place");
 #pragma unroll
-    for (int k = 0; k < KPL; ++k)
+    for (int c = 0; c < CL; ++c)
 #pragma unroll
-        for (int c = 0; c < CT; ++c) {
-            const float2 two = unpack2(acc[k][c / 2]);
-            float v = c & 1 ? two.y : two.x;
+        for (int k = 0; k < NC; ++k) {
+            const float2 two = unpack2(acc[c][k / 2]);
+            float v = k & 1 ? two.y : two.x;
 #pragma unroll
             for (int off = 16; off >= G; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-            if (lane < G) red[(tid >> 5) * OUT + (KPL * lane + k) * CT + c] = v;
+            if (lane < G) red[(tid >> 5) * OUT + k * CT + CL * lane + c] = v;
         }
     __syncthreads();
     for (int e = tid; e < NC * CT; e += ADJ_THREADS) {
