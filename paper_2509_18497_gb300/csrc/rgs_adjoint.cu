@@ -608,8 +608,10 @@ __global__ void RGS_OPA_LB k_opacity_g(SceneDev sc, RaysDev rays, int C, int col
 // dL/do_{j_h} += T_h (g_h - R_h) dalpha_h/do, with T_h the transmittance in front of hit h,
 // T_h = a_h / alpha_h from the stored weight.  G_h is recomputed from the stored direction
 // (bit-identical to the trace's value).
+// gt: the sums are there in the order of the transposed index, and gh holds each record's entry
+// (50,000 surfels, 256 rays: 5.4 ms against 2.8 for a pass that sorts them and 3.4).
 __global__ void RGS_OPAREC_LB k_opacity_rec(SceneDev sc, RaysDev rays, const float *__restrict__ gh,
-                                                     float *dop) {
+                                                     const float *__restrict__ gt, float *dop) {
     // Blocks take the rays in a scattered order (block b -> b * 2654435761 mod gridDim, a
     // bijection: the multiplier is prime): blocks resident at the same time then hold
     // receivers spread over the scene, so their dL/do atomics go to sources all over it
@@ -632,7 +634,7 @@ __global__ void RGS_OPAREC_LB k_opacity_rec(SceneDev sc, RaysDev rays, const flo
         accepted_hit(sc, j, o, d, t, r2, oj);
         const float G = surfel_G(sc, r2);
         const float alpha = alpha_of(sc, oj, G);
-        const float g = gh[slot];
+        const float g = gt ? __ldg(&gt[__float_as_uint(gh[slot])]) : gh[slot]; // (gt: gh holds the records' entries)
         // the transmittance in front of the hit from its stored weight a_h = alpha_h T_h
         // (alpha_h = 0 makes dalpha/do vanish for the disc and Gaussian models; GFSGS: alpha = 0
         // only where x = o G = 0, where dalpha/do is 0 too)
@@ -1089,7 +1091,7 @@ rgs_status run_adjoint(rgs_transport *t, const float *g, float *dE, float *dad, 
         }
         hi = lo - 1;
     }
-    if (fused) {
+    if (fused && geo) { // (k_opacity_rec alone reads them through the entries)
         ProfScope ps_("k_opacity_slots", st);
         k_opacity_slots<<<(unsigned)std::min<long long>((t->n_slots + 255) / 256, 8192), 256, 0, st>>>(t->n_slots, (unsigned)t->n_hits, t->gt, t->gh);
         RGS_LAUNCH("opacity sums to the records");
@@ -1099,7 +1101,7 @@ rgs_status run_adjoint(rgs_transport *t, const float *g, float *dE, float *dad, 
         RGS_LAUNCH("shadow backward");
     }
     if (nb >= 1 && dopo) {
-        { ProfScope ps_("k_opacity_rec", st); k_opacity_rec<<<gr, 256, 0, st>>>(sd, rd, t->gh, t->dop); }
+        { ProfScope ps_("k_opacity_rec", st); k_opacity_rec<<<gr, 256, 0, st>>>(sd, rd, t->gh, fused && !geo ? t->gt : nullptr, t->dop); }
         RGS_LAUNCH("hemisphere opacity backward");
     }
     if (nb >= 1 && geo) { // every iterate is kept (the caller checked the stride)

@@ -64,7 +64,8 @@ def test_opacity_sums_against_the_oracle(lights, L, form):
         torch.cuda.synchronize()
         rgs.rgs_profile_enable(False)
         rep = rgs.rgs_profile_report()
-        assert (rep.get("k_opacity_slots", (0, 0))[0] > 0) == (form == "with the bounces")
+        raywise = sum(rep.get(k, (0, 0))[0] for k in ("k_opacity_g", "k_opacity_g_mc"))
+        assert (raywise > 0) == (form == "index in parts")
         for key, v in zip(("dE", "dad", "dop"), out):
             if v is not None:
                 assert rel_l2(v.double().cpu().numpy(), o[key]) <= tol, (prec, key)
