@@ -7,9 +7,11 @@
 // K^T v is a gather over the records grouped by source surfel j:
 //   (K^T v)_j[c][k] = sum_{hits e on j} a_e Y_k(-d_e) y_e[c],
 //   y_e[c] = (pi/nd) o_i sum_k' c_{i,l(k'),ch} Y_k'(R_i d_e) v_i[c][k']      (i = receiver of e)
-// k_adj_ray forms y per ray once (ray-major, next to the stored direction) and k_adj_src
-// gathers (d, y) per entry, 32 bytes, instead of a 192-byte row of v_i per entry.
-// k_opacity_g / k_opacity_rec and k_shadow_bwd run the compositing backward of every
+// k_adj_ray forms y per ray once (one record with the ray's direction) and k_adj_src gathers
+// (d, y) per entry, 32 bytes, instead of a 192-byte row of v_i per entry (k_adj_src_tile: 12
+// columns, 64 bytes).  With it go the hits' opacity sums g_e = sum_a y_e^(a) . (Y(-d_e) B_j^(n-1-a));
+// k_opacity_g forms them ray by ray where the index comes in parts.
+// k_opacity_rec and k_shadow_bwd run the compositing backward of every
 // hemisphere and shadow ray (dL/dalpha_h = T_h (g_h - R_h), dL/dT = -prod of the other (1 - alpha)).
 #include <algorithm>
 #include <vector>

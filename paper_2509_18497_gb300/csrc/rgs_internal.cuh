@@ -25,7 +25,8 @@
 // is sized for that many resident blocks per SM (these latency-bound kernels gain from more
 // resident warps as long as nothing spills); undefined, the compiler's default budget.
 // Build-time knobs, set from measurements on GB300 (50,000-surfel bowl, 1 and 16 lights):
-// 5 blocks for the 3-column bounce (-9 %, despite a few spilled registers), 4 for the
+// 5 blocks for the 3-column bounce (-9 %, despite a few spilled registers; 6 at 16
+// coefficients, rgs_solve.cu), 4 for the
 // lane-per-column bounce (-18 %) and opacity gather (-5 %); the 3-column opacity gather keeps
 // the default (tighter budgets measured slower).
 #define RGS_LB_(threads, minb) __launch_bounds__(threads, minb)

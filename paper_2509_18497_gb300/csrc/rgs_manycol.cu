@@ -2,7 +2,7 @@
 //
 // With C columns the per-hit work of the gather is a row of C x nc coefficients of the
 // source surfel.  The 3-column kernels (rgs_solve.cu, rgs_adjoint.cu) would re-read every
-// hit record once per 3-column tile; here a warp takes one ray (or one transposed entry) at
+// hit record once per 3-column tile; here a warp takes one ray at
 // a time and its 32 lanes take 32 consecutive columns, so each hit is read once per
 // 32-column tile and every row load is one contiguous 512-byte (BF16) or 1-KiB (FP32)
 // warp access.  Which layout a launch uses is decided per kernel family by wide_bounce and
@@ -22,7 +22,7 @@ __global__ void RGS_MCB_LB k_bounce_mc(SceneDev sc, RaysDev rays, int C, const T
 }
 
 // ------------------------------------------------------------------ adjoint
-// opacity backward: per hit g_h (partial over this column tile and iterate chunk)
+// opacity backward, ray by ray: per hit g_h (partial over this column tile and iterate chunk)
 // accumulated into gh[slot]; a warp per ray, lanes over columns.  The lanes hold 32 of the ray's
 // records at a time, four hits' rows are requested together, and their four sums over the
 // columns share one reduction: with a hit, its row and a five-step reduction at a time every

@@ -124,3 +124,17 @@ def test_far_from_the_origin(alpha):
     sc = scenes.random_cluster(n=200, seed=11, L=2, nd=64, nb=2, n_lights=1)
     sc["p"][:100] = np.asarray(sc["p"][:100] + 8.0, np.float32).astype(np.float64)
     _check(sc, alpha=alpha)
+
+
+@pytest.mark.parametrize("n", [1024, 1025, 4097, 8192, 8193])
+def test_surfel_order_at_the_sort_sizes(n):
+    """Scenes at the sizes where the Morton sort pads, fills its block, or goes over to the radix
+    passes, with equal keys (pairs of surfels at one centre): sampled receivers against the oracle."""
+    sc = scenes.random_cluster(n=n, seed=n, L=1, nd=32, nb=1, n_lights=1, extent=4.0)
+    sc["s"] = sc["s"] * 0.3
+    sc["p"][1::2] = sc["p"][0:n - n % 2:2]
+    g = run_gpu(sc, iterates=True)
+    orc = O.Oracle(sc)
+    recv = np.random.default_rng(1).choice(n, size=12, replace=False)
+    assert rel_l2(g["iters"][0][recv], orc.sample_direct(recv)) <= TOL
+    assert rel_l2(g["iters"][1][recv], orc.sample_bounce1(recv)) <= TOL
