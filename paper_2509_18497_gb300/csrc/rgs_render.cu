@@ -3,7 +3,7 @@
 // outgoing SH radiance (Sec. 5.3, end) -- and its transpose, the dL/dB a loss on the image
 // hands to rgs_adjoint (Sec. 6, opening).
 //
-//  k_render : a warp per tile of 8 x 4 pixels.  The pixel rays o + t d meet the surfels in depth
+//  k_render : a warp per tile of 8 x 1 to 8 x 4 pixels.  The pixel rays o + t d meet the surfels in depth
 //             order under the transport's hit rules (eps_plane, the cutoff, tie runs; no surfel
 //             excluded), composited a_h = alpha_h prod_{k<h} (1 - alpha_k) until the
 //             transmittance is below RGS_T_EPS, and the warp shades each pixel's hits at
@@ -143,14 +143,14 @@ __device__ __forceinline__ void scatter_pixel(const int4 *hits, int n, float3 d,
     }
 }
 
-// Persistent warps take tiles of 8 x 4 pixels from a counter; the lanes trace their pixels'
+// Persistent warps take tiles of 8 x rows pixels from a counter; the lanes trace their pixels'
 // rays together (rgs_warp_trace.cuh), then the warp composites and shades one pixel after the
 // other from its scratch lists: no record leaves the SM's neighbourhood, and every ray is
 // traced once.  A ray with more than RGS_HMAX hits in front of the transmittance cut takes
 // further passes, each behind the last composited hit, so any number is composited.
 // ADJ: in = dL/dimg, out = dL/dB (zeroed); else in = B, out = the image.
 template <int NC, bool ADJ>
-__global__ void __launch_bounds__(RN_THREADS, RN_MINB) k_render(SceneDev sc, Cam cam, int W, int H, float fov, int C,
+__global__ void __launch_bounds__(RN_THREADS, RN_MINB) k_render(SceneDev sc, Cam cam, int W, int H, int rows, float fov, int C,
                                                                const float *__restrict__ in, float *out, unsigned *work,
                                                                int4 *lists, int *flags) {
     __shared__ WarpHits sm_all[RN_THREADS / 32];
@@ -158,15 +158,15 @@ __global__ void __launch_bounds__(RN_THREADS, RN_MINB) k_render(SceneDev sc, Cam
     WarpHits &sm = sm_all[threadIdx.x >> 5];
     int4 *list = lists + (size_t)(blockIdx.x * (RN_THREADS / 32) + (threadIdx.x >> 5)) * (32 * WT_LIST);
     const float eps = *sc.eps_plane;
-    const int tx = (W + 7) / 8, ty = (H + 3) / 4;
+    const int tx = (W + 7) / 8, ty = (H + rows - 1) / rows;
     const float3 o = make_float3(cam.v[0], cam.v[1], cam.v[2]);
     while (true) {
         unsigned w = 0;
         if (lane == 0) w = atomicAdd(work, 1u);
         w = __shfl_sync(WT_FULL, w, 0);
         if (w >= (unsigned)tx * (unsigned)ty) return;
-        const int x = (int)(w % (unsigned)tx) * 8 + (lane & 7), y = (int)(w / (unsigned)tx) * 4 + (lane >> 3);
-        const bool live = x < W && y < H;
+        const int x = (int)(w % (unsigned)tx) * 8 + (lane & 7), y = (int)(w / (unsigned)tx) * rows + (lane >> 3);
+        const bool live = x < W && y < H && (lane >> 3) < rows;
         const float3 d = pixel_dir(cam.v, W, H, fov, x, y);
         const size_t pix = (size_t)y * W + x;
         float T = 1.f;
@@ -234,6 +234,16 @@ rgs_status check_args(const rgs_transport *t, const float *in, const float *cam,
     return RGS_OK;
 }
 
+// Rows of a warp's tile. A warp lasts as long as its slowest pixels (grazing rays meet hundreds
+// of surfels, some take several passes), so an image with few tiles for the 4,256 warps in
+// flight is traced 8 or 16 pixels to a warp: less is shared, but the last warp ends sooner.
+// 200,000 pixels: 4 rows 0.8 to 4.2 ms, 2 rows 0.6 to 2.2, 1 row 0.5 to 1.4 (thread per pixel
+// before: 1.7 to 4.7); 532,000: 1.3 to 3.5, 1.3 to 2.2, 1.6 to 1.9; 2,074,000: 3.3, 3.3, 4.3.
+int tile_rows(int W, int H) {
+    const long long px = (long long)W * H;
+    return px < 500000 ? 1 : (px < 1200000 ? 2 : 4);
+}
+
 // the tiles' launch, and the check that no traversal stack overflowed
 template <int NC, bool ADJ>
 rgs_status run_tiles(rgs_transport *t, const float *in, const float *cam, int W, int H, float fov, float *out,
@@ -244,12 +254,13 @@ rgs_status run_tiles(rgs_transport *t, const float *in, const float *cam, int W,
     Cam c;
     for (int q = 0; q < 9; ++q) c.v[q] = cam[q];
     WarpLists warps{s.st};
-    const long long tiles = (long long)((W + 7) / 8) * ((H + 3) / 4);
+    const int rows = tile_rows(W, H);
+    const long long tiles = (long long)((W + 7) / 8) * ((H + rows - 1) / rows);
     if ((r = warps.get((const void *)k_render<NC, ADJ>, RN_THREADS, tiles)) != RGS_OK) return r;
     RGS_CUDA(cudaMemsetAsync(warps.work, 0, sizeof(unsigned), s.st));
     {
         ProfScope ps_(ADJ ? "k_render_adj" : "k_render", s.st);
-        k_render<NC, ADJ><<<warps.blocks, RN_THREADS, 0, s.st>>>(t->sc->dev(), c, W, H, fov, t->C, in, out, warps.work,
+        k_render<NC, ADJ><<<warps.blocks, RN_THREADS, 0, s.st>>>(t->sc->dev(), c, W, H, rows, fov, t->C, in, out, warps.work,
                                                                 warps.lists, s.flag);
     }
     RGS_LAUNCH("render");
