@@ -400,13 +400,13 @@ struct ShadowWarp {
     float gp[32][3], gw[32][3];
 };
 template <int NC, bool GEO>
-__global__ void __launch_bounds__(SHADOW_THREADS) k_shadow_bwd(SceneDev sc, int nl, int ldir, const float *__restrict__ lpos, const float *__restrict__ lint,
+__global__ void __launch_bounds__(SHADOW_THREADS) k_shadow_bwd(SceneDev sc, int nl, int per, int ldir, const float *__restrict__ lpos, const float *__restrict__ lint,
                              int C, const float *__restrict__ u, float *P, float *dop, float *dp, float *ds, float *gF) {
     extern __shared__ __align__(16) unsigned char shadow_smem[];
     ShadowWarp &sm = reinterpret_cast<ShadowWarp *>(shadow_smem)[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
-    const int tid = blockIdx.x * blockDim.x + threadIdx.x;
-    const bool live = tid < sc.n * nl;
+    const int tid = (blockIdx.x * (SHADOW_THREADS / 32) + (threadIdx.x >> 5)) * per + lane;
+    const bool live = lane < per && tid < sc.n * nl;
     const int i = live ? tid / nl : 0, lt = live ? tid - i * nl : 0;
     const float4 Pi = sc.P[i];
     const float3 o = f3(Pi), n = f3(sc.N4[i]);
@@ -522,12 +522,12 @@ __global__ void __launch_bounds__(SHADOW_THREADS) k_shadow_bwd(SceneDev sc, int 
 
 template <int NC>
 void launch_shadow(rgs_transport *t, cudaStream_t st, float *dp, float *ds, float *gF) {
-    const int nth = t->n * t->nl;
-    const unsigned blocks = (unsigned)((nth + SHADOW_THREADS - 1) / SHADOW_THREADS);
+    const int per = shadow_pairs((long long)t->n * t->nl), pb = SHADOW_THREADS / 32 * per; // pairs of a warp, a block
+    const unsigned blocks = (unsigned)((t->n * t->nl + pb - 1) / pb);
     const size_t smem = sizeof(ShadowWarp) * (SHADOW_THREADS / 32);
     ProfScope ps_("k_shadow_bwd", st);
-    if (dp) k_shadow_bwd<NC, true><<<blocks, SHADOW_THREADS, smem, st>>>(t->sc->dev(), t->nl, t->ldir, t->lpos, t->lint, t->C, t->u, t->Pg, t->dop, dp, ds, gF);
-    else k_shadow_bwd<NC, false><<<blocks, SHADOW_THREADS, smem, st>>>(t->sc->dev(), t->nl, t->ldir, t->lpos, t->lint, t->C, t->u, t->Pg, t->dop, dp, ds, gF);
+    if (dp) k_shadow_bwd<NC, true><<<blocks, SHADOW_THREADS, smem, st>>>(t->sc->dev(), t->nl, per, t->ldir, t->lpos, t->lint, t->C, t->u, t->Pg, t->dop, dp, ds, gF);
+    else k_shadow_bwd<NC, false><<<blocks, SHADOW_THREADS, smem, st>>>(t->sc->dev(), t->nl, per, t->ldir, t->lpos, t->lint, t->C, t->u, t->Pg, t->dop, dp, ds, gF);
 }
 
 // Hemisphere rays, part 1: for every stored hit h of ray r (receiver i, source j_h),

@@ -21,13 +21,13 @@ constexpr int HEMI_THREADS = 128, DIRECT_THREADS = 128;
 
 namespace {
 
-// A warp per patch of 32 rays of one surfel, patches handed out by a counter.  The lanes walk
+// A warp per patch of 32 rays of one surfel (or a part of it), patches handed out by a counter.  The lanes walk
 // the tree for their own rays and pool the surfel tests (rgs_warp_trace.cuh); accepted hits
 // go to per-ray lists in this warp's scratch (rewritten for every patch, so it stays in
 // L2), each ray's traversal ends once the hits found make the rest invisible, and the warp
 // then orders and composites one ray after the other, a lane per hit.  It allocates exactly
 // its rays' kept hits with one atomic and stores every ray's records contiguously.
-__global__ void __launch_bounds__(HEMI_THREADS, RGS_TRACE_MINB) k_trace_hemi(SceneDev sc, RaysDev rays, int n_patches, long long cap_slots,
+__global__ void __launch_bounds__(HEMI_THREADS, RGS_TRACE_MINB) k_trace_hemi(SceneDev sc, RaysDev rays, long long jobs, int split, long long cap_slots,
                                                        unsigned long long *slot_ctr, unsigned *work, int2 *rec_ja,
                                                        long long *off_out, int *cnt_out, float4 *dir_out,
                                                        int *src_cnt, int *flags, int pa, int4 *lists) {
@@ -38,10 +38,13 @@ __global__ void __launch_bounds__(HEMI_THREADS, RGS_TRACE_MINB) k_trace_hemi(Sce
     const float eps = *sc.eps_plane;
     const int per = rays.nd >> 5; // patches of a surfel
     while (true) {
-        unsigned w = 0;
-        if (lane == 0) w = atomicAdd(work, 1u);
-        w = __shfl_sync(WT_FULL, w, 0);
-        if (w >= (unsigned)n_patches) return;
+        unsigned job = 0;
+        if (lane == 0) job = atomicAdd(work, 1u);
+        job = __shfl_sync(WT_FULL, job, 0);
+        if (job >= jobs) return;
+        // a patch of 32 rays, or one of its `split` parts
+        const unsigned w = job / (unsigned)split;
+        const bool active = lane / (32 / split) == (int)(job - w * (unsigned)split);
         // the warps of surfel i take patches of pa x (32 / pa) strata (elevation x azimuth) of its
         // na x nbs grid, so that a warp's rays leave in similar directions; pa = 0: 32 consecutive rays
         const int i = (int)(w / (unsigned)per), pt = (int)(w - (unsigned)i * (unsigned)per);
@@ -54,9 +57,9 @@ __global__ void __launch_bounds__(HEMI_THREADS, RGS_TRACE_MINB) k_trace_hemi(Sce
         const int r = i * rays.nd + q; // this lane's ray (outputs are indexed by ray)
         const float3 o = f3(sc.P[i]);
         const float3 d = ray_dir(rays.seed, sc.uid[i], q, rays.na, rays.nbs, f3(sc.FU[i]), f3(sc.FV[i]), f3(sc.N4[i]));
-        dir_out[r] = make_float4(d.x, d.y, d.z, 0.f);
+        if (active) dir_out[r] = make_float4(d.x, d.y, d.z, 0.f);
         bool full;
-        if (!warp_collect<false>(sc, o, d, i, true, eps, 0, sm, list, full)) atomicAdd(&flags[FLAG_STACK], 1);
+        if (!warp_collect<false>(sc, o, d, i, active, eps, 0, sm, list, full)) atomicAdd(&flags[FLAG_STACK], 1);
         int kept = 0; // of this lane's ray
         for (int x = 0; x < 32; ++x) {
             int H = sm.cnt[x];
@@ -84,9 +87,11 @@ __global__ void __launch_bounds__(HEMI_THREADS, RGS_TRACE_MINB) k_trace_hemi(Sce
         sbase = __shfl_sync(WT_FULL, sbase, 31);
         const unsigned long long mine = sbase + (unsigned long long)(incl - kept);
         const bool fits = mine + (unsigned long long)kept <= (unsigned long long)cap_slots;
-        off_out[r] = (long long)mine;
-        cnt_out[r] = fits ? kept : 0;
-        if (!fits) atomicAdd(&flags[FLAG_CAPACITY], 1);
+        if (active) {
+            off_out[r] = (long long)mine;
+            cnt_out[r] = fits ? kept : 0;
+        }
+        if (!fits && active) atomicAdd(&flags[FLAG_CAPACITY], 1);
         const unsigned store = __ballot_sync(WT_FULL, fits && kept > 0);
         for (unsigned m = store; m; m &= m - 1) {
             const int x = __ffs(m) - 1;
@@ -104,13 +109,13 @@ __global__ void __launch_bounds__(HEMI_THREADS, RGS_TRACE_MINB) k_trace_hemi(Sce
 
 // Direct term (Sec. 5.2): D_i[L*3+ch][k] = o_i c_{i,l(k),ch} Y_k(R_i w) I_{L,ch} (n_i.w)/r^2 T
 // (no 1/r^2 and a shadow ray to infinity for a directional light)
-// A warp per 32 (surfel, light) pairs, their shadow rays traced together (rgs_warp_trace.cuh).
+// A warp per 32 or 16 (surfel, light) pairs, their shadow rays traced together (rgs_warp_trace.cuh).
 template <int NC>
-__global__ void __launch_bounds__(DIRECT_THREADS) k_direct(SceneDev sc, int nl, int ldir, const float *__restrict__ lpos,
+__global__ void __launch_bounds__(DIRECT_THREADS) k_direct(SceneDev sc, int nl, int per, int ldir, const float *__restrict__ lpos,
                                                           const float *__restrict__ lint, int C, float *D, int *flags) {
     __shared__ WarpOcclusion sm[DIRECT_THREADS / 32];
-    const int tid = blockIdx.x * blockDim.x + threadIdx.x;
-    const bool live = tid < sc.n * nl;
+    const int tid = (blockIdx.x * (DIRECT_THREADS / 32) + (threadIdx.x >> 5)) * per + (threadIdx.x & 31);
+    const bool live = (threadIdx.x & 31) < per && tid < sc.n * nl;
     const int i = live ? tid / nl : 0, lt = live ? tid - i * nl : 0;
     const float4 Pi = sc.P[i];
     const float3 o = f3(Pi), n = f3(sc.N4[i]);
@@ -194,12 +199,13 @@ rgs_status rgs_transport_common(rgs_transport *t, const rgs_lights *L, cudaStrea
 rgs_status rgs_direct_term(rgs_transport *t, cudaStream_t st) {
     SceneDev sd = t->sc->dev();
     if (t->nl > 0) {
-        const int nth = t->n * t->nl;
+        const int per = shadow_pairs((long long)t->n * t->nl), pb = DIRECT_THREADS / 32 * per; // pairs of a warp, a block
+        const int blocks = (t->n * t->nl + pb - 1) / pb;
         switch (t->nc) {
-        case 1: { ProfScope ps_("k_direct", st); k_direct<1><<<(nth + DIRECT_THREADS - 1) / DIRECT_THREADS, DIRECT_THREADS, 0, st>>>(sd, t->nl, t->ldir, t->lpos, t->lint, t->C, t->D, t->flags); } break;
-        case 4: { ProfScope ps_("k_direct", st); k_direct<4><<<(nth + DIRECT_THREADS - 1) / DIRECT_THREADS, DIRECT_THREADS, 0, st>>>(sd, t->nl, t->ldir, t->lpos, t->lint, t->C, t->D, t->flags); } break;
-        case 9: { ProfScope ps_("k_direct", st); k_direct<9><<<(nth + DIRECT_THREADS - 1) / DIRECT_THREADS, DIRECT_THREADS, 0, st>>>(sd, t->nl, t->ldir, t->lpos, t->lint, t->C, t->D, t->flags); } break;
-        default: { ProfScope ps_("k_direct", st); k_direct<16><<<(nth + DIRECT_THREADS - 1) / DIRECT_THREADS, DIRECT_THREADS, 0, st>>>(sd, t->nl, t->ldir, t->lpos, t->lint, t->C, t->D, t->flags); }
+        case 1: { ProfScope ps_("k_direct", st); k_direct<1><<<blocks, DIRECT_THREADS, 0, st>>>(sd, t->nl, per, t->ldir, t->lpos, t->lint, t->C, t->D, t->flags); } break;
+        case 4: { ProfScope ps_("k_direct", st); k_direct<4><<<blocks, DIRECT_THREADS, 0, st>>>(sd, t->nl, per, t->ldir, t->lpos, t->lint, t->C, t->D, t->flags); } break;
+        case 9: { ProfScope ps_("k_direct", st); k_direct<9><<<blocks, DIRECT_THREADS, 0, st>>>(sd, t->nl, per, t->ldir, t->lpos, t->lint, t->C, t->D, t->flags); } break;
+        default: { ProfScope ps_("k_direct", st); k_direct<16><<<blocks, DIRECT_THREADS, 0, st>>>(sd, t->nl, per, t->ldir, t->lpos, t->lint, t->C, t->D, t->flags); }
         }
         RGS_LAUNCH("direct");
     } else {
@@ -245,9 +251,12 @@ rgs_status rgs_trace_impl(rgs_transport *t, const rgs_lights *L, const rgs_trace
     int pa = 0;
     for (int c = RGS_TRACE_PATCH_A; c >= 1 && !pa; c >>= 1)
         if (t->na % c == 0 && 32 % c == 0 && t->nbs % (32 / c) == 0) pa = c;
-    const int n_patches = (int)(n_rays / 32);
+    // A warp lasts as long as its slowest ray: few patches are traced in 2 or 4 parts (500
+    // patches: 0.26, 0.19, 0.16 ms in 1, 2, 4 parts; 2,000: 0.33, 0.28, 0.31; 4,000: 0.46, 0.45, 0.59).
+    const int split = n_rays < 750 * 32 ? 4 : (n_rays < 1500 * 32 ? 2 : 1);
+    const long long jobs = n_rays / 32 * split;
     WarpLists warps{st};
-    if ((r = warps.get((const void *)k_trace_hemi, HEMI_THREADS, n_patches)) != RGS_OK) return r;
+    if ((r = warps.get((const void *)k_trace_hemi, HEMI_THREADS, jobs)) != RGS_OK) return r;
     for (int attempt = 0; attempt < 2; ++attempt) {
         if (want > t->cap_slots) {
             if ((r = dev_alloc(&t->rec_ja, (size_t)want, &t->device_bytes)) != RGS_OK) return r;
@@ -258,7 +267,7 @@ rgs_status rgs_trace_impl(rgs_transport *t, const rgs_lights *L, const rgs_trace
         RGS_CUDA(cudaMemsetAsync(t->src_cnt, 0, sizeof(int) * n, st));
         RaysDev rd = t->rays();
         RGS_CUDA(cudaMemsetAsync(warps.work, 0, sizeof(unsigned), st));
-        { ProfScope ps_("k_trace_hemi", st); k_trace_hemi<<<warps.blocks, HEMI_THREADS, 0, st>>>(sd, rd, n_patches, t->cap_slots, t->counter, warps.work, t->rec_ja, t->off, t->cnt, t->dir, t->src_cnt, t->flags, pa, warps.lists); }
+        { ProfScope ps_("k_trace_hemi", st); k_trace_hemi<<<warps.blocks, HEMI_THREADS, 0, st>>>(sd, rd, jobs, split, t->cap_slots, t->counter, warps.work, t->rec_ja, t->off, t->cnt, t->dir, t->src_cnt, t->flags, pa, warps.lists); }
         RGS_LAUNCH("trace_hemi");
         unsigned long long used = 0;
         int flags[FLAG_COUNT];
