@@ -112,7 +112,7 @@ def _src_sha(name):
 # DRAM bytes per launch from one ncu capture (profiles/), keyed by kernel; valid only
 # while the kernel's source file is unchanged since the capture.
 NCU_TRAFFIC = {
-    "k_trace_hemi": {"bytes_per_launch": 0.999770e9 + 2.009972e9, "n": 10000, "src_sha": "77c7ef57011d69f1"},
+    "k_trace_hemi": {"bytes_per_launch": 0.446134e9 + 1.667045e9, "n": 10000, "src_sha": "ca603cdd76f7fe9c"},
 }
 
 
@@ -124,6 +124,7 @@ def _launch_bytes(kernel, sc):
     rays = n * nd
     tile = A * 3 // C           # one 3-column tile of such an array
     T3 = C // 3                 # 3-column tiles
+    T12 = (C + 11) // 12        # 12-column tiles
     tiles = (C + 31) // 32      # 32-column tiles
     A16 = n * C * (16 if nc >= 9 else nc) * 2  # BF16 copy of an iterate (rows padded)
     bounce = H * 8 + rays * (4 + 8 + 16) + 4 * A  # records, counts, offsets, directions; B^(k-1), S in; Q, B^(k) out
@@ -132,15 +133,18 @@ def _launch_bytes(kernel, sc):
         "k_trace_hemi": (n * 64 + (n - 1) * 64 + H * 8 + rays * (4 + 8 + 16) + n * 4, 1),
         "k_bounce": (bounce, nb),
         "k_bounce_persistent": (bounce * nb, 1),  # summed over the scenes of the launch
-        # transposed records, (direction, y) per ray, offsets; v^(a) tile out, u tile read + written
-        "k_adj_src": (H * 8 + rays * 32 + (n + 1) * 8 + 3 * tile, nb * T3),
-        "k_adj_ray": (rays * 32 + tile, nb * T3),   # directions + v^(a-1) tile in; y per ray out
+        # transposed records, (direction, y) per ray, offsets, the paired iterate's tile, opacity sums
+        # read + written; v^(a) tile out, u tile read + written.  3 columns, or tiles of 12 (64 B a ray)
+        "k_adj_src": (H * (8 + 8) + rays * 32 + (n + 1) * 8 + 4 * tile, nb),
+        "k_adj_src_tile": (H * (8 + 8) + rays * 64 + (n + 1) * 8 + 4 * A // T12, nb * T12),
+        # directions + v^(a-1) tile in; records out
+        "k_adj_ray": (rays * (16 + 32) + tile, nb) if C <= 3 else (rays * (16 + 64) + A // T12, nb * T12),
         # records (j) + counts + offsets + directions; four iterates of v and B tiles; g per hit out
         "k_opacity_g": (H * (8 + 4) + rays * (4 + 8 + 16) + 2 * min(nb, 4) * tile, -(-nb // 4) * T3),
-        # records (j) + g per hit, counts, offsets, directions, geometry of the hit surfels; dL/do
+        # records (j, a), g per hit, counts, offsets, directions, geometry of the hit surfels; dL/do
         "k_opacity_rec": (H * (8 + 4) + rays * (4 + 8 + 16) + n * 64 + n * 4, 1),
         # records in, transposed entries out, counts, offsets, cursors
-        "k_src_fill": (H * 16 + rays * 12 + n * 8, 1),
+        "k_src_fill": (H * 20 + rays * 12 + n * 8, 1),  # (and each record's entry)
         # center-to-center (H = pairs): the pair records written once (traversal reads are
         # the scene and tree); the bounce reads them with the iterate rows once
         "k_pair_fill": (n * 64 + (n - 1) * 64 + H * 8, 1),
@@ -165,8 +169,6 @@ def _launch_bytes(kernel, sc):
         "k_bounce_mc": (tiles * (H * 8 + rays * (4 + 8 + 16)) + A16 + 4 * A + A16, nb),
         # one tile and up to four iterates: records + ray data; v (FP32) and B (BF16) tiles; g per hit
         "k_opacity_g_mc": (H * (8 + 4) + rays * (4 + 8 + 16) + min(nb, 4) * (A + A16) // tiles, -(-nb // 4) * tiles),
-        # one tile: transposed records, directions, y; v tile out, u read + written
-        "k_adj_src_mc": (H * 8 + rays * (16 + 128) + (n + 1) * 8 + 3 * A // tiles, nb * tiles),
     }
     return table.get(kernel, (None, 0))
 
@@ -589,7 +591,7 @@ def main():
     achieved = alg_step / (ms_dom_step * 1e-3) / 1e9 if alg_step else None
     launches_dom = c_dom / args.steps
     src_file = {"k_bounce": "rgs_solve.cu", "k_adj_src": "rgs_adjoint.cu", "k_adj_ray": "rgs_adjoint.cu",
-                "k_bounce_mc": "rgs_manycol.cu", "k_opacity_g_mc": "rgs_manycol.cu", "k_adj_src_mc": "rgs_manycol.cu",
+                "k_bounce_mc": "rgs_manycol.cu", "k_opacity_g_mc": "rgs_manycol.cu", "k_adj_src_tile": "rgs_adjoint.cu",
                 "k_opacity_g": "rgs_adjoint.cu", "k_opacity_rec": "rgs_adjoint.cu",
                 "k_bounce_persistent": "rgs_batch.cu", "k_trace_hemi": "rgs_trace.cu",
                 "k_pair_fill": "rgs_pairs.cu", "k_bounce_pairs": "rgs_pairs.cu", "k_pair_grad": "rgs_pairs.cu",

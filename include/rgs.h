@@ -350,7 +350,8 @@ rgs_status rgs_set_checkpointing(rgs_transport *t, int32_t stride);
  * choices the library makes on its own: the automatic checkpoint stride (stride -1 of
  * rgs_set_checkpointing) and the number of parts rgs_adjoint splits the transposed hit
  * index into (8 bytes per hit; each part is rebuilt from the records for every transposed
- * bounce, so more parts cost time, not accuracy).  Buffers the solve needs regardless are
+ * bounce, so more parts cost time, not accuracy; in one part, 4 more bytes per hit let the
+ * opacity sums be formed with the transposed bounces, else they are gathered ray by ray).  Buffers the solve needs regardless are
  * allocated even above the budget.  Host-only.  Errors: RGS_ERR_ARG. */
 rgs_status rgs_set_memory_budget(rgs_transport *t, int64_t bytes);
 
