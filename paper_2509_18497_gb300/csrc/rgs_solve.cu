@@ -62,7 +62,8 @@ rgs_status launch_bounce(const rgs_transport *t, SceneDev sd, RaysDev rd, bool b
     // A block of a few rays per lane group: with 256 threads whatever the SH degree and ray count,
     // most of a block had no ray (4 coefficients, a thread per ray, 64 rays: 1.81 -> 0.56 ms on
     // 20,000 surfels; 16 coefficients, 32 rays: 1.06 -> 0.55), and at 256 rays the block waited for
-    // its slowest of 4 rays a group instead of 8 (3.94 -> 3.78).
+    // its slowest of 4 rays a group instead of 8 (3.94 -> 3.78,
+    // and 3.50 with 40 registers).
     const int threads = Slice<NC>::G > 1 ? (t->nd >= 128 ? 128 : 64) : (t->nd >= 64 ? 64 : 32);
     if (bf16_rows) {
         ProfScope ps_("k_bounce", st);

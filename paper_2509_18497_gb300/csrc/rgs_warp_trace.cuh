@@ -11,7 +11,8 @@
 // bound by instruction issue (73 % of the slots used; L1 50 %, L2 20 %, DRAM 5 %).  Measured,
 // thread per ray before and warp per 32 rays now: hemisphere rays of the 50,000-surfel bowl
 // (12.8 M) 40.6 -> 24.0 ms, its shadow backward 0.85 -> 0.43 ms; a 1920 x 1080 image of it
-// 7.4 -> 3.3 ms; the pair backward of 4,000 surfels 46.4 -> 23.0 ms.
+// 7.4 -> 3.3 ms; the pair backward of 4,000 surfels 46.4 -> 23.0 ms
+// (19.3 with the blocks of rgs_pairs.cu).
 #pragma once
 #include "rgs_internal.cuh"
 
@@ -30,11 +31,11 @@ struct __align__(16) WarpQueue {
 // Traversal of every lane's ray o + t d, 0 < t < tmax (lanes with active == false take part in
 // the pooled tests only).  ORDERED: nearer children first all the way, which is what makes a
 // limit found on the way cut anything off (with the waiting children in any order, half of the
-// camera directions traced an image 2-4 times slower); otherwise only the nearest is first.  test(j, ray, valid) is called by the whole warp,
-// each lane with one candidate (valid: it has one), and followed by a warp barrier; after every
-// pooled test limit(tmax) returns the lane's current tmax, so that what the tests found may
-// cut the traversal short.  Returns false if this lane's stack overflowed (part of the
-// tree was then skipped).
+// camera directions traced an image 2-4 times slower); otherwise only the nearest is first.
+// test(j, ray, valid) is called by the whole warp, each lane with one candidate (valid: it has
+// one), and followed by a warp barrier; after every pooled test limit(tmax) returns the lane's
+// current tmax, so that what the tests found may cut the traversal short.  Returns false if
+// this lane's stack overflowed (part of the tree was then skipped).
 template <bool ORDERED, class Test, class Limit>
 __device__ __forceinline__ bool warp_traverse(const SceneDev &sc, float3 o, float3 d, float tmax, bool active,
                                               WarpQueue &q, Test &&test, Limit &&limit) {
