@@ -505,7 +505,7 @@ __global__ void __launch_bounds__(SHADOW_THREADS) k_shadow_bwd(SceneDev sc, int 
                     gw = gw + make_float3(sm.gw[b][0], sm.gw[b][1], sm.gw[b][2]);
                 });
         };
-        warp_traverse<false>(sc, o, w, r, second, sm.w.q, test, [](float m) { return m; });
+        warp_traverse<false, false>(sc, o, w, r, second, sm.w.q, test, [](float m) { return m; });
     }
     if constexpr (GEO) {
         if (!lit) return;

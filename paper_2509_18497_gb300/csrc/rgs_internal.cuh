@@ -76,9 +76,9 @@ enum {
 // Node of the traversal's four-wide tree, 64 bytes (two 32-byte requests): the boxes of a
 // binary LBVH node's up to four grandchildren (a child that is a leaf stands for itself) in 8
 // bits per coordinate, org + scale q rounded outwards, on the grid of their union (whose
-// widest side is 253 steps, so a box grows by under 1 % of the node).  A traversal step costs
-// mostly what is not box arithmetic (votes, queue, stack, branches); four boxes per step
-// make half the steps of two.
+// widest side is 252 steps, so a box grows by about 1 % of the node).  Every plane also has
+// the slack that makes slab4 conservative (k_pack).  A traversal step costs mostly what is not
+// box arithmetic (votes, queue, stack, branches); four boxes per step make half the steps of two.
 struct __align__(64) BvhNode {
     float ox, oy, oz, scale;
     unsigned lox, hix, loy, hiy; // byte c: child c
@@ -527,14 +527,22 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
 
 // A ray as the slab tests use it: 1/d and -o/d.  A direction component of (nearly) zero takes
 // a huge finite reciprocal, so that no product below is 0 * inf.
+// Bound on the distance, in units of |o|_1 + R, between a hit as hit_rec computes it (the point
+// o + t d at its FP32 depth t) and the box planes as slab4 computes them; R: the sum over the axes
+// of the scene's largest coordinate.  hit_rec's t leaves the point off the surfel's plane by up to
+// 8 roundings (2^-24) of |p - o| and t, and places it in the plane to 3; slab4's plane of an axis
+// is off by |o| + 4 |org - o| + 2 t of them, beside C's rounding at |S|, 0.002 steps of the node.
+constexpr float SLAB_ERR = 1.f / (1 << 19);
 struct SlabRay {
     float3 inv, noi;
+    float wid; // by how far an origin outside the scene moves the planes (slab4<true>)
 };
 __device__ __forceinline__ SlabRay slab_ray(float3 o, float3 d) {
     auto rcp = [](float v) { return fabsf(v) > 1e-18f ? 1.f / v : copysignf(1e18f, v); };
     SlabRay r;
     r.inv = make_float3(rcp(d.x), rcp(d.y), rcp(d.z));
     r.noi = make_float3(-o.x * r.inv.x, -o.y * r.inv.y, -o.z * r.inv.z);
+    r.wid = SLAB_ERR * (fabsf(o.x) + fabsf(o.y) + fabsf(o.z));
     return r;
 }
 __device__ __forceinline__ float max3(float a, float b, float c) {
@@ -549,20 +557,27 @@ __device__ __forceinline__ float min3(float a, float b, float c) {
 }
 // plane distance of child c on one axis: byte c of w placed in a float's mantissa is
 // v = 1 + q 2^-15 (one byte permutation), so t = (org + scale q - o)/d = v S + C with
-// S = 2^15 scale/d and C = (org - o)/d - S (exact to 0.002 steps)
+// S = 2^15 scale/d and C = (org - o)/d - S (rounded at |S|: to 0.002 steps)
 __device__ __forceinline__ float slab_dist(unsigned w, int c, float S, float C) {
     return fmaf(__uint_as_float(__byte_perm(w, 0x3f800000u, 0x7604u | (c << 4))), S, C);
 }
 // Slab tests of a node's four boxes against the segment (0, tmax): bit c of the result is set
 // where box c is crossed, t[c] is then its entry distance (clamped to 0).  The near and far
 // planes are picked by the sign of d before the bytes are taken apart, which leaves two
-// three-input minima and maxima per box.  The rounding of org/d - o/d, of the order of
-// 1e-7 |o|, is within the boxes' padding, as that of (org - o)/d is.
+// three-input minima and maxima per box.  Conservative: t[c] is never behind the FP32 depth of a
+// hit inside box c, so a limit on tmax found among the hits loses none in front of it.  What
+// that takes (SLAB_ERR, C's 0.002 steps) is part of the boxes for origins within the scene
+// (k_pack), at no cost here; FAR: the origin may lie outside, its share is added to the planes.
+template <bool FAR>
 __device__ __forceinline__ unsigned slab4(const BvhNode &nd, const SlabRay &r, float tmax, float (&t)[4]) {
     const float s15 = 32768.f * nd.scale;
     const float Sx = s15 * r.inv.x, Sy = s15 * r.inv.y, Sz = s15 * r.inv.z;
     const float Cx = fmaf(nd.ox, r.inv.x, r.noi.x) - Sx, Cy = fmaf(nd.oy, r.inv.y, r.noi.y) - Sy,
                 Cz = fmaf(nd.oz, r.inv.z, r.noi.z) - Sz;
+    auto near_C = [&](float C, float inv) { return FAR ? fmaf(-r.wid, fabsf(inv), C) : C; };
+    auto far_C = [&](float C, float inv) { return FAR ? fmaf(r.wid, fabsf(inv), C) : C; };
+    const float nCx = near_C(Cx, r.inv.x), nCy = near_C(Cy, r.inv.y), nCz = near_C(Cz, r.inv.z);
+    const float fCx = far_C(Cx, r.inv.x), fCy = far_C(Cy, r.inv.y), fCz = far_C(Cz, r.inv.z);
     const bool nx = r.inv.x < 0.f, ny = r.inv.y < 0.f, nz = r.inv.z < 0.f;
     const unsigned ax = nx ? nd.hix : nd.lox, bx = nx ? nd.lox : nd.hix;
     const unsigned ay = ny ? nd.hiy : nd.loy, by = ny ? nd.loy : nd.hiy;
@@ -570,8 +585,8 @@ __device__ __forceinline__ unsigned slab4(const BvhNode &nd, const SlabRay &r, f
     unsigned hit = 0u;
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-        t[c] = fmaxf(max3(slab_dist(ax, c, Sx, Cx), slab_dist(ay, c, Sy, Cy), slab_dist(az, c, Sz, Cz)), 0.f);
-        const float f = fminf(min3(slab_dist(bx, c, Sx, Cx), slab_dist(by, c, Sy, Cy), slab_dist(bz, c, Sz, Cz)), tmax);
+        t[c] = fmaxf(max3(slab_dist(ax, c, Sx, nCx), slab_dist(ay, c, Sy, nCy), slab_dist(az, c, Sz, nCz)), 0.f);
+        const float f = fminf(min3(slab_dist(bx, c, Sx, fCx), slab_dist(by, c, Sy, fCy), slab_dist(bz, c, Sz, fCz)), tmax);
         if (t[c] <= f) hit |= 0x11u << c;
     }
     return hit & nd.mask;

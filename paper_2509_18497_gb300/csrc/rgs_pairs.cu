@@ -550,7 +550,7 @@ __global__ void __launch_bounds__(PT, 7) k_pair_grad(SceneDev sc, int n, int chu
                         gd = gd + make_float3(smw.gd[b][0], smw.gd[b][1], smw.gd[b][2]);
                     });
             };
-            if (!warp_traverse<false>(sc, pi, d, r, second, sm.p.w.q, test, [](float m) { return m; })) atomicAdd(&flags[FLAG_STACK], 1);
+            if (!warp_traverse<false, false>(sc, pi, d, r, second, sm.p.w.q, test, [](float m) { return m; })) atomicAdd(&flags[FLAG_STACK], 1);
         }
         if constexpr (GEO) {
             if (live) {

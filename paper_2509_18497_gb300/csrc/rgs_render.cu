@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(RN_THREADS, RN_MINB) k_render(SceneDev sc, Cam
         for (bool first = true; __any_sync(WT_FULL, more); first = false) {
             bool full;
             const int lg0 = first ? 0 : (int)(65536.f * __log2f(fmaxf(T, 1e-30f)));
-            if (!warp_collect<true>(sc, o, d, -1, more, eps, lg0, sm, list, full)) atomicAdd(&flags[FLAG_STACK], 1);
+            if (!warp_collect<true, true>(sc, o, d, -1, more, eps, lg0, sm, list, full)) atomicAdd(&flags[FLAG_STACK], 1);
             const unsigned rays = __ballot_sync(WT_FULL, more), fulls = __ballot_sync(WT_FULL, full);
             more = false;
             for (unsigned m = rays; m; m &= m - 1) {

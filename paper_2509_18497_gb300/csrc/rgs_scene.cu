@@ -303,9 +303,19 @@ __global__ void k_refit(int n, const int2 *__restrict__ kids, const int *__restr
 // leaf stands for itself), their boxes in 8 bits per coordinate, rounded outwards on the grid
 // of their union.  Infinite sides are cut at 1e18 (the node then covers everything).  A walk
 // from the root only meets nodes of even depth; the others are written all the same.
+// Each plane moves outwards by what makes slab4 conservative for rays that start in the scene
+// (|o|_1 + R <= 2 R), SLAB_ERR 2 R, and keeps at least 0.01 steps more to the stored plane for the
+// rounding of slab4's C: the grid starts half a step in front of the union, and 0.01 is taken
+// off (added) before rounding down (up).  Without this a ray's bound at its 96th hit cuts off
+// nodes with nearer hits inside (a bowl of 16,648 surfels with 2,113 such rays: one receiver's B
+// off by a third).  The boxes of a 10-unit scene grow by 4e-5.
+constexpr float PACK_SLACK = 0.01f;
 __global__ void k_pack(int n, const int2 *__restrict__ kids, const float *__restrict__ boxes, BvhNode *nodes) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n - 1) return;
+    float R = 0.f; // over the root's box
+    for (int a = 0; a < 3; ++a) R += fminf(fmaxf(fabsf(boxes[a]), fabsf(boxes[3 + a])), 1e18f);
+    const float pad = 2.f * SLAB_ERR * R;
     const int2 c = kids[i];
     int kid[4], m = 0;
     const int two[2] = {c.x, c.y};
@@ -323,22 +333,23 @@ __global__ void k_pack(int n, const int2 *__restrict__ kids, const float *__rest
         float l = INFINITY, h = -INFINITY;
         for (int q = 0; q < m; ++q) {
             const float *b = boxes + (size_t)(kid[q] < 0 ? (n - 1 + ~kid[q]) : kid[q]) * 6;
-            lo[q][a] = fmaxf(b[a], -1e18f);
-            hi[q][a] = fminf(b[3 + a], 1e18f);
+            lo[q][a] = fmaxf(b[a] - pad, -1e18f);
+            hi[q][a] = fminf(b[3 + a] + pad, 1e18f);
             l = fminf(l, lo[q][a]);
             h = fmaxf(h, hi[q][a]);
         }
         org[a] = l;
         ext = fmaxf(ext, h - l);
     }
-    const float scale = fmaxf(ext / 253.f, 1e-30f), inv = 1.f / scale;
+    const float scale = fmaxf(ext / 252.f, 1e-30f), inv = 1.f / scale;
+    for (int a = 0; a < 3; ++a) org[a] -= 0.5f * scale;
     unsigned wl[3] = {0u, 0u, 0u}, wh[3] = {0u, 0u, 0u}, mask = 0u;
     BvhNode out;
     for (int q = 0; q < 4; ++q) out.kid[q] = 0;
     for (int q = 0; q < m; ++q) {
         for (int a = 0; a < 3; ++a) {
-            int ql = min(max((int)floorf((lo[q][a] - org[a]) * inv), 0), 255);
-            int qh = min(max((int)ceilf((hi[q][a] - org[a]) * inv), 0), 255);
+            int ql = min(max((int)floorf((lo[q][a] - org[a]) * inv - PACK_SLACK), 0), 255);
+            int qh = min(max((int)ceilf((hi[q][a] - org[a]) * inv + PACK_SLACK), 0), 255);
             while (ql > 0 && org[a] + scale * (float)ql > lo[q][a]) --ql;
             while (qh < 255 && org[a] + scale * (float)qh < hi[q][a]) ++qh;
             wl[a] |= (unsigned)ql << (8 * q);

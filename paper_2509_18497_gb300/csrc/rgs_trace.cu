@@ -59,7 +59,7 @@ __global__ void __launch_bounds__(HEMI_THREADS, RGS_TRACE_MINB) k_trace_hemi(Sce
         const float3 d = ray_dir(rays.seed, sc.uid[i], q, rays.na, rays.nbs, f3(sc.FU[i]), f3(sc.FV[i]), f3(sc.N4[i]));
         if (active) dir_out[r] = make_float4(d.x, d.y, d.z, 0.f);
         bool full;
-        if (!warp_collect<false>(sc, o, d, i, active, eps, 0, sm, list, full)) atomicAdd(&flags[FLAG_STACK], 1);
+        if (!warp_collect<false, false>(sc, o, d, i, active, eps, 0, sm, list, full)) atomicAdd(&flags[FLAG_STACK], 1);
         int kept = 0; // of this lane's ray
         for (int x = 0; x < 32; ++x) {
             int H = sm.cnt[x];

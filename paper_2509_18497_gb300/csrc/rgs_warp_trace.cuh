@@ -34,9 +34,10 @@ struct __align__(16) WarpQueue {
 // camera directions traced an image 2-4 times slower); otherwise only the nearest is first.
 // test(j, ray, valid) is called by the whole warp, each lane with one candidate (valid: it has
 // one), and followed by a warp barrier; after every pooled test limit(tmax) returns the lane's
-// current tmax, so that what the tests found may cut the traversal short.  Returns false if
-// this lane's stack overflowed (part of the tree was then skipped).
-template <bool ORDERED, class Test, class Limit>
+// current tmax, so that what the tests found may cut the traversal short (no hit up to tmax is
+// lost to it: slab4 is conservative).  FAR: the origin may lie outside the scene.  Returns false
+// if this lane's stack overflowed (part of the tree was then skipped).
+template <bool ORDERED, bool FAR, class Test, class Limit>
 __device__ __forceinline__ bool warp_traverse(const SceneDev &sc, float3 o, float3 d, float tmax, bool active,
                                               WarpQueue &q, Test &&test, Limit &&limit) {
     const int lane = threadIdx.x & 31;
@@ -60,7 +61,7 @@ __device__ __forceinline__ bool warp_traverse(const SceneDev &sc, float3 o, floa
         int kid[4];
         if (node >= 0) {
             const BvhNode nd = ld_node(sc, node);
-            hit = slab4(nd, ray, tmax, t);
+            hit = slab4<FAR>(nd, ray, tmax, t);
 #pragma unroll
             for (int c = 0; c < 4; ++c) kid[c] = nd.kid[c];
         }
@@ -126,7 +127,7 @@ __device__ __forceinline__ bool warp_traverse(const SceneDev &sc, float3 o, floa
         while (next < 0 && sp > 0) { // the last waiting node that the limit has not passed
             --sp;
             const int2 e = sp < WT_SMEM_STACK ? q.stack[sp][lane] : deep[sp - WT_SMEM_STACK];
-            if (__int_as_float(e.y) <= tmax) next = e.x;
+            if (__int_as_float(e.y & ~3) <= tmax) next = e.x; // (the lowest bits are the child's number)
         }
         node = next;
     }
@@ -192,7 +193,7 @@ __device__ __forceinline__ bool warp_transmittance(const SceneDev &sc, WarpOcclu
             else T *= om;
         });
     };
-    return warp_traverse<false>(sc, o, d, tmax, active, s.q, test, [](float m) { return m; });
+    return warp_traverse<false, false>(sc, o, d, tmax, active, s.q, test, [](float m) { return m; });
 }
 
 // ------------------------------------------------------------------ ordered compositing
@@ -270,7 +271,8 @@ struct WarpHits {
 // s.cnt.  lg0: log2 of the transmittance in front (log_transmit's steps).  A ray's traversal
 // ends once the hits found make the rest invisible.  full: this lane's ray had more than
 // RGS_HMAX (in front of that end).  Returns false if this lane's stack overflowed.
-template <bool LOWER>
+// LOWER: `lower` is looked at; FAR: o may lie outside the scene (a camera).
+template <bool LOWER, bool FAR>
 __device__ __forceinline__ bool warp_collect(const SceneDev &sc, float3 o, float3 d, int self, bool active, float eps,
                                              int lg0, WarpHits &s, int4 *lists, bool &full) {
     const int lane = threadIdx.x & 31;
@@ -308,7 +310,7 @@ __device__ __forceinline__ bool warp_collect(const SceneDev &sc, float3 o, float
         __syncwarp();
         return tmax;
     };
-    return warp_traverse<true>(sc, o, d, INFINITY, active, s.q, test, limit);
+    return warp_traverse<true, FAR>(sc, o, d, INFINITY, active, s.q, test, limit);
 }
 
 // One ray's H <= 32 K collected hits, put in depth order (ascending t; runs of near-equal depth
