@@ -305,9 +305,9 @@ typedef struct rgs_batch_opts {
  *   opts      : host, may be NULL (FP32, graph, autotune, default wait limit).
  *   B_out     : host array of count device pointers [N_s][nc_s][C_s] (entries may be NULL), or NULL.
  *   residual_norms : host [count][RGS_MAX_BOUNCES] FP64 norms per bounce, or NULL.
- * Launch plans (device descriptors, graph, tuned shape) are cached per set of transports, bounce
- * counts, precision and wait limit (E and B_out may change from call to call); the first call
- * with a new set also runs the autotuning candidates.  Synchronises `stream` (the
+ * Launch plans (device descriptors, graph, tuned shape) are cached per set of transports (as last
+ * built and traced), bounce counts, precision and wait limit (E and B_out may change from call to
+ * call); the first call with a new set also runs the autotuning candidates.  Synchronises `stream` (the
  * device-side timeout flag is read back).  Errors: RGS_ERR_ARG, RGS_ERR_STATE (untraced
  * transport), RGS_ERR_OOM, RGS_ERR_CUDA, RGS_ERR_TIMEOUT (a barrier wait ran out; the iterates
  * of the batch are then invalid, the context stays usable). */

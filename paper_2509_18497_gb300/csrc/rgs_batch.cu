@@ -346,26 +346,25 @@ rgs_status rgs_solve_batched_impl(rgs_transport *const *tsp, int count, const fl
     for (int s = 0; s < count; ++s)
         if ((r = rgs_solve_prepare(ts[s], nbs[s], precision, 0, st)) != RGS_OK) return r;
 
-    // plan: keyed by every pointer and size the launches bake in
+    // plan: keyed by everything of a descriptor that the launches bake in.  Handles are rebuilt
+    // in place, in buffers that only grow: the pointers alone do not tell another SH degree or
+    // opacity model from the last one.  (E and B_out are read and written outside the captured launches.)
     std::vector<const void *> key;
-    key.push_back((const void *)(size_t)precision);
-    key.push_back((const void *)(size_t)spin_limit);
+    auto add = [&](auto... v) { (key.push_back((const void *)(size_t)v), ...); };
+    add(precision, spin_limit);
     for (int s = 0; s < count; ++s) {
-        key.push_back(ts[s]);
-        key.push_back((const void *)(size_t)ts[s]->n);
-        key.push_back((const void *)(size_t)ts[s]->nd);
-        key.push_back((const void *)(size_t)ts[s]->C);
-        key.push_back(ts[s]->sc->P);
-        key.push_back(ts[s]->sc->nodes);
-        key.push_back(ts[s]->sc->rec);
-        key.push_back(ts[s]->off);
-        key.push_back(ts[s]->dir);
-        key.push_back(ts[s]->Q);
-        key.push_back(ts[s]->iters);
-        key.push_back(ts[s]->iters16);
-        key.push_back(ts[s]->rec_ja);
-        key.push_back((const void *)(size_t)nbs[s]);
-    } // (E and B_out are read and written outside the captured launches)
+        const rgs_transport *t = ts[s];
+        const SceneDev sd = t->sc->dev();
+        const RaysDev rd = t->rays();
+        key.push_back(t);
+        add(t->n, t->nd, t->C, t->nc, nbs[s], sd.n, sd.L, sd.alpha_model, rd.na, rd.nbs);
+        for (const void *p : {(const void *)sd.P, (const void *)sd.N4, (const void *)sd.FU, (const void *)sd.FV,
+                              (const void *)sd.rec, (const void *)sd.cl, (const void *)sd.uid, (const void *)sd.inv,
+                              (const void *)sd.nodes, (const void *)sd.eps_plane, (const void *)rd.rec_ja,
+                              (const void *)rd.off, (const void *)rd.cnt, (const void *)rd.dir, (const void *)t->Q,
+                              (const void *)t->iters, (const void *)t->iters16, (const void *)t->norm2})
+            key.push_back(p);
+    }
     std::lock_guard<std::mutex> lk(g_plan_mu);
     Plan *P = g_plans.count(key) ? g_plans[key] : nullptr;
     const bool fresh = (P == nullptr);
