@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(RN_THREADS, RN_MINB) k_render(SceneDev sc, Cam
                 float Tq = __shfl_sync(WT_FULL, T, q);
                 unsigned long long last = 0ull;
                 int kept = 0;
-                if (n > 0) kept = warp_composite_any(sc, n, list + q * WT_LIST, sm, cut, Tq, last);
+                if (n > 0) kept = warp_composite_any(sc, n, list + q * WT_LIST, sm, cut, true, Tq, last);
                 __syncwarp();
                 if (lane == q) {
                     T = Tq;

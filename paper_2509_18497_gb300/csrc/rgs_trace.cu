@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(HEMI_THREADS, RGS_TRACE_MINB) k_trace_hemi(Sce
             if (H == 0) continue;
             float T = 1.f;
             unsigned long long last;
-            const int k = warp_composite_any(sc, H, list + x * WT_LIST, sm, false, T, last);
+            const int k = warp_composite_any(sc, H, list + x * WT_LIST, sm, false, false, T, last);
             __syncwarp();
             if (lane == x) {
                 kept = k;

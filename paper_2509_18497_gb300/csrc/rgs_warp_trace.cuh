@@ -199,9 +199,10 @@ __device__ __forceinline__ bool warp_transmittance(const SceneDev &sc, WarpOcclu
 // ------------------------------------------------------------------ ordered compositing
 // log2(1 - alpha) in steps of 2^-16, for the early-out bound only (a fast approximation; whole
 // numbers, because shared memory adds those in one instruction and floats in a
-// compare-and-swap loop).  An opaque hit counts as 2^-24; an alpha above 1 (NaN) as 2^24, no bound.
+// compare-and-swap loop).  An opaque hit counts as 2^-24, and so does an alpha above 1: the
+// transmittance behind it is below the cut.  A NaN counts as 2^24, no bound.
 __device__ __forceinline__ int log_transmit(float alpha) {
-    return (int)(65536.f * fmaxf(fminf(__log2f(1.f - alpha), 24.f), -24.f));
+    return (int)(65536.f * (alpha > 1.f ? -24.f : fmaxf(fminf(__log2f(1.f - alpha), 24.f), -24.f)));
 }
 // Once the hits found so far on a ray multiply to a transmittance below RGS_T_EPS, no hit
 // behind the farthest of them is composited, so the ray may end there.  -20.2 leaves a
@@ -315,15 +316,17 @@ __device__ __forceinline__ bool warp_collect(const SceneDev &sc, float3 o, float
 
 // One ray's H <= 32 K collected hits, put in depth order (ascending t; runs of near-equal depth
 // by caller index) and composited by the whole warp: (j, a_h) to the first half of
-// list[0 .. kept).  Returns kept, the hits in front of the transmittance cut; T: the
-// transmittance in front of the ray's first hit, and then behind its last.  cut: the last
+// list[0 .. kept).  Returns kept, the hits up to the first whose transmittance in front is below
+// the cut (an alpha above 1 makes the product negative, and a second one positive again); T: the
+// transmittance in front of the ray's first hit, and then behind its last (0 where the list ended
+// before).  nan_ends: whether a NaN transmittance ends the list.  cut: the last
 // run of near-equal depths may go on behind the list, so it is left out (unless it is the whole
 // list); H becomes the hits that count and last the largest key (depth bits, surfel) among them.
 // K hits per lane; all lanes call.  sa, su: RGS_HMAX more words of shared memory each (the
 // traversal's stack, which is empty by now).
 template <int K>
 __device__ __forceinline__ int warp_composite(const SceneDev &sc, int &H, int4 *list, WarpSort &s, float *sa, int *su,
-                                              bool cut, float &T, unsigned long long &last) {
+                                              bool cut, bool nan_ends, float &T, unsigned long long &last) {
     const int lane = threadIdx.x & 31;
     float t[K], al[K];
     int j[K], rank[K];
@@ -457,21 +460,23 @@ __device__ __forceinline__ int warp_composite(const SceneDev &sc, int &H, int4 *
         }
         float exc = __shfl_up_sync(WT_FULL, inc, 1);
         exc = T * (lane == 0 ? 1.f : exc);
-        const bool keep = e < H && exc >= RGS_T_EPS;
-        if (keep) *reinterpret_cast<int2 *>(&list[e]) = make_int2(j[k], __float_as_int(al[k] * exc));
-        kept += __popc(__ballot_sync(WT_FULL, keep));
+        const unsigned ends = __ballot_sync(WT_FULL, e >= H || (nan_ends ? !(exc >= RGS_T_EPS) : exc < RGS_T_EPS));
+        const int here = kept == 32 * k ? (ends ? __ffs(ends) - 1 : 32) : 0; // (nothing behind an end)
+        if (lane < here) *reinterpret_cast<int2 *>(&list[e]) = make_int2(j[k], __float_as_int(al[k] * exc));
+        kept += here;
         T *= __shfl_sync(WT_FULL, inc, 31);
     }
+    if (kept < H) T = 0.f;
     return kept;
 }
 
 __device__ __forceinline__ int warp_composite_any(const SceneDev &sc, int &H, int4 *list, WarpHits &s, bool cut,
-                                                  float &T, unsigned long long &last) {
+                                                  bool nan_ends, float &T, unsigned long long &last) {
     float *sa = reinterpret_cast<float *>(&s.q.stack[0][0]);
     int *su = reinterpret_cast<int *>(sa + RGS_HMAX);
-    if (H <= 32) return warp_composite<1>(sc, H, list, s.sort, sa, su, false, T, last); // (cut lists are full)
-    if (H <= 64) return warp_composite<2>(sc, H, list, s.sort, sa, su, false, T, last);
-    return warp_composite<3>(sc, H, list, s.sort, sa, su, cut, T, last);
+    if (H <= 32) return warp_composite<1>(sc, H, list, s.sort, sa, su, false, nan_ends, T, last); // (cut lists are full)
+    if (H <= 64) return warp_composite<2>(sc, H, list, s.sort, sa, su, false, nan_ends, T, last);
+    return warp_composite<3>(sc, H, list, s.sort, sa, su, cut, nan_ends, T, last);
 }
 // the composited hit e of a list
 __device__ __forceinline__ int2 wt_hit(const int4 *list, int e) { return *reinterpret_cast<const int2 *>(&list[e]); }
