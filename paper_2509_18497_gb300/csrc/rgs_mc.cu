@@ -544,15 +544,17 @@ template <int T> __device__ __forceinline__ LumIdx lum_block(LumIdx x, LumIdx *s
 // The luminances are kept beside dB: a shot changes the rows of its receivers, whose warps have
 // the new values in hand, so the search for the next shot reads 8 bytes per surfel instead of
 // a row.  The sum of lum(c) |x| over a row is formed in whole numbers, at least as exact as adding
-// in FP64: a column's 24-bit significands, aligned to its largest exponent with 8 bits below,
-// times its weight in units of 2^-27; the columns aligned to the row's largest exponent in 128
-// bits.  It is handed on as the bits of the double it truncates to.
+// in FP64: a column's 24-bit significands, aligned to its largest exponent with 36 bits below
+// (what is cut off is under 2^-55 of the column, a rounding in FP64 up to 2^-53), times its
+// weight in units of 2^-27; the columns aligned to the row's largest exponent in 128 bits.  It is
+// handed on as the bits of the double it truncates to.
 struct LumSum {
-    unsigned __int128 sum = 0; // in units of 2^(top - 150 - 8 - 27 - LUM_BELOW)
+    unsigned __int128 sum = 0; // in units of 2^(top - 150 - LUM_COLUMN - 27 - LUM_BELOW)
     int top = 0;
     unsigned bad = 0; // 1: an infinity, 2: a NaN
 };
-constexpr int LUM_BELOW = 40; // 24 + 4 + 8 + 27 bits of a column, 40 below, 15 for the count of columns
+// 128 bits: 24 + 36 + 4 (the count of coefficients) + 27 of a column, 22 below, 15 for the count of columns
+constexpr int LUM_COLUMN = 36, LUM_BELOW = 22;
 __device__ __forceinline__ void lum_align(LumSum &s, int top) {
     const int d = top - s.top;
     s.sum = d > 127 ? 0 : s.sum >> d;
@@ -568,16 +570,16 @@ template <int NC> __device__ __forceinline__ void lum_column(LumSum &s, const fl
         ex[k] = max((int)(b >> 23), 1);
         top = max(top, ex[k]);
     }
-    unsigned long long t = 0ull; // 24 + 8 + 4 bits
+    unsigned long long t = 0ull; // 24 + 36 + 4 bits
 #pragma unroll
     for (int k = 0; k < NC; ++k) {
         const unsigned b = __float_as_uint(x[k]) & 0x7fffffffu;
         const unsigned m = (b & 0x7fffffu) | (b >= 0x800000u ? 0x800000u : 0u);
         const int d = top - ex[k];
-        t += d > 31 ? 0u : (m << 8) >> d;
+        t += d > 63 ? 0ull : ((unsigned long long)m << LUM_COLUMN) >> d;
     }
     const unsigned w27 = (unsigned)(lum_w(c) * 134217728.f); // (exact)
-    const unsigned __int128 p = (unsigned __int128)(t * w27) << LUM_BELOW; // 63 bits before the shift
+    const unsigned __int128 p = (unsigned __int128)t * w27 << LUM_BELOW; // 91 bits before the shift
     if (top > s.top) lum_align(s, top);
     const int d = s.top - top;
     if (d <= 127) s.sum += p >> d;
@@ -603,7 +605,7 @@ __device__ __forceinline__ unsigned long long lum_bits(const LumSum &s, int base
     if (!t.sum) return 0ull;
     const unsigned long long hi = (unsigned long long)(t.sum >> 64);
     const int z = hi ? __clzll((long long)hi) : 64 + __clzll((long long)(unsigned long long)t.sum);
-    const int e = 1023 + (127 - z) + t.top - 150 - 8 - 27 - LUM_BELOW; // > 0: floats are far above FP64's least
+    const int e = 1023 + (127 - z) + t.top - 150 - LUM_COLUMN - 27 - LUM_BELOW; // > 0: floats are far above FP64's least
     const unsigned long long lead = (unsigned long long)((t.sum << z) >> 64);
     return (unsigned long long)e << 52 | (lead << 1) >> 12;
 }
