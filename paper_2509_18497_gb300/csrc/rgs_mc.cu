@@ -813,7 +813,9 @@ rgs_status cluster_shots(rgs_transport *t, const int2 *tr, int shots, unsigned l
     attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
     const void *fn = (const void *)k_pr_shoot<NC>;
     if (cfg.dynamicSmemBytes > SHOOT_MAX_SMEM) return RGS_OK;
-    RGS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes));
+    // (the same value in every call: the attribute is the function's, and another thread's call with
+    // less shared memory must not lower it before this one launches)
+    RGS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SHOOT_MAX_SMEM));
     RGS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     int fit = 0;
     unsigned blocks = 16;
