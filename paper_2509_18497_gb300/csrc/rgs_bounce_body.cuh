@@ -245,8 +245,7 @@ __device__ __forceinline__ void bounce_receiver_mc(const SceneDev &sc, const Ray
             for (int q = 0; q < m; q += HALF ? 2 : 1) { // HALF: the upper 16 lanes take the next hit
                 const int h = HALF ? q + (lane >> 4) : q, hc = HALF ? min(h, m - 1) : h;
                 const int j = __shfl_sync(0xffffffffu, rec.x, hc);
-                const float aw = __int_as_float(__shfl_sync(0xffffffffu, rec.y, hc));
-                const float a = HALF && h >= m ? 0.f : aw;
+                const float a = __int_as_float(__shfl_sync(0xffffffffu, rec.y, hc));
                 if constexpr (COOP) {
                     x += a * TileDot<T, NC>::dot(Bg + ((size_t)j * C + tile * 32) * RS, ncols, lane, ys);
                 } else {
@@ -255,7 +254,7 @@ __device__ __forceinline__ void bounce_receiver_mc(const SceneDev &sc, const Ray
                     float s = 0.f;
 #pragma unroll
                     for (int k = 0; k < NC; ++k) s += Yo[k] * v[k];
-                    x += a * s;
+                    if (!HALF || h < m) x += a * s; // (no weight of 0: the row may hold an infinity)
                 }
             }
         }
