@@ -190,7 +190,8 @@ rgs_status rgs_trace_transport(rgs_scene *scene, const rgs_lights *lights, const
  * c = 0.03279 o^3.4 and Ein(c) = int_0^c (1 - e^{-y}) / y dy.  The direct term is that of rgs_trace_transport.  The result is a transport
  * handle that rgs_solve, rgs_get_iterate and rgs_adjoint accept (every iterate is kept;
  * rgs_solve_batched does not take it).  Cost: N^2 front tests and one segment trace per
- * front pair; memory 8 bytes per pair.
+ * front pair; memory 8 bytes per pair, and 4 more (the segment's transmittance, which saves the
+ * adjoint a trace) where that is at most a sixteenth of the free memory and within the budget.
  *   opts : host, may be NULL (lambda = 1).  Other arguments as rgs_trace_transport.
  * Synchronises `stream` (the pair count decides the buffer size).  Errors: RGS_ERR_ARG,
  * RGS_ERR_OOM, RGS_ERR_CUDA, RGS_ERR_CAPACITY (traversal stack). */

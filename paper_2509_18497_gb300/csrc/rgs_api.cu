@@ -582,6 +582,7 @@ void rgs_destroy_transport(rgs_transport *t) {
     dev_free(t->dir);
     dev_free(t->pair_off);
     dev_free(t->pair_rec);
+    dev_free(t->pair_T);
     dev_free(t->chunk_off);
     dev_free(t->chunk_cnt);
     dev_free(t->chunk_tmp);

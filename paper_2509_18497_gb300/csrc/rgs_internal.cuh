@@ -656,6 +656,10 @@ struct rgs_transport {
     long long *pair_off = nullptr;
     int2 *pair_rec = nullptr;
     long long pair_cap = 0, n_pairs = 0;
+    // transmittance of every pair's segment (0: an opaque occluder, or below FP32's range), kept for
+    // the adjoint where there is room for it
+    float *pair_T = nullptr;
+    long long pair_T_cap = 0;
     long long *chunk_off = nullptr;
     int *chunk_cnt = nullptr;
     long long chunk_cap = 0;

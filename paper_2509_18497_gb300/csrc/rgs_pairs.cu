@@ -155,7 +155,7 @@ struct PairWarp {
 constexpr size_t PAIR_FILL_SMEM = sizeof(PairChunk) + (PT / 32) * sizeof(PairWarp);
 __global__ void __launch_bounds__(PT, 6) k_pair_fill(SceneDev sc, int n, int chunks, int pch, const long long *__restrict__ chunk_off,
                                                    const float *__restrict__ lam, const float *__restrict__ aarea,
-                                                   int2 *rec, int *flags) {
+                                                   int2 *rec, float *pt, int *flags) {
     extern __shared__ __align__(16) unsigned char pair_smem[];
     PairChunk &ck = *reinterpret_cast<PairChunk *>(pair_smem);
     PairWarp &sm = reinterpret_cast<PairWarp *>(pair_smem + sizeof(PairChunk))[threadIdx.x >> 5];
@@ -185,6 +185,7 @@ __global__ void __launch_bounds__(PT, 6) k_pair_fill(SceneDev sc, int n, int chu
             const float geo = fabsf(dot3(ni, d)) * fabsf(dot3(nj, d)) / (r * r);
             const float V = __ldg(&lam[j]) * __ldg(&aarea[j]) * T * geo;
             rec[chunk_off[blk] + rank] = make_int2(j, __float_as_int(V));
+            if (pt) pt[chunk_off[blk] + rank] = T;
         }
     }
 }
@@ -410,10 +411,9 @@ __global__ void __launch_bounds__(PAIR_THREADS) k_pair_g(SceneDev sc, int C, int
 // and source chunk, the front sources packed, a lane per source):
 //   dL/dlambda_j += g A_j T geo,  dL/do_j += g lambda_j (A_j/o_j) T geo,
 //   dL/do_k += -g lambda_j A_j geo prod_{m != k}(1 - alpha_m) G_k for the segment's occluders.
-// T is V / (lambda_j A_j geo) from the pair's record, so the segment is traced once, for its
-// occluders; only where the record is 0 (an opaque occluder, a T below FP32's range, lambda = 0)
-// does a first trace find T and the zero factors (the 20k-bowl's backward used to trace every
-// segment twice).
+// T is the fill's (pt, 4 bytes a pair), so the segment is traced once, for its occluders; where it
+// is 0 (an opaque occluder, a product below FP32's range), or was not kept, a first trace finds T and
+// the zero factors (4,000 surfels: 20.4 ms with T kept, 36.0 without).
 // With dp (and ds) also the geometry gradients of Eqs. dl-dgeo-0/1: the decay term
 // V = lambda_j A_j T geo through geo = (n_i.d)|n_j.d|/r^2, through A_j (proportional to
 // s^u_j s^v_j) and through every occluder's crossing point and scales, plus the directional
@@ -431,7 +431,7 @@ template <bool GEO>
 constexpr size_t PAIR_GRAD_SMEM = sizeof(PairChunk) + (PT / 32) * (GEO ? sizeof(PairGeoWarp) : sizeof(PairGradWarp));
 template <bool GEO>
 __global__ void __launch_bounds__(PT, 7) k_pair_grad(SceneDev sc, int n, int chunks, int pch, const long long *__restrict__ chunk_off,
-                                                   const int2 *__restrict__ rec, const float *__restrict__ lam,
+                                                   const float *__restrict__ pt, const float *__restrict__ lam,
                                                    const float *__restrict__ aarea, const float *__restrict__ daarea,
                                                    const float *__restrict__ gpair, const float4 *__restrict__ gq,
                                                    float *dop, float *dlam, float *dp, float *ds, float *gF, int *flags) {
@@ -466,10 +466,8 @@ __global__ void __launch_bounds__(PT, 7) k_pair_grad(SceneDev sc, int n, int chu
             const float4 x = sm.p.pj[ray];
             return pair_occludes(k, s, __float_as_int(x.w), f3(x), eps);
         };
-        // T from the record; a record of (nearly) 0 says too little about it
-        const float V = __int_as_float(__ldg(&rec[e].y)), den = lj * Aj * geo;
-        const bool known = fabsf(V) > 1e-30f && fabsf(den) > 1e-30f;
-        float Tnz = known ? V / den : 0.f;
+        float Tnz = pt ? __ldg(&pt[e]) : 0.f;
+        const bool known = Tnz != 0.f;
         int nzero = 0;
         if (__any_sync(WT_FULL, live && !known)) {
             float T1;
@@ -625,6 +623,25 @@ __global__ void k_lam_out(int n, const int *__restrict__ uid, const float *__res
 } // namespace
 
 // ------------------------------------------------------------------ host side
+// Room for the segments' transmittances beside `total` pair records: within the memory budget and at
+// most a sixteenth of the free memory, so that what the solve and the adjoint need (28 bytes a
+// pair more with geometry gradients) finds its place as without them.  None: t->pair_T is null.
+static void keep_pair_T(rgs_transport *t, long long total) {
+    const long long others = t->device_bytes - 4 * t->pair_T_cap, bytes = 4 * std::max(total, 1ll);
+    bool room = t->mem_budget <= 0 || others + bytes <= t->mem_budget;
+    if (room && total <= t->pair_T_cap) return;
+    if (t->pair_T) {
+        t->device_bytes -= (long long)rgs_alloc_forget(t->pair_T);
+        cudaFree(t->pair_T);
+        t->pair_T = nullptr;
+        t->pair_T_cap = 0;
+    }
+    size_t free_b = 0, total_b = 0;
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) cudaGetLastError();
+    if (room && bytes <= (long long)(free_b / 16) && dev_alloc(&t->pair_T, (size_t)total, &t->device_bytes) == RGS_OK)
+        t->pair_T_cap = std::max(total, 1ll);
+}
+
 rgs_status rgs_trace_pairs_impl(rgs_transport *t, const rgs_lights *L, const float *lambda, cudaStream_t st) {
     rgs_status r;
     t->kind = RGS_KIND_PAIRS;
@@ -670,12 +687,13 @@ rgs_status rgs_trace_pairs_impl(rgs_transport *t, const rgs_lights *L, const flo
         if ((r = dev_alloc(&t->pair_rec, (size_t)total, &t->device_bytes)) != RGS_OK) return r;
         t->pair_cap = total;
     }
+    keep_pair_T(t, total);
     t->n_pairs = total;
     t->n_hits = total;
     t->n_slots = total;
     t->n_full = 0;
     RGS_CUDA(cudaFuncSetAttribute(k_pair_fill, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PAIR_FILL_SMEM));
-    { ProfScope ps_("k_pair_fill", st); k_pair_fill<<<(unsigned)nchunk, PT, PAIR_FILL_SMEM, st>>>(sd, n, chunks, pch, t->chunk_off, t->lam, t->aarea, t->pair_rec, t->flags); }
+    { ProfScope ps_("k_pair_fill", st); k_pair_fill<<<(unsigned)nchunk, PT, PAIR_FILL_SMEM, st>>>(sd, n, chunks, pch, t->chunk_off, t->lam, t->aarea, t->pair_rec, t->pair_T, t->flags); }
     { ProfScope ps_("k_pair_off", st); k_pair_off<<<(n + 256) / 256, 256, 0, st>>>(t->chunk_off, chunks, n, t->pair_off); }
     RGS_LAUNCH("pair fill");
     if ((r = rgs_direct_term(t, st)) != RGS_OK) return r;
@@ -758,11 +776,11 @@ rgs_status run_adjoint_pairs(rgs_transport *t, const float *g, float *dE, float 
         if (geo.dp) {
             RGS_CUDA(cudaFuncSetAttribute(k_pair_grad<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PAIR_GRAD_SMEM<true>));
             ProfScope ps_("k_pair_grad", st);
-            k_pair_grad<true><<<(unsigned)((long long)n * chunks), PT, PAIR_GRAD_SMEM<true>, st>>>(sd, n, chunks, pch, t->chunk_off, t->pair_rec, t->lam, t->aarea, t->daarea, t->gh, geo.gq, dopo ? t->dop : nullptr, dlam_acc, geo.dp, geo.ds, geo.gF, t->flags);
+            k_pair_grad<true><<<(unsigned)((long long)n * chunks), PT, PAIR_GRAD_SMEM<true>, st>>>(sd, n, chunks, pch, t->chunk_off, t->pair_T, t->lam, t->aarea, t->daarea, t->gh, geo.gq, dopo ? t->dop : nullptr, dlam_acc, geo.dp, geo.ds, geo.gF, t->flags);
         } else {
             RGS_CUDA(cudaFuncSetAttribute(k_pair_grad<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PAIR_GRAD_SMEM<false>));
             ProfScope ps_("k_pair_grad", st);
-            k_pair_grad<false><<<(unsigned)((long long)n * chunks), PT, PAIR_GRAD_SMEM<false>, st>>>(sd, n, chunks, pch, t->chunk_off, t->pair_rec, t->lam, t->aarea, t->daarea, t->gh, nullptr, dopo ? t->dop : nullptr, dlam_acc, nullptr, nullptr, nullptr, t->flags);
+            k_pair_grad<false><<<(unsigned)((long long)n * chunks), PT, PAIR_GRAD_SMEM<false>, st>>>(sd, n, chunks, pch, t->chunk_off, t->pair_T, t->lam, t->aarea, t->daarea, t->gh, nullptr, dopo ? t->dop : nullptr, dlam_acc, nullptr, nullptr, nullptr, t->flags);
         }
         RGS_LAUNCH("pair backward");
     }
