@@ -347,13 +347,16 @@ rgs_status rgs_get_iterate(rgs_transport *t, int32_t b, float *out, void *stream
 rgs_status rgs_set_checkpointing(rgs_transport *t, int32_t stride);
 
 /* Device-memory budget of t: the bytes its own buffers and the pooled scratch of its calls
- * may take (0 = no budget: the device's free memory decides).  It steers the two memory
- * choices the library makes on its own: the automatic checkpoint stride (stride -1 of
- * rgs_set_checkpointing) and the number of parts rgs_adjoint splits the transposed hit
- * index into (8 bytes per hit; each part is rebuilt from the records for every transposed
- * bounce, so more parts cost time, not accuracy; in one part, 4 more bytes per hit let the
- * opacity sums be formed with the transposed bounces, else they are gathered ray by ray).  Buffers the solve needs regardless are
- * allocated even above the budget.  Host-only.  Errors: RGS_ERR_ARG. */
+ * may take (0 = no budget: the device's free memory decides).  It steers the memory choices
+ * the library makes on its own, which cost time, not accuracy: the automatic checkpoint stride
+ * (stride -1 of rgs_set_checkpointing); the number of parts rgs_adjoint splits the transposed
+ * hit index into (8 bytes per hit; each part is rebuilt from the records for every transposed
+ * bounce); its per-ray records (64 bytes a ray for 12 columns at a time where that leaves
+ * the index in one part, else 32 for 3); with the index in one part, whether the opacity sums
+ * are formed with the transposed bounces (4 more bytes per hit) or gathered ray by ray; and whether
+ * rgs_trace_pairs keeps the segments' transmittances (4 bytes per pair).
+ * Buffers the solve needs regardless are allocated even above the budget.  Host-only.
+ * Errors: RGS_ERR_ARG. */
 rgs_status rgs_set_memory_budget(rgs_transport *t, int64_t bytes);
 
 /* Which contraction the batched precision modes (RGS_BF16_FP32ACC, RGS_BF16_FP32ACC_RESCORR)

@@ -1233,16 +1233,6 @@ rgs_status rgs_adjoint_impl(rgs_transport *t, const float *g, float *dE, float *
     const int n_v = t->stride ? t->stride + 1 : nb + 1;
     if ((r = pool_alloc(&t->v, A * n_v, st)) != RGS_OK) return r;
     if ((r = pool_alloc(&t->u, A, st)) != RGS_OK) return r;
-    if (!tcp) {
-        // records of 12-column tiles (64 bytes a ray) unless they do not fit, or 3 are all there are
-        t->dy_cols = t->C > 3 ? 12 : 3;
-        r = pool_alloc(&t->dy, (size_t)n_rays * (t->dy_cols == 12 ? 16 : 8), st);
-        if (r == RGS_ERR_OOM && t->dy_cols == 12) {
-            t->dy_cols = 3;
-            r = pool_alloc(&t->dy, (size_t)n_rays * 8, st);
-        }
-        if (r != RGS_OK) return r;
-    }
     if (want_gh && (r = pool_alloc(&t->gh, (size_t)t->n_slots, st)) != RGS_OK) return r;
     // The transposed index in one part when it fits next to the segment scratch of a
     // checkpointed adjoint, else in P parts of about equal entry counts, each rebuilt from
@@ -1252,8 +1242,20 @@ rgs_status rgs_adjoint_impl(rgs_transport *t, const float *g, float *dE, float *
     const double tr_all = 8.0 * (double)t->n_hits;
     double avail = 0.92 * (double)pool_available_bytes() - seg;
     if (t->mem_budget > 0) {
-        const double scratch = 4.0 * A * (n_v + 1) + (t->dy_cols == 12 ? 64.0 : 32.0) * n_rays + (want_gh ? 4.0 * t->n_slots : 0.0);
+        const double scratch = 4.0 * A * (n_v + 1) + (want_gh ? 4.0 * t->n_slots : 0.0);
         avail = std::min(avail, (double)t->mem_budget - (double)t->device_bytes - scratch - seg);
+    }
+    if (!tcp) {
+        // records of 12-column tiles (64 bytes a ray) where 3 are not all there are and they leave
+        // the index in one part, else of 3-column tiles (32 bytes)
+        t->dy_cols = t->C > 3 && 64.0 * n_rays + tr_all <= avail ? 12 : 3;
+        r = pool_alloc(&t->dy, (size_t)n_rays * (t->dy_cols == 12 ? 16 : 8), st);
+        if (r == RGS_ERR_OOM && t->dy_cols == 12) {
+            t->dy_cols = 3;
+            r = pool_alloc(&t->dy, (size_t)n_rays * 8, st);
+        }
+        if (r != RGS_OK) return r;
+        avail -= (t->dy_cols == 12 ? 64.0 : 32.0) * n_rays;
     }
     int P = 1;
     while (!tcp && P < 64 && tr_all / P > avail) P *= 2;
