@@ -173,6 +173,8 @@ rgs_status rgs_build_scene(const rgs_surfels *surfels, const rgs_build_opts *opt
  * diagonal) of the ray origin; compositing stops once the transmittance drops below 1e-6.
  *   scene  : built scene.  lights: host struct of device pointers (copied during the call).
  *   opts   : host.  inout: as in rgs_build_scene.
+ * Pooled scratch, returned before the call ends: hit lists of 64 KB per warp in flight, at most
+ * 319 MB (fewer warps where that is not to be had or the memory budget leaves less, down to 40 MB).
  * Synchronises `stream` (the record count decides the buffer size).  Errors: RGS_ERR_ARG,
  * RGS_ERR_OOM, RGS_ERR_CUDA, RGS_ERR_CAPACITY (opts->hit_capacity too small). */
 rgs_status rgs_trace_transport(rgs_scene *scene, const rgs_lights *lights, const rgs_trace_opts *opts, void *stream,
@@ -353,8 +355,9 @@ rgs_status rgs_set_checkpointing(rgs_transport *t, int32_t stride);
  * hit index into (8 bytes per hit; each part is rebuilt from the records for every transposed
  * bounce); its per-ray records (64 bytes a ray for 12 columns at a time where that leaves
  * the index in one part, else 32 for 3); with the index in one part, whether the opacity sums
- * are formed with the transposed bounces (4 more bytes per hit) or gathered ray by ray; and whether
- * rgs_trace_pairs keeps the segments' transmittances (4 bytes per pair).
+ * are formed with the transposed bounces (4 more bytes per hit) or gathered ray by ray; how many
+ * warps trace at a time (64 KB of hit lists each, not below 40 MB); and whether rgs_trace_pairs
+ * keeps the segments' transmittances (4 bytes per pair).
  * Buffers the solve needs regardless are allocated even above the budget.  Host-only.
  * Errors: RGS_ERR_ARG. */
 rgs_status rgs_set_memory_budget(rgs_transport *t, int64_t bytes);
@@ -420,7 +423,7 @@ rgs_status rgs_set_wait_limit(rgs_transport *t, int64_t ns);
  * up = right x forward; fov is the vertical field of view in radians (0, pi); pixel (x, y),
  * y pointing down, is sampled at its centre.  B: device float [N][nc][C] in caller order (the
  * layout rgs_solve writes); img: device float [H][W][C], fully written.  Device buffers are
- * the caller's; pooled scratch (a copy of B and at most 319 MB of hit lists) is returned
+ * the caller's; pooled scratch (a copy of B and hit lists as in rgs_trace_transport) is returned
  * before the call ends.  Every pixel ray is traced, composited and shaded in one pass.
  * Synchronises `stream` once (the traversal's overflow check).  Errors: RGS_ERR_ARG (NULL
  * pointer, W or H <= 0, W*H > 2^26, fov outside (0, pi)), RGS_ERR_NONFINITE (camera),

@@ -19,7 +19,8 @@
 #define RGS_HMAX 96           // per-ray hit buffer; when full the nearest RGS_HMAX hits are kept
 #define RGS_T_EPS 1e-6f       // compositing stops once the transmittance is below this
 #define RGS_STACK 96          // BVH traversal stack depth: three waiting nodes per level of the four-wide
-                              // tree, at most (30 Morton bits + log2 N) / 2 levels
+                              // tree, at most (30 Morton bits + log2 N) / 2 levels: 93 at N = 2^31, so
+                              // that no traversal overflows it (the flag is a check of this)
 
 // Launch bounds of the gather kernels: with RGS_<KERNEL>_MINB defined, the register budget
 // is sized for that many resident blocks per SM (these latency-bound kernels gain from more
@@ -747,6 +748,10 @@ struct rgs_transport {
         return r;
     }
     size_t arr() const { return (size_t)n * C * nc; }
+    // bytes that the memory budget leaves beside the handle's own and `more` (-1: no budget)
+    long long budget_room(long long more) const {
+        return mem_budget <= 0 ? -1 : (mem_budget > device_bytes + more ? mem_budget - device_bytes - more : 0);
+    }
 };
 
 // ------------------------------------------------------------------ host helpers (rgs_api.cu)

@@ -256,7 +256,7 @@ rgs_status run_tiles(rgs_transport *t, const float *in, const float *cam, int W,
     WarpLists warps{s.st};
     const int rows = tile_rows(W, H);
     const long long tiles = (long long)((W + 7) / 8) * ((H + rows - 1) / rows);
-    if ((r = warps.get((const void *)k_render<NC, ADJ>, RN_THREADS, tiles)) != RGS_OK) return r;
+    if ((r = warps.get((const void *)k_render<NC, ADJ>, RN_THREADS, tiles, t->budget_room(4 * (long long)t->arr()))) != RGS_OK) return r;
     RGS_CUDA(cudaMemsetAsync(warps.work, 0, sizeof(unsigned), s.st));
     {
         ProfScope ps_(ADJ ? "k_render_adj" : "k_render", s.st);

@@ -256,7 +256,8 @@ rgs_status rgs_trace_impl(rgs_transport *t, const rgs_lights *L, const rgs_trace
     const int split = n_rays < 750 * 32 ? 4 : (n_rays < 1500 * 32 ? 2 : 1);
     const long long jobs = n_rays / 32 * split;
     WarpLists warps{st};
-    if ((r = warps.get((const void *)k_trace_hemi, HEMI_THREADS, jobs)) != RGS_OK) return r;
+    const long long records = 8 * std::max(want - t->cap_slots, 0ll); // still to be allocated
+    if ((r = warps.get((const void *)k_trace_hemi, HEMI_THREADS, jobs, t->budget_room(records))) != RGS_OK) return r;
     for (int attempt = 0; attempt < 2; ++attempt) {
         if (want > t->cap_slots) {
             if ((r = dev_alloc(&t->rec_ja, (size_t)want, &t->device_bytes)) != RGS_OK) return r;

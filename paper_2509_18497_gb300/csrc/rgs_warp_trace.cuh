@@ -14,6 +14,8 @@
 // 7.4 -> 3.3 ms; the pair backward of 4,000 surfels 46.4 -> 23.0 ms
 // (19.3 with the blocks of rgs_pairs.cu).
 #pragma once
+#include <algorithm>
+
 #include "rgs_internal.cuh"
 
 constexpr unsigned WT_FULL = 0xffffffffu;
@@ -484,6 +486,8 @@ static_assert(WT_SMEM_STACK * 64 >= 2 * RGS_HMAX, "the compositing borrows the s
 
 // Warps of a persistent tracing grid: their scratch lists (2 KB a ray, 319 MB for the 4,864
 // warps GB300 holds; where that is not to be had, fewer warps) and their work counter, pooled.
+// room: bytes that a memory budget leaves for the lists (negative: no budget); under a budget the grid
+// shrinks to what fits, but not below a block per SM (40 MB): fewer would idle the chip.
 struct WarpLists {
     cudaStream_t st;
     int4 *lists = nullptr;
@@ -493,17 +497,20 @@ struct WarpLists {
         pool_release(lists, st);
         pool_release(work, st);
     }
-    rgs_status get(const void *kernel, int threads, long long jobs) {
+    rgs_status get(const void *kernel, int threads, long long jobs, long long room) {
         int dev = 0, sms = 0, per_sm = 0;
         RGS_CUDA(cudaGetDevice(&dev));
         RGS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         RGS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, 0));
         const int warps = threads / 32;
-        const long long want = (jobs + warps - 1) / warps, fit = (long long)sms * (per_sm > 0 ? per_sm : 1);
+        const size_t per_block = (size_t)warps * 32 * WT_LIST;
+        const long long want = (jobs + warps - 1) / warps;
+        long long fit = (long long)sms * (per_sm > 0 ? per_sm : 1);
+        if (room >= 0) fit = std::min(fit, std::max((long long)sms, room / (long long)(per_block * sizeof(int4))));
         blocks = (int)(want < fit ? want : fit);
         if (blocks < 1) blocks = 1;
         rgs_status r;
-        while ((r = pool_alloc(&lists, (size_t)blocks * warps * 32 * WT_LIST, st)) == RGS_ERR_OOM && blocks > 1)
+        while ((r = pool_alloc(&lists, blocks * per_block, st)) == RGS_ERR_OOM && blocks > 1)
             blocks = (blocks + 1) / 2;
         if (r != RGS_OK) return r;
         return pool_alloc(&work, 1, st);
