@@ -104,13 +104,17 @@ def _tensor_peak():
         return 1700.0, "fallback (sustained)"
 
 
-def _src_sha(name):
-    with open(os.path.join(ROOT, "paper_2509_18497_gb300", "csrc", name), "rb") as f:
-        return hashlib.sha256(f.read()).hexdigest()[:16]
+def _src_sha(name, csrc=os.path.join(ROOT, "paper_2509_18497_gb300", "csrc")):
+    """Hash of a kernel's source file and of every header beside it (most of a kernel is in those)."""
+    h = hashlib.sha256()
+    for f in [name] + sorted(f for f in os.listdir(csrc) if f.endswith(".cuh")):
+        with open(os.path.join(csrc, f), "rb") as src:
+            h.update(src.read())
+    return h.hexdigest()[:16]
 
 
 # DRAM bytes per launch from one ncu capture (profiles/), keyed by kernel; valid only
-# while the kernel's source file is unchanged since the capture.
+# while the kernel's source file and the headers are unchanged since the capture.
 NCU_TRAFFIC = {
     "k_trace_hemi": {"bytes_per_launch": 0.446134e9 + 1.667045e9, "n": 10000, "src_sha": "ca603cdd76f7fe9c"},
 }
@@ -141,17 +145,18 @@ def _launch_bytes(kernel, sc):
         "k_adj_ray": (rays * (16 + 32) + tile, nb) if C <= 3 else (rays * (16 + 64) + A // T12, nb * T12),
         # records (j) + counts + offsets + directions; four iterates of v and B tiles; g per hit out
         "k_opacity_g": (H * (8 + 4) + rays * (4 + 8 + 16) + 2 * min(nb, 4) * tile, -(-nb // 4) * T3),
-        # records (j, a), g per hit, counts, offsets, directions, geometry of the hit surfels; dL/do
-        "k_opacity_rec": (H * (8 + 4) + rays * (4 + 8 + 16) + n * 64 + n * 4, 1),
+        # records (j, a), their index entries and sums, counts, offsets, directions, geometry of the hit
+        # surfels; dL/do
+        "k_opacity_rec": (H * (8 + 4 + 4) + rays * (4 + 8 + 16) + n * 64 + n * 4, 1),
         # records in, transposed entries out, counts, offsets, cursors
         "k_src_fill": (H * 20 + rays * 12 + n * 8, 1),  # (and each record's entry)
-        # center-to-center (H = pairs): the pair records written once (traversal reads are
-        # the scene and tree); the bounce reads them with the iterate rows once
-        "k_pair_fill": (n * 64 + (n - 1) * 64 + H * 8, 1),
+        # center-to-center (H = pairs): the pair records and transmittances written once (traversal
+        # reads are the scene and tree); the bounce reads the records with the iterate rows once
+        "k_pair_fill": (n * 64 + (n - 1) * 64 + H * (8 + 4), 1),
         "k_bounce_pairs": (H * 8 + 4 * A, nb),
         "k_adj_src_pairs": (H * 8 + 3 * A, nb),
         "k_pair_g": (H * (8 + 4) + 2 * nb * A, 1),
-        "k_pair_grad": (n * 64 + (n - 1) * 64 + H * 4 + n * 8, 1),
+        "k_pair_grad": (n * 64 + (n - 1) * 64 + H * (4 + 4) + n * 8, 1),
         # tensor-core contraction: per (tile, source) group one BF16 source row block (Cp x 32 B)
         # and its hit records (16 B each) into shared memory; the epilogue's arrays once
         # (bounce: S, B^(k-1) in, Q, B^(k) FP32 and two BF16 copies out; adjoint: v out, u read
