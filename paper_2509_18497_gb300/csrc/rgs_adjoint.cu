@@ -391,7 +391,8 @@ __global__ void __launch_bounds__(ADJ_THREADS, OPA ? 4 : 6) k_adj_src_tile(int C
 // term H (n_i.w) fall T moves with w (through Y(R_i w) and n_i.w), with fall = 1/r^2 and with
 // each shadow occluder's crossing point; a directional light has a fixed w and fall = 1.
 // gF (with dp): the frame gradients, through n_i (cos and R_i) and the occluders' frames.
-// A warp per 32 (surfel, light) pairs, their shadow rays traced together twice (rgs_warp_trace.cuh):
+// A warp per 32 or 16 (surfel, light) pairs (shadow_pairs), their shadow rays traced together twice
+// (rgs_warp_trace.cuh):
 // for the transmittances, then for the occluders' terms.
 struct ShadowWarp {
     WarpOcclusion w;

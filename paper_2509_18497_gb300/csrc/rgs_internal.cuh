@@ -639,7 +639,17 @@ enum { RGS_KIND_NONE = 0, RGS_KIND_HEMISPHERE = 1, RGS_KIND_PAIRS = 2 };
 struct rgs_tc_state;
 // Monte-Carlo solver state of a transport (rgs_mc.cu): the cached K-means groups
 struct rgs_mc_cache;
-// the batched modes take the tensor-core contraction from this many columns on (automatic mode)
+// The batched modes take the tensor-core contraction from this many columns on (automatic mode).
+// The line is that of row gathers half as fast as today's.  Measured with the present ones, four
+// bounces with the corrected last one, solve + adjoint in ms, row gathers against tensor cores:
+//   3,000 surfels, 128 rays:    96 columns 7.6 + 11.1 / 21.0 + 25.2, 300: 23.7 + 32.0 / 22.4 + 33.8,
+//                               1,536: 114 + 158 / 79 + 126
+//   16,000 surfels, 256 rays:   96: 79 + 87 / 209 + 180, 300: 257 + 262 / 223 + 237
+//   50,000 surfels, 256 rays:   96: 252 + 266 / 812 + 568, 300: 829 + 798 / 878 + 731
+//   200,000 surfels, 256 rays:  300: 4,029 + 3,153 / 4,632 + 3,159
+// so between 96 and some 300 columns, and on large scenes beyond, row gathers are the faster form
+// (rgs_set_tensor_cores 0).  The two round different values to 16 bits: moving the line changes
+// the results of calls between, by up to 1e-4 of the gradients.
 #define RGS_TC_MIN_COLS 96
 
 struct rgs_transport {

@@ -301,7 +301,7 @@ __global__ void k_refit(int n, const int2 *__restrict__ kids, const int *__restr
 
 // The traversal's four-wide node i from the binary node i: its grandchildren (a child that is a
 // leaf stands for itself), their boxes in 8 bits per coordinate, rounded outwards on the grid
-// of their union.  Infinite sides are cut at 1e18 (the node then covers everything).  A walk
+// of their union (quantised wide nodes: Ylitie, Karras and Laine, HPG 2017).  Infinite sides are cut at 1e18 (the node then covers everything).  A walk
 // from the root only meets nodes of even depth; the others are written all the same.
 // Each plane moves outwards by what makes slab4 conservative for rays that start in the scene
 // (|o|_1 + R <= 2 R), SLAB_ERR 2 R, and keeps at least 0.01 steps more to the stored plane for the

@@ -23,9 +23,10 @@ namespace {
 
 // A warp per patch of 32 rays of one surfel (or a part of it), patches handed out by a counter.  The lanes walk
 // the tree for their own rays and pool the surfel tests (rgs_warp_trace.cuh); accepted hits
-// go to per-ray lists in this warp's scratch (rewritten for every patch, so it stays in
-// L2), each ray's traversal ends once the hits found make the rest invisible, and the warp
-// then orders and composites one ray after the other, a lane per hit.  It allocates exactly
+// go to per-ray lists in this warp's scratch (rewritten for every patch; all warps' 319 MB are
+// more than the L2 holds, and what of them reaches DRAM is four times the records' bytes, a
+// twentieth of the time at the copy rate), each ray's traversal ends once the hits found make the
+// rest invisible, and the warp then orders and composites one ray after the other, a lane per hit.  It allocates exactly
 // its rays' kept hits with one atomic and stores every ray's records contiguously.
 __global__ void __launch_bounds__(HEMI_THREADS, RGS_TRACE_MINB) k_trace_hemi(SceneDev sc, RaysDev rays, long long jobs, int split, long long cap_slots,
                                                        unsigned long long *slot_ctr, unsigned *work, int2 *rec_ja,
