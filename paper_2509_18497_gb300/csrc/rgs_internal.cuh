@@ -77,7 +77,7 @@ enum {
 // Node of the traversal's four-wide tree, 64 bytes (two 32-byte requests): the boxes of a
 // binary LBVH node's up to four grandchildren (a child that is a leaf stands for itself) in 8
 // bits per coordinate, org + scale q rounded outwards, on the grid of their union (whose
-// widest side is 252 steps, so a box grows by about 1 % of the node).  Every plane also has
+// widest side is 253 steps, so a box grows by under 1 % of the node).  Every plane also has
 // the slack that makes slab4 conservative (k_pack).  A traversal step costs mostly what is not
 // box arithmetic (votes, queue, stack, branches); four boxes per step make half the steps of two.
 struct __align__(64) BvhNode {
@@ -530,9 +530,11 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
 // a huge finite reciprocal, so that no product below is 0 * inf.
 // Bound on the distance, in units of |o|_1 + R, between a hit as hit_rec computes it (the point
 // o + t d at its FP32 depth t) and the box planes as slab4 computes them; R: the sum over the axes
-// of the scene's largest coordinate.  hit_rec's t leaves the point off the surfel's plane by up to
-// 8 roundings (2^-24) of |p - o| and t, and places it in the plane to 3; slab4's plane of an axis
-// is off by |o| + 4 |org - o| + 2 t of them, beside C's rounding at |S|, 0.002 steps of the node.
+// of the scene's largest coordinate.  In roundings (2^-24): hit_rec's t leaves the point off the
+// surfel's plane by up to 4 |p - o| + 3 t + |h| and out of the ellipse by 1.5 |p - o|, at most
+// 9.5 (|o| + R); slab4's plane of an axis is off by |o| + 6 |org - o| of that axis.  Together they
+// stay below 16 (|o|_1 + R), and twice that costs nothing measurable (k_pack).  (C's rounding at
+// |S| is 0.002 steps of the node: k_pack too.)
 constexpr float SLAB_ERR = 1.f / (1 << 19);
 struct SlabRay {
     float3 inv, noi;
