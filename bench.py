@@ -116,7 +116,7 @@ def _src_sha(name, csrc=os.path.join(ROOT, "paper_2509_18497_gb300", "csrc")):
 # DRAM bytes per launch from one ncu capture (profiles/), keyed by kernel; valid only
 # while the kernel's source file and the headers are unchanged since the capture.
 NCU_TRAFFIC = {
-    "k_trace_hemi": {"bytes_per_launch": 0.446134e9 + 1.667045e9, "n": 10000, "src_sha": "ca603cdd76f7fe9c"},
+    "k_trace_hemi": {"bytes_per_launch": 0.448522e9 + 1.676959e9, "n": 10000, "src_sha": "35e329c147b7397b"},
 }
 
 

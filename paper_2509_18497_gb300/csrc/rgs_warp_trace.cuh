@@ -10,8 +10,8 @@
 // the same reason: a step costs votes, queue and stack beside the boxes.  These kernels are
 // bound by instruction issue (73 % of the slots used; L1 50 %, L2 20 %, DRAM 5 %).  Measured,
 // thread per ray before and warp per 32 rays now: hemisphere rays of the 50,000-surfel bowl
-// (12.8 M) 40.6 -> 24.9 ms, its shadow backward 0.85 -> 0.39 ms; a 1920 x 1080 image of it
-// 7.4 -> 3.2 ms; the pair backward of 4,000 surfels 46.4 -> 19.7 ms (with the blocks of rgs_pairs.cu).
+// (12.8 M) 40.6 -> 25.0 ms, its shadow backward 0.85 -> 0.39 ms; a 1920 x 1080 image of it
+// 7.4 -> 3.1 ms; the pair backward of 4,000 surfels 46.4 -> 19.7 ms (with the blocks of rgs_pairs.cu).
 #pragma once
 #include <algorithm>
 
