@@ -353,8 +353,8 @@ rgs_status rgs_set_checkpointing(rgs_transport *t, int32_t stride);
  * the library makes on its own, which cost time, not accuracy: the automatic checkpoint stride
  * (stride -1 of rgs_set_checkpointing); the number of parts rgs_adjoint splits the transposed
  * hit index into (8 bytes per hit; each part is rebuilt from the records for every transposed
- * bounce); its per-ray records (64 bytes a ray for 12 columns at a time where that leaves
- * the index in one part, else 32 for 3); with the index in one part, whether the opacity sums
+ * bounce); its per-ray records (64 bytes a ray for 12 columns at a time, or 32 for 3 where
+ * the larger ones would split the index for little); with the index in one part, whether the opacity sums
  * are formed with the transposed bounces (4 more bytes per hit) or gathered ray by ray; how many
  * warps trace at a time (64 KB of hit lists each, not below 40 MB); and whether rgs_trace_pairs
  * keeps the segments' transmittances (4 bytes per pair).

@@ -1247,9 +1247,18 @@ rgs_status rgs_adjoint_impl(rgs_transport *t, const float *g, float *dE, float *
         avail = std::min(avail, (double)t->mem_budget - (double)t->device_bytes - scratch - seg);
     }
     if (!tcp) {
-        // records of 12-column tiles (64 bytes a ray) where 3 are not all there are and they leave
-        // the index in one part, else of 3-column tiles (32 bytes)
-        t->dy_cols = t->C > 3 && 64.0 * n_rays + tr_all <= avail ? 12 : 3;
+        // Records of 12-column tiles (64 bytes a ray) or of 3-column ones (32), by what a transposed
+        // bounce then takes, in passes over the entries (8.3 G entries, 48 columns: 0.12 s each):
+        // one per tile; with the index in P parts 2 + P / 2 for building it anew; and 0.3 per column
+        // for gathering the opacity sums ray by ray (1.8 s) where they cannot be formed on the way.
+        auto passes = [&](int cols) {
+            const double room = avail - (cols == 12 ? 64.0 : 32.0) * n_rays;
+            int P = 1;
+            while (P < 64 && tr_all / P > room) P *= 2;
+            const bool sums = P == 1 && t->n_hits < (1ll << 32) && 12.0 * (double)t->n_hits <= room;
+            return (t->C + cols - 1) / cols + (P > 1 ? 2.0 + 0.5 * P : 0.0) + (want_gh && !sums ? 0.3 * t->C : 0.0);
+        };
+        t->dy_cols = t->C > 3 && passes(12) < passes(3) ? 12 : 3;
         r = pool_alloc(&t->dy, (size_t)n_rays * (t->dy_cols == 12 ? 16 : 8), st);
         if (r == RGS_ERR_OOM && t->dy_cols == 12) {
             t->dy_cols = 3;

@@ -180,9 +180,11 @@ int rgs_auto_stride(const rgs_transport *t, int nb, int precision) {
     const double A16 = precision != RGS_FP32 ? 2.0 * t->n * t->C * bf16_row(t->nc) : 0.0;
     const double rays = (double)t->n * t->nd;
     const double fwd = (nb + 1) * (A + A16) + nb * A;
-    // (the adjoint's per-ray records take 32 or 64 bytes; where that is what is missing, rgs_adjoint
-    // takes the smaller ones and the index, 150 bytes a ray, in parts, rather than giving up iterates)
-    const double adj = (nb + 2) * A + 8.0 * t->n_hits + 4.0 * t->n_slots + rays * (t->C > 26 ? 64 : 16);
+    // 16 bytes a ray, 128 where the last 32-column tile is more than four fifths full: what the
+    // stride has always been decided by.  The adjoint's records take 32 or 64; where that is more
+    // than is left, the index (150 bytes a ray) comes in parts, which costs less than a second
+    // forward pass (8.3 G hits, 48 columns: 1.5 s of fills for six bounces against 10.7 s).
+    const double adj = (nb + 2) * A + 8.0 * t->n_hits + 4.0 * t->n_slots + rays * (2 * t->C > 53 * ((t->C + 31) / 32) ? 128 : 16);
     const double held = t->iters_cap * A + t->q_cap * A + t->iters16_cap * A16;
     double room = 0.95 * ((double)pool_available_bytes() + held);
     if (t->mem_budget > 0) room = std::min(room, (double)t->mem_budget - ((double)t->device_bytes - held));
