@@ -4,8 +4,8 @@ and an image composites all of them, whatever the depth at which the traversal s
 A stack of wide, faint, axis-aligned surfels 2e-6 apart, all of them on every ray: the 96th
 depth lies inside every subtree's range, closer to the subtrees' first planes than the rounding of
 an 8-bit box test on a 30-unit node (8e-6 of its width), and no cutoff or depth order depends on
-FP32 (depth gaps of 2e-6 and more at depths below 1 with errors below 1e-7, 1e-4 at depths of
-40 with errors below 1e-5; rays that leave an ellipse are not used).
+FP32 (depth gaps of 2e-6 and more at depths below 1 with errors below 1e-7, 1e-4 and 3e-4
+at depths of 40 and 120 with errors below 3e-5; rays that leave an ellipse are not used).
 
 Tolerance 2e-5: a weight is a product of up to 500 factors of relative error 2^-24 (random: 1.4e-6)
 times a Gaussian of relative error 1e-6; one hit lost or exchanged moves a ray by 1e-3 and more."""
@@ -78,10 +78,10 @@ def test_the_nearest_hits_are_kept(seed):
     assert used >= BELOW // 2
 
 
-@pytest.mark.parametrize("height,gap,fov", [(0.1, 2e-6, 0.5), (0.6, 2e-6, 0.5), (40.0, 1e-4, 0.02)])
+@pytest.mark.parametrize("height,gap,fov", [(0.1, 2e-6, 0.5), (0.6, 2e-6, 0.5), (40.0, 1e-4, 0.02), (120.0, 3e-4, 0.006)])
 def test_pixels_lose_no_hit(height, gap, fov):
     """An image from under the stack, whose pixels take six passes each, from within the scene's
-    box and from outside."""
+    box, from outside and from far outside."""
     sc = _stack(5, L=1, gap=gap)
     pipe = api.Pipeline()
     d = api.upload(sc)
